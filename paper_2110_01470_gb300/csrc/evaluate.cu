@@ -5,6 +5,7 @@
 #include <string>
 #include <vector>
 
+#include "eval64.cuh"
 #include "psso.h"
 #include "sso_kernel.cuh"
 
@@ -107,7 +108,8 @@ extern "C" psso_status psso_evaluate(psso_fn fn, int64_t N, int64_t D, const dou
         if (f32 && (double)(float)o64[j] != o64[j])
             return bad(PSSO_ERR_ARG, "psso_evaluate: FP32 needs a float-exact shift");
         o32[j] = (float)o64[j];
-        w64[j] = weights ? weights[j] : 0.0;
+        // Griewank: the divisors of its cosines (eval64)
+        w64[j] = weights ? weights[j] : fn == PSSO_GRIEWANK ? std::sqrt((double)(j + 1)) : 0.0;
         w32[j] = (float)w64[j];
     }
     const size_t nM = rot ? (size_t)D * D : 0;
@@ -156,16 +158,33 @@ extern "C" psso_status psso_evaluate(psso_fn fn, int64_t N, int64_t D, const dou
         in.maxc = maxc;
         in.o64 = do64;
         in.o32 = do32;
-        in.w64 = weights ? dw64 : nullptr;
+        in.w64 = weights || fn == PSSO_GRIEWANK ? dw64 : nullptr;
         in.w32 = weights ? dw32 : nullptr;
         in.M64 = rot ? dM64 : nullptr;
         in.M32 = rot ? dM32 : nullptr;
         in.M32lo = rot ? dM32 + nM : nullptr;
         const int wpb = 8;
         const unsigned grid = (unsigned)((N + wpb - 1) / wpb);
-        if (f32) evaluate_rows<true><<<grid, 32 * wpb, 0, s>>>(in, dX, N, df, derr);
-        else evaluate_rows<false><<<grid, 32 * wpb, 0, s>>>(in, dX, N, df, derr);
-        if (cudaGetLastError() != cudaSuccess ||
+        cudaError_t le = cudaSuccess;
+        if (f32) {
+            evaluate_rows<true><<<grid, 32 * wpb, 0, s>>>(in, dX, N, df, derr);
+        } else if (ev64::covers(fn)) {
+            Hot h{};
+            h.fn = fn;
+            h.D = (int)D;
+            h.Dp = Dp;
+            h.nchunks = nchunks;
+            h.o64 = do64;
+            h.w64 = in.w64;
+            int dev_id = 0, sms = 0;
+            le = cudaGetDevice(&dev_id);
+            if (le == cudaSuccess) le = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev_id);
+            if (le == cudaSuccess)
+                le = ev64::launch(h, reinterpret_cast<const double*>(dX), Dp, N, sms, df, derr, s);
+        } else {
+            evaluate_rows<false><<<grid, 32 * wpb, 0, s>>>(in, dX, N, df, derr);
+        }
+        if (le != cudaSuccess || cudaGetLastError() != cudaSuccess ||
             cudaMemcpyAsync(f, df, N * 8, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
             (err && cudaMemcpyAsync(err, derr, N * 8, cudaMemcpyDeviceToHost, s) != cudaSuccess) ||
             cudaStreamSynchronize(s) != cudaSuccess) {

@@ -13,6 +13,7 @@
 // streams, no ordering between them) race on the array.
 #include <mutex>
 
+#include "eval64.cuh"
 #include "psso.h"
 #include "sso_kernel.cuh"
 
@@ -42,10 +43,11 @@ namespace {
 constexpr int MAX_DEVICES = 64;
 std::mutex g_setup_mutex;
 NoAllocScratch* g_scratch_addr[MAX_DEVICES] = {};
+int g_sms[MAX_DEVICES] = {};
 
 // Device address of the scratch array on the current device (set up once per
 // device, on the first call made with that device current).
-psso_status scratch_on_current_device(NoAllocScratch** out)
+psso_status scratch_on_current_device(NoAllocScratch** out, int* sms)
 {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEVICES) {
@@ -60,25 +62,50 @@ psso_status scratch_on_current_device(NoAllocScratch** out)
             set_last_error("psso_evaluate_noalloc: cudaGetSymbolAddress of the scratch array failed");
             return PSSO_ERR_CUDA;
         }
+        if (cudaDeviceGetAttribute(&g_sms[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+            set_last_error("psso_evaluate_noalloc: cannot read the number of SMs");
+            return PSSO_ERR_CUDA;
+        }
         g_scratch_addr[dev] = static_cast<NoAllocScratch*>(p);
     }
     *out = g_scratch_addr[dev];
+    *sms = g_sms[dev];
     return PSSO_OK;
 }
 
 // Fills the padded shift / weight vectors (zeros beyond D); hyper: the
-// weights of the hyper-ellipsoid, w_j = j + 1.
+// weights of the hyper-ellipsoid, w_j = j + 1; griewank: the divisors of its
+// cosines, sqrt(j + 1), once per call instead of once per row.
 __global__ void fill_scratch(NoAllocScratch* s, const double* shift, const double* weights, int D, int Dp,
-                             bool hyper)
+                             bool hyper, bool griewank)
 {
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < Dp; j += gridDim.x * blockDim.x) {
         const double o = (j < D && shift) ? shift[j] : 0.0;
-        const double w = j >= D ? 0.0 : hyper ? (double)(j + 1) : weights ? weights[j] : 0.0;
+        const double w = j >= D     ? 0.0
+                         : hyper    ? (double)(j + 1)
+                         : griewank ? __dsqrt_rn((double)(j + 1))
+                         : weights  ? weights[j]
+                                    : 0.0;
         s->o64[j] = o;
         s->o32[j] = (float)o;
         s->w64[j] = w;
         s->w32[j] = (float)w;
     }
+}
+
+// d as a float when it is exactly one: a normal float's exponent and no bits
+// below its 24, read from the bit pattern (a conversion and a compare through
+// the FP64 unit, which an SM runs at 1.66 lanes per clock, only for the rest:
+// zeros, denormals, infinities, NaN and values that are not floats).
+__device__ __forceinline__ float exact_float(double d, bool& exact)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
+    const uint32_t mag = hi & 0x7fffffffu;
+    if (mag - (897u << 20) < ((1151u - 897u) << 20) && (lo & 0x1fffffffu) == 0u)
+        return __uint_as_float((hi & 0x80000000u) | __funnelshift_l(lo, mag - (896u << 20), 3));
+    const float f = (float)d;
+    exact = exact && ((double)f == d);
+    return f;
 }
 
 // One warp per row of X (N x D doubles, unpadded): the same fitness routines
@@ -95,12 +122,10 @@ __device__ void eval_row(const Hot& in, const double* xr, double* f, double* err
 #pragma unroll
             for (int m = 0; m < 4; ++m) {
                 const int j = 4 * (lane + 32 * q) + m;
-                const double d = j < in.D ? xr[j] : 0.0;
-                x[q][m] = (float)d;
-                exact = exact && ((double)x[q][m] == d);
+                x[q][m] = j < in.D ? exact_float(xr[j], exact) : 0.f;
                 // the FP32 terms use the shift rounded to float; the bound holds for
                 // the FP64 value only when that rounding is exact
-                if (j < in.D) exact = exact && ((double)in.o32[j] == in.o64[j]);
+                if (j < in.D) (void)exact_float(in.o64[j], exact);
             }
         const Fit32 r = fit32<MAXC>(in, x, lane, 0xffffffffu, 32);
         exact = __all_sync(0xffffffffu, exact);
@@ -181,7 +206,8 @@ extern "C" psso_status psso_evaluate_noalloc(psso_fn fn, int64_t N, int64_t D, c
         return PSSO_ERR_ARG;
     }
     NoAllocScratch* s = nullptr;
-    const psso_status st = scratch_on_current_device(&s);
+    int sms = 0;
+    const psso_status st = scratch_on_current_device(&s, &sms);
     if (st != PSSO_OK) return st;
 
     const int nchunks = (int)((D + 3) / 4), Dp = 4 * nchunks;
@@ -196,17 +222,20 @@ extern "C" psso_status psso_evaluate_noalloc(psso_fn fn, int64_t N, int64_t D, c
     in.maxc = maxc;
     in.o64 = s->o64;
     in.o32 = s->o32;
-    in.w64 = (weights || hyper) ? s->w64 : nullptr;
+    const bool griewank = fn == PSSO_GRIEWANK;
+    in.w64 = (weights || hyper || griewank) ? s->w64 : nullptr;
     in.w32 = (weights || hyper) ? s->w32 : nullptr;
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     // clear an earlier, unrelated launch error so that only this call's launches are reported
     (void)cudaGetLastError();
-    fill_scratch<<<(Dp + 255) / 256, 256, 0, cs>>>(s, shift, weights, (int)D, Dp, hyper);
+    fill_scratch<<<(Dp + 255) / 256, 256, 0, cs>>>(s, shift, weights, (int)D, Dp, hyper, griewank);
     const int wpb = 8;
     const unsigned grid = (unsigned)((N + wpb - 1) / wpb);
+    cudaError_t e = cudaSuccess;
     if (precision == PSSO_PREC_F32_RECHECK) eval_noalloc<true><<<grid, 32 * wpb, 0, cs>>>(in, X, N, f, err);
+    else if (ev64::covers(fn)) e = ev64::launch(in, X, D, N, sms, f, err, cs);
     else eval_noalloc<false><<<grid, 32 * wpb, 0, cs>>>(in, X, N, f, err);
-    const cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) {
         set_last_error("psso_evaluate_noalloc: kernel launch failed");
         return PSSO_ERR_CUDA;
