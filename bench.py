@@ -294,13 +294,12 @@ def job_rate(units_per_step, steps, world, max_total_ms):
 TRAFFIC = {
     ("rot_gemm_fit", "rotated_d1000"): ("0b1474d8c773c520", 75.650048e6 + 2.041344e6),
     ("sso_generations", "rastrigin_d100"): ("c5a611e6e84c4e41", 1.407488e6 + 0.055552e6),
-    ("bat_stream", "batched_512"): ("b96e79894cdf97df", 668.860928e6 + 913.625856e6),
 }
 _COMMON = ["sso_common.cuh", "devmath.cuh", "psso_internal.h", "checked.cuh"]
 KERNEL_SOURCES = {
     "rot_gemm_fit": ["tc_gemm.cuh", "rot_pipeline.cu", "rot_pipeline.h", *_COMMON],
     "sso_generations": ["sso_kernel.cuh", "gen_variant.cu", *_COMMON],
-    "bat_stream": ["bat_stream.cuh", "sso_kernel.cuh", "gen_variant.cu", *_COMMON],
+    "bat_rows": ["bat_rows.cuh", "sso_kernel.cuh", "rows_variant.cu", *_COMMON],
 }
 
 
@@ -439,9 +438,9 @@ def batched_roofline(psso, problems, prec, t, sptr, live, workload, gens=20):
                     for p, a in zip(problems, alpha))
     return {"bound": "hbm", "achieved": b_alg[dom] / t_dom / 1e9, "peak": peaks["hbm_gbs"],
             "unit": "GB/s", "frac": b_alg[dom] / t_dom / hbm,
-            "traffic": traffic_of("bat_stream", workload) if dom == "stream" else None,
-            "kernel": "bat_stream (batched step kernel, rows over 128 variables)" if dom == "stream"
-                      else "bat_step (batched step kernel, rows up to 128 variables)",
+            "traffic": traffic_of("bat_rows", workload) if dom == "stream" else None,
+            "kernel": "bat_rows (batched row kernel, rows over 128 variables, one launch per function)"
+                      if dom == "stream" else "bat_rows (batched row kernel, rows up to 128 variables)",
             "kernel_ms_per_launch": ms[dom],
             "bytes_per_update_algorithmic": b_alg[dom] / (stream_upd if dom == "stream" else step_upd),
             "achieved_compulsory_gbs": b_cmp[dom] / t_dom / 1e9,

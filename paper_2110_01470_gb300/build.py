@@ -1,7 +1,8 @@
 """Builds ``libpsso.so`` (the CUDA library behind include/psso.h) in-tree.
 
 Every ``csrc/*.cu`` translation unit is compiled by nvcc for sm_103a in
-parallel (``gen_variant.cu`` once per kernel variant and width), then linked
+parallel (``gen_variant.cu`` once per kernel variant and width,
+``rows_variant.cu`` once per variant), then linked
 into one shared library next to this file.  Usage:
 ``python -m paper_2110_01470_gb300.build`` or ``build_library()``.
 
@@ -67,11 +68,14 @@ def build_library(force: bool = False, verbose: bool = False, trace: bool = Fals
         return lib
     os.makedirs(objdir, exist_ok=True)
     variant_src = os.path.join(CSRC, "gen_variant.cu")
+    rows_src = os.path.join(CSRC, "rows_variant.cu")
     jobs = [(src, os.path.basename(src)[:-3], [])
-            for src in sorted(glob.glob(os.path.join(CSRC, "*.cu"))) if src != variant_src]
+            for src in sorted(glob.glob(os.path.join(CSRC, "*.cu"))) if src not in (variant_src, rows_src)]
     # the persistent kernel: one object per (variant, width), compiled in parallel
     jobs += [(variant_src, f"gen_variant_{v}_{m}", [f"-DPSSO_VARIANT={v}", f"-DPSSO_MC={m}"])
              for v in range(3) for m in (1, 2, 4, 8)]
+    # the batched row kernel: one object per precision variant
+    jobs += [(rows_src, f"rows_variant_{v}", [f"-DPSSO_VARIANT={v}"]) for v in range(3)]
     # longest first
     jobs.sort(key=lambda j: (j[0] != variant_src, -int(j[1][-1]) if j[0] == variant_src else 0))
     exe = nvcc()

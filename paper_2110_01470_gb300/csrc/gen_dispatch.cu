@@ -45,6 +45,19 @@ cudaError_t bat_call(int variant, int mc_index, int op, const BatParams* p, int 
     return table[variant][mc_index](op, p, grid, block, s, out);
 }
 
+using RowsFn = cudaError_t (*)(int, bool, int, const BatRowsParams*, int, cudaStream_t, int*);
+#define PSSO_RDECL(v) cudaError_t rows_variant_##v(int, bool, int, const BatRowsParams*, int, cudaStream_t, int*);
+PSSO_RDECL(0) PSSO_RDECL(1) PSSO_RDECL(2)
+#undef PSSO_RDECL
+
+cudaError_t bat_rows_call(int variant, int fn, bool wide, int op, const BatRowsParams* p, int grid, cudaStream_t s,
+                          int* out)
+{
+    static const RowsFn table[3] = {rows_variant_0, rows_variant_1, rows_variant_2};
+    if (variant < 0 || variant > 2) return cudaErrorInvalidValue;
+    return table[variant](fn, wide, op, p, grid, s, out);
+}
+
 // gBest of one instance per block: the lowest-index arg-min of the pBests
 // (FP32 mode: certain from the bounds, else the pBests that may be the
 // minimum made exact in FP64 and the exact arg-min taken), then the record,

@@ -85,8 +85,11 @@ struct HostInst {
 struct BatHost {
     struct Class {
         int mc_index = 0, G = 32, grid = 0;
-        bool stream = false;       // wide unrotated rows: the streaming kernel
-        int32_t* ids = nullptr;
+        int fn = -1;               // a plain function: the row kernel (bat_rows.cuh); else bat_step
+        bool wide = false;         // row kernel: rows over 128 variables
+        RowTask* tasks = nullptr;  // row kernel
+        int32_t n_tasks = 0;
+        int32_t* ids = nullptr;    // bat_step
         int64_t* first = nullptr;
         int32_t n = 0;
         int64_t total = 0;
@@ -626,9 +629,12 @@ cudaError_t enqueue_bat_generation(psso_ctx* h, cudaStream_t s, cudaEvent_t* ev 
     const InstDev* inst = reinterpret_cast<const InstDev*>(h->arena + h->off_instdev);
     BatHost& B = h->bat;
     auto step = [&](const BatHost::Class& c, cudaStream_t st) {
+        if (c.fn >= 0) {
+            BatRowsParams p{inst, c.tasks, c.n_tasks, B.gen, B.cnt};
+            return bat_rows_call(h->variant, c.fn, c.wide, 0, &p, c.grid, st, nullptr);
+        }
         BatParams p{inst, c.ids, c.first, c.n, c.G, c.total, B.gen, B.cnt};
-        return c.stream ? bat_call(h->variant, 3, 2, &p, c.grid, 256, st, nullptr)
-                        : bat_call(h->variant, c.mc_index, 0, &p, c.grid, 256, st, nullptr);
+        return bat_call(h->variant, c.mc_index, 0, &p, c.grid, 256, st, nullptr);
     };
     int q = 0;
     if (ev) cudaEventRecord(ev[q++], s);
@@ -655,23 +661,35 @@ cudaError_t enqueue_bat_generation(psso_ctx* h, cudaStream_t s, cudaEvent_t* ev 
     return e;
 }
 
-// Classes of equal (lane-group width, chunks per lane), their device tables,
-// grid sizes from the occupancy of each step kernel, and the captured graphs.
+// Particles of instance I per task of the row kernel when a task covers at
+// most `slices` slices (32 chunks each): a wide row takes ceil(chunks / 32)
+// slices, a slice holds 32 / G narrow rows.
+int rows_per_task(const HostInst& I, int slices)
+{
+    const int nq = (I.nchunks + 31) / 32;
+    return nq > 1 ? std::max(1, slices / nq) : slices * (32 / I.G);
+}
+
+// The step-kernel classes, their device tables, grid sizes from the occupancy
+// of each step kernel, and the captured graphs.  The plain functions' swarms
+// form one class per function and row width (up to / over 128 variables) on
+// the row kernel; the others (rotated, FP64-only functions) one per lane-group
+// width and chunks per lane on bat_step.
 psso_status setup_bat(psso_ctx* h)
 {
     BatHost& B = h->bat;
     std::vector<std::vector<int32_t>> members;
-    std::vector<std::pair<int, int>> keys;   // (mc_index, G); mc_index 4 = streaming kernel
+    std::vector<std::pair<int, int>> keys;   // (fn, wide) or (16 + mc_index, G)
     std::vector<int32_t> all;
+    int64_t slices = 0;                      // of the row kernel's classes
     for (size_t k = 0; k < h->inst.size(); ++k) {
         const HostInst& I = h->inst[k];
         if (!I.bp) continue;
-        int mci = I.maxc >= 8 ? 3 : I.maxc >= 4 ? 2 : I.maxc >= 2 ? 1 : 0;
-        // Unrotated rows over 128 variables (one particle per warp) run on the
-        // streaming kernel: it holds one 32-chunk slice in registers instead
-        // of the whole row, so more warps fit on an SM.
-        if (mci >= 1 && I.pr.fn < PSSO_ROT_ELLIPSOID) mci = 4;
-        const std::pair<int, int> key(mci, I.G);
+        const bool rows = I.pr.fn <= PSSO_ACKLEY;
+        const std::pair<int, int> key =
+            rows ? std::pair<int, int>(I.pr.fn, I.maxc > 1)
+                 : std::pair<int, int>(16 + (I.maxc >= 8 ? 3 : I.maxc >= 4 ? 2 : I.maxc >= 2 ? 1 : 0), I.G);
+        if (rows) slices += I.pr.N * ((I.nchunks + 31) / 32) / (32 / I.G) + 1;
         size_t c = 0;
         while (c < keys.size() && keys[c] != key) ++c;
         if (c == keys.size()) {
@@ -683,6 +701,12 @@ psso_status setup_bat(psso_ctx* h)
     }
     B.n_all = (int32_t)all.size();
     if (B.n_all == 0) return PSSO_OK;
+    cudaDeviceProp prop;
+    CUDA_TRY(cudaGetDeviceProperties(&prop, h->device));
+    // Slices per task: as many as leave every one of the 32 warps an SM holds
+    // a task (more slices fill the rounds of fresh-value blocks better).
+    int per_task = 1;
+    while (per_task < 8 && slices / (2 * per_task) >= (int64_t)prop.multiProcessorCount * 32) per_task *= 2;
     size_t bytes = 0;
     auto take = [&](size_t n) {
         bytes = align_up(bytes, 256);
@@ -691,35 +715,58 @@ psso_status setup_bat(psso_ctx* h)
         return at;
     };
     std::vector<size_t> oid(keys.size()), ofirst(keys.size());
+    std::vector<std::vector<RowTask>> tasks(keys.size());
     for (size_t c = 0; c < keys.size(); ++c) {
-        oid[c] = take(members[c].size() * 4);
-        ofirst[c] = take((members[c].size() + 1) * 8);
+        if (keys[c].first < 16) {
+            // longest tasks first, so that the grid's last tasks are short
+            std::stable_sort(members[c].begin(), members[c].end(), [&](int32_t a, int32_t b) {
+                return h->inst[a].nchunks > h->inst[b].nchunks;
+            });
+            for (int32_t k : members[c]) {
+                const int64_t n = rows_per_task(h->inst[k], per_task), N = h->inst[k].pr.N;
+                for (int64_t i = 0; i < N; i += n)
+                    tasks[c].push_back(RowTask{k, (int32_t)i, (int32_t)std::min(n, N - i)});
+            }
+            if (tasks[c].size() > 0x7fffffffu) return fail(PSSO_ERR_UNSUPPORTED, "too many particles for one batch");
+            oid[c] = take(tasks[c].size() * sizeof(RowTask));
+        } else {
+            oid[c] = take(members[c].size() * 4);
+            ofirst[c] = take((members[c].size() + 1) * 8);
+        }
     }
     const size_t oall = take(all.size() * 4), ocnt = take(h->inst.size() * sizeof(BatCounters)),
                  ogen = take(sizeof(long long));
     CUDA_TRY(cudaMalloc(&B.mem, bytes));
     std::vector<char> host(bytes, 0);
     char* base = static_cast<char*>(B.mem);
-    cudaDeviceProp prop;
-    CUDA_TRY(cudaGetDeviceProperties(&prop, h->device));
     for (size_t c = 0; c < keys.size(); ++c) {
         BatHost::Class cl;
-        cl.stream = keys[c].first == 4;
-        cl.mc_index = cl.stream ? 3 : keys[c].first;
-        cl.G = keys[c].second;
-        cl.n = (int32_t)members[c].size();
-        std::vector<int64_t> first(members[c].size() + 1, 0);
-        for (size_t q = 0; q < members[c].size(); ++q) first[q + 1] = first[q] + h->inst[members[c][q]].pr.N;
-        cl.total = first.back();
-        std::memcpy(host.data() + oid[c], members[c].data(), members[c].size() * 4);
-        std::memcpy(host.data() + ofirst[c], first.data(), first.size() * 8);
-        cl.ids = reinterpret_cast<int32_t*>(base + oid[c]);
-        cl.first = reinterpret_cast<int64_t*>(base + ofirst[c]);
         int bps = 0;
-        CUDA_TRY(bat_call(h->variant, cl.mc_index, cl.stream ? 3 : 1, nullptr, 0, 256, nullptr, &bps));
+        int64_t need;
+        if (keys[c].first < 16) {
+            cl.fn = keys[c].first;
+            cl.wide = keys[c].second != 0;
+            std::memcpy(host.data() + oid[c], tasks[c].data(), tasks[c].size() * sizeof(RowTask));
+            cl.tasks = reinterpret_cast<RowTask*>(base + oid[c]);
+            cl.n_tasks = (int32_t)tasks[c].size();
+            CUDA_TRY(bat_rows_call(h->variant, cl.fn, cl.wide, 1, nullptr, 0, nullptr, &bps));
+            need = ((int64_t)cl.n_tasks + 7) / 8;
+        } else {
+            cl.mc_index = keys[c].first - 16;
+            cl.G = keys[c].second;
+            cl.n = (int32_t)members[c].size();
+            std::vector<int64_t> first(members[c].size() + 1, 0);
+            for (size_t q = 0; q < members[c].size(); ++q) first[q + 1] = first[q] + h->inst[members[c][q]].pr.N;
+            cl.total = first.back();
+            std::memcpy(host.data() + oid[c], members[c].data(), members[c].size() * 4);
+            std::memcpy(host.data() + ofirst[c], first.data(), first.size() * 8);
+            cl.ids = reinterpret_cast<int32_t*>(base + oid[c]);
+            cl.first = reinterpret_cast<int64_t*>(base + ofirst[c]);
+            CUDA_TRY(bat_call(h->variant, cl.mc_index, 1, nullptr, 0, 256, nullptr, &bps));
+            const int64_t groups_per_block = 256 / cl.G;
+            need = (cl.total + groups_per_block - 1) / groups_per_block;
+        }
         if (h->cfg.batch_blocks_per_sm > 0) bps = std::min(bps, (int)h->cfg.batch_blocks_per_sm);
-        const int64_t groups_per_block = cl.stream ? 8 : 256 / cl.G;
-        const int64_t need = (cl.total + groups_per_block - 1) / groups_per_block;
         cl.grid = (int)std::max<int64_t>(1, std::min<int64_t>(need, (int64_t)std::max(1, bps) * prop.multiProcessorCount));
         B.classes.push_back(cl);
     }
@@ -1364,7 +1411,7 @@ static psso_status time_bat_kernels(psso_ctx* h, int32_t generations, float* ms,
         for (int q = 0; q < K && e == cudaSuccess; ++q) {
             float t = 0.f;
             e = cudaEventElapsedTime(&t, ev[q], ev[q + 1]);
-            const int slot = q + 1 == K ? 2 : (h->bat.classes[q].stream ? 0 : 1);
+            const int slot = q + 1 == K ? 2 : (h->bat.classes[q].wide ? 0 : 1);
             acc[slot] += t;
         }
     }

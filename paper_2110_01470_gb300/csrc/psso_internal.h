@@ -178,10 +178,25 @@ struct BatParams {
     BatCounters* cnt;              // [instances]
 };
 // op 0: launch bat_step over p (grid x block); op 1: occupancy (blocks per SM
-// into *out) for `block` threads; ops 2 / 3: the same for the streaming kernel
-// of wide unrotated rows (one warp per particle; mc_index 3 only).
+// into *out) for `block` threads.
 cudaError_t bat_call(int variant, int mc_index, int op, const BatParams* p, int grid, int block, cudaStream_t s,
                      int* out);
+// The plain functions' row kernel (bat_rows.cuh): n consecutive particles of
+// one instance per task, a task per warp.
+struct RowTask {
+    int32_t inst, i0, n;
+};
+struct BatRowsParams {
+    const InstDev* inst;
+    const RowTask* tasks;
+    int32_t n_tasks;
+    const long long* gen;          // generation being run (device)
+    BatCounters* cnt;              // [instances]
+};
+// op 0: launch (grid blocks of 256 threads), op 1: occupancy (blocks per SM
+// into *out); wide: rows of more than 128 variables.
+cudaError_t bat_rows_call(int variant, int fn, bool wide, int op, const BatRowsParams* p, int grid, cudaStream_t s,
+                          int* out);
 // One block per listed instance: gBest arg-min (exact lowest index), record,
 // log, gBest row; then the generation counter + 1 (last kernel of a generation).
 cudaError_t launch_bat_argmin(int variant, const InstDev* inst, const int32_t* ids, int n_ids, long long* gen,
