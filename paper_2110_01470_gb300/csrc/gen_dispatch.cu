@@ -1,5 +1,7 @@
 // gen_dispatch.cu -- variant dispatch for occupancy / shared-memory queries and
 // the on-demand FP64 evaluation of gBest rows.
+#include <climits>
+
 #include "sso_kernel.cuh"
 
 namespace psso {
@@ -61,93 +63,175 @@ cudaError_t bat_rows_call(int variant, int fn, bool wide, int op, const BatRowsP
 // gBest of one instance per block: the lowest-index arg-min of the pBests
 // (FP32 mode: certain from the bounds, else the pBests that may be the
 // minimum made exact in FP64 and the exact arg-min taken), then the record,
-// log and gBest row.
-template <class Pos, bool F32R>
-__global__ void __launch_bounds__(256) bat_argmin(const InstDev* inst, const int32_t* ids, const long long* gen,
-                                                  BatCounters* cnt)
+// log and gBest row; the last block advances the generation.
+//
+// Bound: latency (a few loads and block reductions per swarm).  Only the keys
+// are read and reduced -- FP32: the smallest and second-smallest lower bound,
+// the first's index, the smallest upper bound; FP64: the value as an integer
+// key and the index -- and the winner's other fields afterwards.  The
+// candidates of the exact pass are first collected by a scan over all
+// threads: one warp walking the particles one load at a time cost a load
+// latency per particle and warp.  40 swarms, FP64: 17 -> 10 us per launch.
+constexpr int ARGMIN_LIST = 2048;
+
+struct BatKey {
+    long long v;      // FP64: order_key of the value
+    float l1, l2, mh; // FP32
+    int i;
+};
+template <bool F32R>
+__device__ __forceinline__ BatKey key_merge(const BatKey& a, const BatKey& b)
 {
-    __shared__ Cand sh[32];
+    BatKey r;
+    if constexpr (F32R) {
+        const bool bf = b.l1 < a.l1 || (b.l1 == a.l1 && b.i < a.i);
+        r.v = 0;
+        r.l1 = bf ? b.l1 : a.l1;
+        r.i = bf ? b.i : a.i;
+        r.l2 = fminf(fminf(a.l2, b.l2), bf ? a.l1 : b.l1);
+        r.mh = fminf(a.mh, b.mh);
+    } else {
+        const bool bf = b.v < a.v || (b.v == a.v && b.i < a.i);
+        r.v = bf ? b.v : a.v;
+        r.i = bf ? b.i : a.i;
+        r.l1 = r.l2 = r.mh = 0.f;
+    }
+    return r;
+}
+template <bool F32R>
+__device__ __forceinline__ BatKey key_warp(BatKey k)
+{
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        BatKey o;
+        o.i = __shfl_xor_sync(0xffffffffu, k.i, off);
+        o.v = F32R ? 0 : __shfl_xor_sync(0xffffffffu, k.v, off);
+        o.l1 = F32R ? __shfl_xor_sync(0xffffffffu, k.l1, off) : 0.f;
+        o.l2 = F32R ? __shfl_xor_sync(0xffffffffu, k.l2, off) : 0.f;
+        o.mh = F32R ? __shfl_xor_sync(0xffffffffu, k.mh, off) : 0.f;
+        k = key_merge<F32R>(k, o);
+    }
+    return k;
+}
+// Every thread gets the block's result (256 threads).
+template <bool F32R>
+__device__ __forceinline__ BatKey key_block(BatKey k, BatKey* sh)
+{
+    k = key_warp<F32R>(k);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = k;
+    __syncthreads();
+    k = sh[0];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) k = key_merge<F32R>(k, sh[w]);
+    return k;
+}
+
+template <class Pos, bool F32R>
+__global__ void __launch_bounds__(256) bat_argmin(const InstDev* inst, const int32_t* ids, long long* gen,
+                                                  unsigned* ticket, BatCounters* cnt)
+{
+    __shared__ BatKey sh[8];
+    __shared__ int list[F32R ? ARGMIN_LIST : 1];
+    __shared__ int n_list;
     __shared__ unsigned long long extra;
     const int k = ids[blockIdx.x];
     const InstDev& d = inst[k];
-    const int64_t g = *gen;
-    const int64_t N = d.N;
+    const long long g = *gen;
+    const int N = (int)d.N;
     if (threadIdx.x == 0) extra = 0;
-    Cand c = cand_none();
-    for (int64_t i = threadIdx.x; i < N; i += blockDim.x)
-        c = cand_merge<F32R>(c, cand_of<F32R>((long long)i, d.pf64[i], F32R ? d.plo[i] : 0.f,
-                                              F32R ? d.phi[i] : 0.f, F32R ? (int)(d.pflag[i] & 1u) : 1,
-                                              d.pver[i]));
-    Cand b = block_reduce_cand<F32R>(c, sh);
-    if (F32R && b.l2 <= b.mh) {
-        const Hot hin = hot_of(d);
-        const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-        for (int64_t i = threadIdx.x >> 5; i < N; i += nw) {
-            if (!(d.plo[i] <= b.mh && !(d.pflag[i] & 1u))) continue;   // uniform over the warp
-            const double f = fit64_row<Pos>(hin, static_cast<const Pos*>(d.P) + i * d.Dp, false);
-            if (lane == 0) {
-                d.pf64[i] = f;
-                d.pflag[i] = 1u;
-                d.plo[i] = f64_to_f32_rd(f);
-                d.phi[i] = f64_to_f32_ru(f);
-                atomicAdd(&extra, 1ull);
-            }
+    const BatKey none = {LLONG_MAX, FLT_MAX, FLT_MAX, FLT_MAX, INT_MAX};
+    BatKey c = none;
+    for (int i = threadIdx.x; i < N; i += 256) {
+        BatKey q = none;
+        q.i = i;
+        if constexpr (F32R) {
+            q.l1 = d.plo[i];
+            q.mh = d.phi[i];
+        } else {
+            q.v = order_key(d.pf64[i]);
         }
-        __syncthreads();
-        // every pBest that can be the minimum has its FP64 value now
-        Cand e = cand_none();
-        for (int64_t i = threadIdx.x; i < N; i += blockDim.x)
-            if (d.pflag[i] & 1u) {
-                Cand q = cand_none();
-                q.v = d.pf64[i];
-                q.i = (long long)i;
-                q.ver = d.pver[i];
-                e = cand_merge<false>(e, q);
-            }
-        b = block_reduce_cand<false>(e, sh);
-        b.has1 = 1;
-        b.l1 = f64_to_f32_rd(b.v);
-        b.h1 = f64_to_f32_ru(b.v);
+        c = key_merge<F32R>(c, q);
     }
-    const Pos* src = static_cast<const Pos*>(d.P) + b.i * d.Dp;
+    BatKey b = key_block<F32R>(c, sh);
+    bool exact = !F32R;
+    if constexpr (F32R) {
+        if (b.l2 <= b.mh) {
+            // every pBest that can be the minimum gets its FP64 value, a list of
+            // candidates at a time, a warp per candidate
+            const Hot hin = hot_of(d);
+            const int lane = threadIdx.x & 31;
+            const float m = b.mh;
+            for (int base = 0; base < N; base += ARGMIN_LIST) {
+                __syncthreads();
+                if (threadIdx.x == 0) n_list = 0;
+                __syncthreads();
+                const int top = min(N, base + ARGMIN_LIST);
+                for (int i = base + threadIdx.x; i < top; i += 256)
+                    if (d.plo[i] <= m && !(d.pflag[i] & 1u)) list[atomicAdd(&n_list, 1)] = i;
+                __syncthreads();
+                for (int e = threadIdx.x >> 5; e < n_list; e += 8) {
+                    const int i = list[e];
+                    const double f = fit64_row<Pos>(hin, static_cast<const Pos*>(d.P) + (int64_t)i * d.Dp, false);
+                    if (lane == 0) {
+                        d.pf64[i] = f;
+                        d.pflag[i] = 1u;
+                        d.plo[i] = f64_to_f32_rd(f);
+                        d.phi[i] = f64_to_f32_ru(f);
+                        atomicAdd(&extra, 1ull);
+                    }
+                }
+            }
+            __syncthreads();
+            BatKey e = none;
+            for (int i = threadIdx.x; i < N; i += 256)
+                if (d.pflag[i] & 1u) {
+                    BatKey q = none;
+                    q.i = i;
+                    q.v = order_key(d.pf64[i]);
+                    e = key_merge<false>(e, q);
+                }
+            b = key_block<false>(e, sh);
+            exact = true;
+        }
+    }
+    const int wi = b.i < N ? b.i : 0;        // no finite value at all: the first particle
+    const Pos* src = static_cast<const Pos*>(d.P) + (int64_t)wi * d.Dp;
     Pos* dst = static_cast<Pos*>(d.gbrow);
-    for (int j = threadIdx.x; j < d.Dp; j += blockDim.x) dst[j] = src[j];
-    __syncthreads();
+    for (int q = threadIdx.x; q < d.nchunks; q += 256) {
+        Pos v[4];
+        ld4(src + 4 * q, v);
+        st4(dst + 4 * q, v);
+    }
     if (threadIdx.x == 0) {
         Winner w;
-        w.idx = b.i;
-        w.ver = b.ver;
+        w.idx = wi;
+        w.ver = d.pver[wi];
         w.acc = cnt[k].acc;
         w.rck = cnt[k].rck + extra;
-        if (!F32R) {
-            w.has64 = 1;
-            w.f64 = b.v;
-            w.lo = f64_to_f32_rd(b.v);
-            w.hi = f64_to_f32_ru(b.v);
-        } else {
-            w.has64 = b.has1;
-            w.f64 = b.has1 ? b.v : 0.0;
-            w.lo = b.l1;
-            w.hi = b.h1;
-        }
+        const bool has = exact || (F32R && (d.pflag[wi] & 1u));
+        w.has64 = has ? 1 : 0;
+        w.f64 = has ? d.pf64[wi] : 0.0;
+        w.lo = exact ? f64_to_f32_rd(w.f64) : d.plo[wi];
+        w.hi = exact ? f64_to_f32_ru(w.f64) : d.phi[wi];
         write_gbest(d, w, g);
         cnt[k].acc = 0;
         cnt[k].rck = 0;
+        // every block has read the generation before it takes a ticket
+        __threadfence();
+        if (atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1) *gen = g + 1;
     }
 }
 
-__global__ void bat_next(long long* gen) { *gen += 1; }
 __global__ void bat_set(long long* gen, long long g) { *gen = g; }
 
 cudaError_t launch_bat_argmin(int variant, const InstDev* inst, const int32_t* ids, int n_ids, long long* gen,
                               BatCounters* cnt, cudaStream_t s)
 {
-    if (variant == 0) bat_argmin<double, false><<<n_ids, 256, 0, s>>>(inst, ids, gen, cnt);
-    else if (variant == 1) bat_argmin<float, false><<<n_ids, 256, 0, s>>>(inst, ids, gen, cnt);
-    else bat_argmin<float, true><<<n_ids, 256, 0, s>>>(inst, ids, gen, cnt);
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    bat_next<<<1, 1, 0, s>>>(gen);
+    unsigned* ticket = reinterpret_cast<unsigned*>(gen + 1);
+    if (variant == 0) bat_argmin<double, false><<<n_ids, 256, 0, s>>>(inst, ids, gen, ticket, cnt);
+    else if (variant == 1) bat_argmin<float, false><<<n_ids, 256, 0, s>>>(inst, ids, gen, ticket, cnt);
+    else bat_argmin<float, true><<<n_ids, 256, 0, s>>>(inst, ids, gen, ticket, cnt);
     return cudaGetLastError();
 }
 

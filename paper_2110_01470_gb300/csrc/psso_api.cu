@@ -98,7 +98,7 @@ struct BatHost {
     int32_t* all_ids = nullptr;   // every batched instance (arg-min blocks)
     int32_t n_all = 0;
     BatCounters* cnt = nullptr;
-    long long* gen = nullptr;
+    long long* gen = nullptr;     // generation, then the arg-min's ticket word
     void* mem = nullptr;
     cudaGraphExec_t graph1 = nullptr, graphG = nullptr;
     static constexpr int GRAPH_GENS = 16;
@@ -506,7 +506,7 @@ psso_status launch(psso_ctx* h, int64_t g_begin, int64_t g_end)
         for (; count >= BatHost::GRAPH_GENS; count -= BatHost::GRAPH_GENS)
             CUDA_TRY(cudaGraphLaunch(h->bat.graphG, h->stream));
         for (; count > 0; --count) CUDA_TRY(cudaGraphLaunch(h->bat.graph1, h->stream));
-        h->launches += 1 + (int64_t)(h->bat.classes.size() + 2) * (g_end - g_begin + 1);
+        h->launches += 1 + (int64_t)(h->bat.classes.size() + 1) * (g_end - g_begin + 1);
     }
     // tensor-pipeline swarms: forked after everything above in stream order,
     // one side stream each (the handle's stream when there is no side stream)
@@ -735,7 +735,7 @@ psso_status setup_bat(psso_ctx* h)
         }
     }
     const size_t oall = take(all.size() * 4), ocnt = take(h->inst.size() * sizeof(BatCounters)),
-                 ogen = take(sizeof(long long));
+                 ogen = take(2 * sizeof(long long));
     CUDA_TRY(cudaMalloc(&B.mem, bytes));
     std::vector<char> host(bytes, 0);
     char* base = static_cast<char*>(B.mem);

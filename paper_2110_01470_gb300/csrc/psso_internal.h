@@ -198,7 +198,8 @@ struct BatRowsParams {
 cudaError_t bat_rows_call(int variant, int fn, bool wide, int op, const BatRowsParams* p, int grid, cudaStream_t s,
                           int* out);
 // One block per listed instance: gBest arg-min (exact lowest index), record,
-// log, gBest row; then the generation counter + 1 (last kernel of a generation).
+// log, gBest row; the last block adds 1 to the generation counter (last kernel
+// of a generation).  gen: the counter, followed by a ticket word (zero).
 cudaError_t launch_bat_argmin(int variant, const InstDev* inst, const int32_t* ids, int n_ids, long long* gen,
                               BatCounters* cnt, cudaStream_t s);
 cudaError_t launch_bat_set_gen(long long* gen, long long g, cudaStream_t s);

@@ -89,6 +89,16 @@ __device__ __forceinline__ bool same_bits(double a, double b)
     return __double_as_longlong(a) == __double_as_longlong(b);
 }
 
+// Order-preserving integer key of a double (sign-magnitude to two's complement,
+// so -0 and +0 are equal; a positive NaN is above everything).  Comparing two
+// keys is integer work, where comparing two doubles takes the FP64 unit: 64
+// clocks each, 19 clocks of the whole SM's unit.
+__device__ __forceinline__ long long order_key(double v)
+{
+    const long long b = __double_as_longlong(v);
+    return b < 0 ? -(b & 0x7fffffffffffffffLL) : b;
+}
+
 // The per-particle fields of an instance descriptor, as a small value type
 // that the inlined hot path keeps in registers.
 struct Hot {
