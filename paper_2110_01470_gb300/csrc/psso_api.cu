@@ -574,7 +574,8 @@ psso_status setup_tc(psso_ctx* h, size_t k)
                  oms = take((size_t)r.Jp * 4), oml1 = take((size_t)r.Jp * 4), ods = take((size_t)r.Np * 4),
                  odl1 = take((size_t)r.Np * 4), osame = take((size_t)N * 4),
                  opart = take((size_t)N * r.nJt * 16), ol1 = take((size_t)N * 4), ol2 = take((size_t)N * 4),
-                 oz = take((size_t)2 * N * I.Dp * 8), oz0 = take((size_t)I.Dp * 8),
+                 oz = take((size_t)2 * N * I.Dp * 8),
+                 osn = take(I.pr.fn == PSSO_ROT_ACKLEY ? (size_t)2 * N * I.Dp * 8 : 0), omt = take((size_t)D * D * 8),
                  octl = take(sizeof(rot::RotCtl)), ol3 = take((size_t)N * 4),
                  omh = take((size_t)D * D * 4), oml = take((size_t)D * D * 4),
                  oz32 = take((size_t)2 * N * I.Dp * 4), oez = take((size_t)2 * N * I.Dp * 4);
@@ -593,7 +594,9 @@ psso_status setup_tc(psso_ctx* h, size_t k)
     r.list1 = reinterpret_cast<int32_t*>(b + ol1);
     r.list2 = reinterpret_cast<int32_t*>(b + ol2);
     r.zbuf = reinterpret_cast<double*>(b + oz);
-    r.zero64 = reinterpret_cast<const double*>(b + oz0);
+    r.sbuf = I.pr.fn == PSSO_ROT_ACKLEY ? reinterpret_cast<double*>(b + osn) : nullptr;
+    R.Mt = reinterpret_cast<double*>(b + omt);
+    r.Mt = R.Mt;
     r.ctl = reinterpret_cast<rot::RotCtl*>(b + octl);
     r.list3 = reinterpret_cast<int32_t*>(b + ol3);
     R.Mh = reinterpret_cast<float*>(b + omh);

@@ -24,8 +24,9 @@
 //   5. rot_fix32     fitness intervals from the refined z; decides the pBest
 //                    update, or the particle goes on list 3.
 //   6. rot_z64       FP64 z = M (x - o) of list-3 rows in the oracle's order
-//                    (k ascending, fma from +0), one thread per output.
-//   7. rot_fix       FP64 fitness of those rows (the oracle's summation) and
+//                    (k ascending, fma from +0) and their fitness terms, one
+//                    thread per output.
+//   7. rot_fix       the FP64 sums of those rows (the oracle's summation) and
 //                    the exact pBest decision.
 //   8. rot_argmin(0) gBest candidates (Alg. 4, lowest index): unique from the
 //                    intervals, or the pBests that can still be the minimum
@@ -199,14 +200,14 @@ __device__ __forceinline__ void term32(int fn, float zt, float ez, const float* 
         s = __fadd_rn(s, tv);
         e = __fadd_rn(e, 4.2f * 0x1p-24f * tv + 1.01f * w * (2.f * az + ez) * ez);
     } else if (fn == FN_RASTRIGIN) {
-        const float sn = sinpi_reduced_f32(__fsub_rn(zt, rintf(zt)));
+        const float sn = sinpi_reduced_f32(__fsub_rn(zt, rint_f32(zt)));
         const float tv = __fmaf_rn(zt, zt, __fmul_rn(20.f, __fmul_rn(sn, sn)));
         s = __fadd_rn(s, tv);
         e = __fadd_rn(e, (2.f * SINPI32_ERR_U + 4.f) * 0x1p-24f * tv +
                              1.01f * (2.f * xi + 62.8318558f * fminf(1.f, 6.28318548f * xi)) * ez);
     } else {   // Ackley
         s = __fadd_rn(s, __fmul_rn(zt, zt));
-        const float sn = sinpi_reduced_f32(__fsub_rn(zt, rintf(zt)));
+        const float sn = sinpi_reduced_f32(__fsub_rn(zt, rint_f32(zt)));
         s2 = __fadd_rn(s2, __fmul_rn(sn, sn));
         e = __fadd_rn(e, 1.01f * (2.f * az + ez) * ez);
         eq = __fadd_rn(eq, 1.01f * 3.14159275f * fminf(1.f, 6.28318548f * xi) * ez);
@@ -464,89 +465,92 @@ __global__ void __launch_bounds__(128) rot_z32(const RotDev r)
 }
 
 // ---- 5. decisions from the refined intervals ---------------------------------------------
-template <int MAXC>
+// One warp per refined row, two per list entry.  The kernel runs once over a
+// handful of entries, so its time is instruction fetch and the chains of one
+// warp: the loops stay rolled (unrolled over the widest row, the straight-line
+// code took longer to fetch than to run) and the entry's two rows run side by
+// side (33 -> 8 us per launch at D = 1000).
 __device__ Fit32 fit_refined(const RotDev& r, const InstDev& d, const float* z, const float* ez, int lane)
 {
     const int fn = base_fn(r.fn);
     float s = 0.f, s2 = 0.f, e = 0.f, eq = 0.f;
-#pragma unroll
-    for (int q = 0; q < MAXC; ++q) {
-        const int c = lane + 32 * q;
-        if (c >= d.nchunks) continue;
+#pragma unroll 1
+    for (int c = lane; c < d.nchunks; c += 32) {
         float zv[4], ev[4];
         ld4(z + 4 * c, zv);
         ld4(ez + 4 * c, ev);
-#pragma unroll
+#pragma unroll 1
         for (int m = 0; m < 4; ++m)
-            if (4 * c + m < d.D) term32(fn, zv[m], ev[m], r.inst_w32, 4 * c + m, s, s2, e, eq);
+            if (4 * c + m < d.D)
+                term32(fn, m == 0 ? zv[0] : m == 1 ? zv[1] : m == 2 ? zv[2] : zv[3],
+                       m == 0 ? ev[0] : m == 1 ? ev[1] : m == 2 ? ev[2] : ev[3], r.inst_w32, 4 * c + m, s, s2, e, eq);
     }
+#pragma unroll 1
     for (int off = 16; off > 0; off >>= 1) {
         s = __fadd_rn(s, __shfl_xor_sync(0xffffffffu, s, off));
         s2 = __fadd_rn(s2, __shfl_xor_sync(0xffffffffu, s2, off));
         e = __fadd_rn(e, __shfl_xor_sync(0xffffffffu, e, off));
         eq = __fadd_rn(eq, __shfl_xor_sync(0xffffffffu, eq, off));
     }
-    return rot_final(fn, d.D, s, s2, e, eq, (float)(4 * MAXC + 5 + 2));
+    return rot_final(fn, d.D, s, s2, e, eq, (float)(4 * d.maxc + 5 + 2));
 }
 
-template <int MAXC>
-__device__ void fix32_one(const RotDev& r, const InstDev& d, long long e, int lane)
+// Copies particle i's position to its pBest row (n threads, this one t).
+__device__ __forceinline__ void accept_row(const InstDev& d, int64_t i, int t, int n)
 {
-    const int32_t i = r.list1[e];
-    if (!PSSO_CHK(i >= 0 && i < r.N, CHK_ROT_ROW, i)) return;
-    const int64_t g = r.ctl->gen;
-    const size_t ox = (size_t)(2 * e) * d.Dp, op = ox + d.Dp;
-    float plo = d.plo[i], phi = d.phi[i];
-    const Fit32 fx = fit_refined<MAXC>(r, d, r.z32 + ox, r.ez32 + ox, lane);
-    const float lox = __fsub_rd(fx.f, fx.E), hix = __fadd_ru(fx.f, fx.E);
-    const bool have_p = (d.pflag[i] & 1u) != 0;
-    if (!have_p) {       // the pBest's interval, tightened the same way (intersection of two bounds)
-        const Fit32 fp = fit_refined<MAXC>(r, d, r.z32 + op, r.ez32 + op, lane);
-        plo = fmaxf(plo, __fsub_rd(fp.f, fp.E));
-        phi = fminf(phi, __fadd_ru(fp.f, fp.E));
-    }
-    const int accept = hix < plo;
-    const int reject = lox > phi;
-    if (accept) {
-        const float* xr = static_cast<const float*>(d.X) + (int64_t)i * d.Dp;
-        float* prow = static_cast<float*>(d.P) + (int64_t)i * d.Dp;
-        for (int c = lane; c < d.nchunks; c += 32) {
-            float v[4];
-            ld4(xr + 4 * c, v);
-            st4(prow + 4 * c, v);
-        }
-    }
-    if (lane == 0) {
-        if (accept) {
-            d.plo[i] = lox;
-            d.phi[i] = hix;
-            d.pflag[i] = 0u;
-            d.pf64[i] = 0.0;
-            d.pver[i] = (uint32_t)g;
-            atomicAdd(&r.ctl->acc, 1ull);
-        } else {
-            d.plo[i] = plo;
-            d.phi[i] = phi;
-            if (!reject) list_push(r.list3, &r.ctl->n3, r.N, i);
-        }
-        atomicAdd(&r.ctl->refined, have_p ? 1ull : 2ull);
+    const float* xr = static_cast<const float*>(d.X) + i * d.Dp;
+    float* prow = static_cast<float*>(d.P) + i * d.Dp;
+    for (int c = t; c < d.nchunks; c += n) {
+        float v[4];
+        ld4(xr + 4 * c, v);
+        st4(prow + 4 * c, v);
     }
 }
 
-__global__ void rot_fix32(const RotDev r)
+__global__ void __launch_bounds__(64) rot_fix32(const RotDev r)
 {
-    const int lane = threadIdx.x & 31;
+    __shared__ Fit32 sh[2];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const InstDev& d = *r.inst;
     const unsigned n = r.ctl->n1;
     if (!PSSO_CHK(n <= r.N, CHK_LIST, n)) return;
-    const long long nwarps = (long long)gridDim.x * (blockDim.x >> 5);
-    for (long long e = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); e < (long long)n;
-         e += nwarps) {
-        switch (d.maxc) {
-        case 1: fix32_one<1>(r, d, e, lane); break;
-        case 2: fix32_one<2>(r, d, e, lane); break;
-        case 4: fix32_one<4>(r, d, e, lane); break;
-        default: fix32_one<8>(r, d, e, lane); break;
+    const int64_t g = r.ctl->gen;
+    for (long long e = blockIdx.x; e < (long long)n; e += gridDim.x) {
+        const int32_t i = r.list1[e];
+        if (!PSSO_CHK(i >= 0 && i < r.N, CHK_ROT_ROW, i)) continue;
+        const bool have_p = (d.pflag[i] & 1u) != 0;
+        float plo = d.plo[i], phi = d.phi[i];
+        __syncthreads();                      // the previous entry's results are consumed
+        if (warp == 0 || !have_p) {
+            const size_t at = (size_t)(2 * e + warp) * d.Dp;
+            const Fit32 f = fit_refined(r, d, r.z32 + at, r.ez32 + at, lane);
+            if (lane == 0) sh[warp] = f;
+        }
+        __syncthreads();
+        const Fit32 fx = sh[0];
+        const float lox = __fsub_rd(fx.f, fx.E), hix = __fadd_ru(fx.f, fx.E);
+        if (!have_p) {       // the pBest's interval, tightened the same way (intersection of two bounds)
+            const Fit32 fp = sh[1];
+            plo = fmaxf(plo, __fsub_rd(fp.f, fp.E));
+            phi = fminf(phi, __fadd_ru(fp.f, fp.E));
+        }
+        const bool accept = hix < plo;
+        const bool reject = lox > phi;
+        if (accept) accept_row(d, i, threadIdx.x, 64);
+        if (threadIdx.x == 0) {
+            if (accept) {
+                d.plo[i] = lox;
+                d.phi[i] = hix;
+                d.pflag[i] = 0u;
+                d.pf64[i] = 0.0;
+                d.pver[i] = (uint32_t)g;
+                atomicAdd(&r.ctl->acc, 1ull);
+            } else {
+                d.plo[i] = plo;
+                d.phi[i] = phi;
+                if (!reject) list_push(r.list3, &r.ctl->n3, r.N, i);
+            }
+            atomicAdd(&r.ctl->refined, have_p ? 1ull : 2ull);
         }
     }
 }
@@ -562,16 +566,38 @@ __global__ void split_m64(const double* M64, long long DD, float* Mh, float* Ml)
     }
 }
 
-// ---- 4/7. FP64 rotation of listed rows ------------------------------------------------
+// M^T for the FP64 rotation (setup): tiles of 32 x 32 through shared memory.
+__global__ void transpose_m64(const double* __restrict__ M, int D, double* __restrict__ Mt)
+{
+    __shared__ double tile[32][33];
+    const int x = blockIdx.x * 32, y = blockIdx.y * 32;
+    for (int r = threadIdx.y; r < 32; r += blockDim.y)
+        if (y + r < D && x + (int)threadIdx.x < D) tile[r][threadIdx.x] = M[(size_t)(y + r) * D + x + threadIdx.x];
+    __syncthreads();
+    for (int r = threadIdx.y; r < 32; r += blockDim.y)
+        if (x + r < D && y + (int)threadIdx.x < D) Mt[(size_t)(x + r) * D + y + threadIdx.x] = tile[threadIdx.x][r];
+}
+
+// ---- 4/7. FP64 rotation of listed rows and their terms -----------------------------------
 // which = 1: entries of list3, row 2e = X_i and row 2e+1 = P_i when its FP64
-// value is not known; which = 2: entries of list2, row 2e+1 = P_i.
-__global__ void rot_z64(const RotDev r, int which)
+// value is not known; which = 2 or 4: entries of list2, row 2e+1 = P_i.
+//
+// One thread per output: z_j is a chain of D dependent FP64 fmas (the oracle's
+// order, k ascending from +0).  An FP64 instruction takes 64 clocks and a warp
+// has one in flight, so a chain of 1000 is 31 us however few rows there are;
+// M^T (outputs of neighbouring threads side by side, 16 loads in flight) keeps
+// the loads off that chain.  The thread then makes its variable's FP64 term
+// too, where every output has a thread, and leaves the sums to rot_fix:
+//   ellipsoid z^2;  Rastrigin z^2 + 20 sin^2(pi z);  Ackley z and sin(pi r).
+constexpr int Z64_AHEAD = 16;
+__global__ void __launch_bounds__(128) rot_z64(const RotDev r, int which)
 {
     __shared__ double dsh[1024];
     const InstDev& d = *r.inst;
     const unsigned n = which == 1 ? r.ctl->n3 : r.ctl->n2;   // which 2 or 4: list 2
     const int D = r.D;
     if (!PSSO_CHK(n <= r.N && D <= 1024, CHK_LIST, n)) return;
+    const int fn = base_fn(r.fn);
     const int nJb = (D + 127) / 128;
     const long long items = (long long)n * 2 * nJb;
     for (long long it = blockIdx.x; it < items; it += gridDim.x) {
@@ -587,58 +613,125 @@ __global__ void rot_z64(const RotDev r, int which)
         for (int k = threadIdx.x; k < D; k += blockDim.x) dsh[k] = __dsub_rn((double)src[k], d.o64[k]);
         __syncthreads();
         const int j = jb * 128 + threadIdx.x;
-        double* out = r.zbuf + (size_t)(2 * e + row) * d.Dp;
+        const double* mt = r.Mt + (j < D ? j : D - 1);
+        double a[Z64_AHEAD], z = 0.0;
+#pragma unroll
+        for (int q = 0; q < Z64_AHEAD; ++q) a[q] = q < D ? __ldg(mt + (size_t)q * D) : 0.0;
+        int k = 0;
+        for (; k + 2 * Z64_AHEAD <= D; k += Z64_AHEAD) {
+            double b[Z64_AHEAD];
+#pragma unroll
+            for (int q = 0; q < Z64_AHEAD; ++q) b[q] = __ldg(mt + (size_t)(k + Z64_AHEAD + q) * D);
+#pragma unroll
+            for (int q = 0; q < Z64_AHEAD; ++q) z = __fma_rn(a[q], dsh[k + q], z);
+#pragma unroll
+            for (int q = 0; q < Z64_AHEAD; ++q) a[q] = b[q];
+        }
+#pragma unroll
+        for (int q = 0; q < Z64_AHEAD; ++q)
+            if (k + q < D) z = __fma_rn(a[q], dsh[k + q], z);
+        for (k += Z64_AHEAD; k < D; ++k) z = __fma_rn(__ldg(mt + (size_t)k * D), dsh[k], z);
         if (j < D) {
-            const double* mrow = d.M64 + (size_t)j * D;
-            double z = 0.0;
-            for (int k = 0; k < D; ++k) z = __fma_rn(__ldg(mrow + k), dsh[k], z);
-            out[j] = z;
-        } else if (j < d.Dp) {
-            out[j] = 0.0;
+            const size_t at = (size_t)(2 * e + row) * d.Dp + j;
+            if (fn == FN_ELLIPSOID) {
+                r.zbuf[at] = __dmul_rn(z, z);
+            } else if (fn == FN_RASTRIGIN) {
+                r.zbuf[at] = __fma_rn(z, z, __dmul_rn(20.0, sinpi_sq_f64(z)));
+            } else {
+                r.zbuf[at] = z;
+                r.sbuf[at] = sinpi_reduced_f64(__dsub_rn(z, rint(z)));
+            }
         }
     }
 }
 
 // ---- 5/8. FP64 fitness of the rotated rows and the exact decisions --------------------
-__device__ void fix_one(const RotDev& r, const InstDev& d, int which, long long e, int lane)
+// One warp's sum over a row's stored values in the oracle's order: lane
+// partials in ascending variable order from +0, then the xor butterfly.
+//   kind 0: sum t_j (Rastrigin's terms); 1: sum w_j t_j (ellipsoid);
+//   2: sum t_j^2 (Ackley's z and sines).
+__device__ double sum_row(const InstDev& d, const double* t, int kind, int lane)
 {
-    Hot hz = hot_of(d);
-    hz.fn = base_fn(d.fn);   // the rows hold z already: the unrotated function with o = 0
-    hz.o64 = r.zero64;
+    double acc = 0.0, nx[4];
+    int c = lane;
+    if (c < d.nchunks) ld4(t + 4 * c, nx);
+#pragma unroll 1
+    while (c < d.nchunks) {
+        double v[4];
+#pragma unroll
+        for (int m = 0; m < 4; ++m) v[m] = nx[m];
+        const int c0 = c;
+        c += 32;
+        if (c < d.nchunks) ld4(t + 4 * c, nx);       // the next chunk travels while this one is added
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+            if (4 * c0 + m >= d.D) break;
+            if (kind == 0) acc = __dadd_rn(acc, v[m]);
+            else if (kind == 1) acc = __fma_rn(__ldg(d.w64 + 4 * c0 + m), v[m], acc);
+            else acc = __fma_rn(v[m], v[m], acc);
+        }
+    }
+#pragma unroll 1
+    for (int off = 16; off > 0; off >>= 1) acc = __dadd_rn(acc, __shfl_xor_sync(0xffffffffu, acc, off));
+    return acc;
+}
+
+// One block of four warps per entry: warp 2 s + row sums row `row` (X_i, P_i),
+// Ackley's second sum on s = 1.  The terms are rot_z64's, so a sum is 32
+// dependent additions per lane (76 -> 9 us per launch, rotated Rastrigin,
+// D = 1000, against evaluating the row's terms in one warp).
+__global__ void __launch_bounds__(128) rot_fix(const RotDev r, int which)
+{
+    __shared__ double sums[2][2], fit[2];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const InstDev& d = *r.inst;
+    const int fn = base_fn(r.fn);
+    const unsigned n = which == 1 ? r.ctl->n3 : r.ctl->n2;
+    if (!PSSO_CHK(n <= r.N, CHK_LIST, n)) return;
     const int64_t g = r.ctl->gen;
-    const double* zx = r.zbuf + (size_t)(2 * e) * d.Dp;
-    const double* zp = zx + d.Dp;
-    if (which == 1) {
-        const int32_t i = r.list3[e];
-        if (!PSSO_CHK(i >= 0 && i < r.N, CHK_ROT_ROW, i)) return;
-        const bool have_p = (d.pflag[i] & 1u) != 0;
-        const double fx = fit64_row<double>(hz, zx, false);
-        const double fp = have_p ? d.pf64[i] : fit64_row<double>(hz, zp, false);
-        const bool accept = fx <= fp;
-        if (accept) {
-            const float* xr = static_cast<const float*>(d.X) + (int64_t)i * d.Dp;
-            float* prow = static_cast<float*>(d.P) + (int64_t)i * d.Dp;
-            for (int c = lane; c < d.nchunks; c += 32) {
-                float v[4];
-                ld4(xr + 4 * c, v);
-                st4(prow + 4 * c, v);
+    const int row = warp & 1, second = warp >> 1;
+    for (long long e = blockIdx.x; e < (long long)n; e += gridDim.x) {
+        const int32_t i = which == 1 ? r.list3[e] : r.list2[e];
+        if (!PSSO_CHK(i >= 0 && i < r.N, CHK_ROT_ROW, i)) continue;
+        const bool have_p = which == 1 && (d.pflag[i] & 1u) != 0;
+        const double known = have_p ? d.pf64[i] : 0.0;
+        const bool mine = row == 0 ? which == 1 : !have_p;
+        __syncthreads();                     // the previous entry's results are consumed
+        if (mine && (second == 0 || fn == FN_ACKLEY)) {
+            const size_t at = (size_t)(2 * e + row) * d.Dp;
+            const double s = sum_row(d, (second ? r.sbuf : r.zbuf) + at,
+                                     fn == FN_RASTRIGIN ? 0 : fn == FN_ELLIPSOID ? 1 : 2, lane);
+            if (lane == 0) sums[row][second] = s;
+        }
+        __syncthreads();
+        if (mine && second == 0 && lane == 0) {
+            double f = sums[row][0];
+            if (fn == FN_ACKLEY) {
+                const double Dd = (double)d.D;
+                const double A = __dsqrt_rn(__ddiv_rn(f, Dd));
+                const double B = expm1_f64(__dmul_rn(-0.2, A));
+                const double C = expm1_f64(__dmul_rn(-2.0, __ddiv_rn(sums[row][1], Dd)));
+                f = -__dadd_rn(__dmul_rn(20.0, B), __dmul_rn(0x1.5bf0a8b145769p+1, C));   // e
             }
+            fit[row] = f;
         }
-        if (lane == 0) {
-            const double v = accept ? fx : fp;
-            d.pf64[i] = v;
-            d.pflag[i] = 1u;
-            d.plo[i] = f64_to_f32_rd(v);
-            d.phi[i] = f64_to_f32_ru(v);
-            if (accept) d.pver[i] = (uint32_t)g;
-            atomicAdd(&r.ctl->rck, have_p ? 1ull : 2ull);
-            if (accept) atomicAdd(&r.ctl->acc, 1ull);
-        }
-    } else {   // list 2 (which 2: in a generation; 4: on demand, outside the counters)
-        const int32_t i = r.list2[e];
-        if (!PSSO_CHK(i >= 0 && i < r.N, CHK_ROT_ROW, i)) return;
-        const double fp = fit64_row<double>(hz, zp, false);
-        if (lane == 0) {
+        __syncthreads();
+        if (which == 1) {
+            const double fx = fit[0], fp = have_p ? known : fit[1];
+            const bool accept = fx <= fp;
+            if (accept) accept_row(d, i, threadIdx.x, 128);
+            if (threadIdx.x == 0) {
+                const double v = accept ? fx : fp;
+                d.pf64[i] = v;
+                d.pflag[i] = 1u;
+                d.plo[i] = f64_to_f32_rd(v);
+                d.phi[i] = f64_to_f32_ru(v);
+                if (accept) d.pver[i] = (uint32_t)g;
+                atomicAdd(&r.ctl->rck, have_p ? 1ull : 2ull);
+                if (accept) atomicAdd(&r.ctl->acc, 1ull);
+            }
+        } else if (threadIdx.x == 0) {   // list 2 (which 2: in a generation; 4: on demand, outside the counters)
+            const double fp = fit[1];
             d.pf64[i] = fp;
             d.pflag[i] = 1u;
             d.plo[i] = f64_to_f32_rd(fp);
@@ -648,59 +741,117 @@ __device__ void fix_one(const RotDev& r, const InstDev& d, int which, long long 
     }
 }
 
-__global__ void rot_fix(const RotDev r, int which)
-{
-    const int lane = threadIdx.x & 31;
-    const InstDev& d = *r.inst;
-    const unsigned n = which == 1 ? r.ctl->n3 : r.ctl->n2;
-    if (!PSSO_CHK(n <= r.N, CHK_LIST, n)) return;
-    const long long nwarps = (long long)gridDim.x * (blockDim.x >> 5);
-    for (long long e = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); e < (long long)n;
-         e += nwarps)
-        fix_one(r, d, which, e, lane);
-}
-
 
 // ---- 6/9. gBest --------------------------------------------------------------------------
+// Lowest-index arg-min of the pBest bounds by one block: only the keys are
+// read and reduced (the smallest and second-smallest lower bound, the first's
+// index, the smallest upper bound), four particles per thread and load; the
+// winner's other fields are read afterwards (12.3 -> 5 us at N = 8192).
+struct Key {
+    float l1, l2, mh;
+    int i;
+};
+__device__ __forceinline__ Key key_merge(const Key& a, const Key& b)
+{
+    const bool bf = b.l1 < a.l1 || (b.l1 == a.l1 && b.i < a.i);
+    Key r;
+    r.l1 = bf ? b.l1 : a.l1;
+    r.i = bf ? b.i : a.i;
+    r.l2 = fminf(fminf(a.l2, b.l2), bf ? a.l1 : b.l1);
+    r.mh = fminf(a.mh, b.mh);
+    return r;
+}
+__device__ __forceinline__ Key key_warp(Key k)
+{
+#pragma unroll 1
+    for (int off = 16; off > 0; off >>= 1) {
+        Key o;
+        o.l1 = __shfl_xor_sync(0xffffffffu, k.l1, off);
+        o.l2 = __shfl_xor_sync(0xffffffffu, k.l2, off);
+        o.mh = __shfl_xor_sync(0xffffffffu, k.mh, off);
+        o.i = __shfl_xor_sync(0xffffffffu, k.i, off);
+        k = key_merge(k, o);
+    }
+    return k;
+}
+
+// FP64 value and index, compared as integers (order_key): a compare of doubles
+// takes the FP64 unit's 64 clocks.
+struct Exact {
+    long long v;
+    int i;
+};
+__device__ __forceinline__ Exact exact_merge(const Exact& a, const Exact& b)
+{
+    return (b.v < a.v || (b.v == a.v && b.i < a.i)) ? b : a;
+}
+__device__ __forceinline__ Exact exact_warp(Exact k)
+{
+#pragma unroll 1
+    for (int off = 16; off > 0; off >>= 1) {
+        Exact o;
+        o.v = __shfl_xor_sync(0xffffffffu, k.v, off);
+        o.i = __shfl_xor_sync(0xffffffffu, k.i, off);
+        k = exact_merge(k, o);
+    }
+    return k;
+}
+
 __global__ void __launch_bounds__(1024) rot_argmin(const RotDev r, int phase)
 {
-    __shared__ Cand sh[32];
+    __shared__ Key shk[32];
+    __shared__ Exact she[32];
     __shared__ unsigned n2;
+    __shared__ long long winner;
     const InstDev& d = *r.inst;
     RotCtl* ctl = r.ctl;
     const int64_t g = ctl->gen;
-    const int64_t N = d.N;
+    const int N = (int)d.N, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (phase == 0) {
-        Cand c = cand_none();
-        for (int64_t i = threadIdx.x; i < N; i += blockDim.x)
-            c = cand_merge<true>(c, cand_of<true>((long long)i, d.pf64[i], d.plo[i], d.phi[i],
-                                                  (int)(d.pflag[i] & 1u), d.pver[i]));
-        const Cand b = block_reduce_cand<true>(c, sh);
-        if (b.l2 > b.mh) {          // one interval lies below every other: the arg-min
+        Key k = {FLT_MAX, FLT_MAX, FLT_MAX, INT_MAX};
+        for (int i = 4 * (int)threadIdx.x; i < N; i += 4096) {
+            if (i + 4 <= N) {
+                float lo[4], hi[4];
+                ld4(d.plo + i, lo);
+                ld4(d.phi + i, hi);
+#pragma unroll
+                for (int m = 0; m < 4; ++m) k = key_merge(k, Key{lo[m], FLT_MAX, hi[m], i + m});
+            } else {
+                for (int m = i; m < N; ++m) k = key_merge(k, Key{d.plo[m], FLT_MAX, d.phi[m], m});
+            }
+        }
+        k = key_warp(k);
+        if (lane == 0) shk[warp] = k;
+        __syncthreads();
+        k = key_warp(shk[lane]);           // 32 warps: every warp has the block's result
+        if (k.i >= N) k.i = 0;             // no finite bound at all
+        if (k.l2 > k.mh) {                 // one interval lies below every other: the arg-min
             if (threadIdx.x == 0) {
                 // the gBest value the generation reports must lie within 1e-6 of
                 // FP64: an interval too wide for that gets the winner's FP64 value
                 // (list 2; the exact pass of phase 1 then keeps the same winner)
-                const bool wide = !b.has1 && too_wide(r.fn, b.l1, b.h1);
+                const int has = (int)(d.pflag[k.i] & 1u);
+                const float hi = d.phi[k.i];
+                const bool wide = !has && too_wide(r.fn, k.l1, hi);
                 ctl->amb = wide ? 1 : 0;
                 if (wide) {
-                    r.list2[0] = (int32_t)b.i;
+                    r.list2[0] = k.i;
                     ctl->n2 = 1;
                 }
-                ctl->win_i = b.i;
-                ctl->win_v = b.v;
-                ctl->win_lo = b.l1;
-                ctl->win_hi = b.h1;
-                ctl->win_has = b.has1;
-                ctl->win_ver = b.ver;
+                ctl->win_i = k.i;
+                ctl->win_v = has ? d.pf64[k.i] : DBL_MAX;
+                ctl->win_lo = k.l1;
+                ctl->win_hi = hi;
+                ctl->win_has = has;
+                ctl->win_ver = d.pver[k.i];
             }
             return;
         }
         // several pBests may be the minimum: those without an FP64 value go on list2
         if (threadIdx.x == 0) n2 = 0;
         __syncthreads();
-        for (int64_t i = threadIdx.x; i < N; i += blockDim.x)
-            if (d.plo[i] <= b.mh && !(d.pflag[i] & 1u)) list_push(r.list2, &n2, r.N, (int32_t)i);
+        for (int i = threadIdx.x; i < N; i += blockDim.x)
+            if (d.plo[i] <= k.mh && !(d.pflag[i] & 1u)) list_push(r.list2, &n2, r.N, i);
         __syncthreads();
         if (threadIdx.x == 0) {
             ctl->amb = 1;
@@ -712,27 +863,29 @@ __global__ void __launch_bounds__(1024) rot_argmin(const RotDev r, int phase)
     if (ctl->amb) {
         // every pBest that can be the minimum now has its FP64 value; the others
         // have a lower bound above the smallest upper bound
-        Cand c = cand_none();
-        for (int64_t i = threadIdx.x; i < N; i += blockDim.x)
-            if (d.pflag[i] & 1u) {
-                Cand q = cand_none();
-                q.v = d.pf64[i];
-                q.i = (long long)i;
-                q.ver = d.pver[i];
-                c = cand_merge<false>(c, q);
-            }
-        const Cand b = block_reduce_cand<false>(c, sh);
-        if (threadIdx.x == 0) {
-            ctl->win_i = b.i;
-            ctl->win_v = b.v;
-            ctl->win_lo = f64_to_f32_rd(b.v);
-            ctl->win_hi = f64_to_f32_ru(b.v);
-            ctl->win_has = 1;
-            ctl->win_ver = b.ver;
-        }
+        Exact k = {LLONG_MAX, INT_MAX};
+        for (int i = threadIdx.x; i < N; i += blockDim.x)
+            if (d.pflag[i] & 1u) k = exact_merge(k, Exact{order_key(d.pf64[i]), i});
+        k = exact_warp(k);
+        if (lane == 0) she[warp] = k;
         __syncthreads();
+        k = exact_warp(she[lane]);
+        if (k.i >= N) k.i = 0;
+        if (threadIdx.x == 0) {
+            const double v = d.pf64[k.i];
+            ctl->win_i = k.i;
+            ctl->win_v = v;
+            ctl->win_lo = f64_to_f32_rd(v);
+            ctl->win_hi = f64_to_f32_ru(v);
+            ctl->win_has = 1;
+            ctl->win_ver = d.pver[k.i];
+            winner = k.i;
+        }
+    } else if (threadIdx.x == 0) {
+        winner = ctl->win_i;
     }
-    const long long wi = ctl->win_i;
+    __syncthreads();
+    const long long wi = winner;
     const float* src = static_cast<const float*>(d.P) + wi * d.Dp;
     float* dst = static_cast<float*>(d.gbrow);
     for (int j = threadIdx.x; j < d.Dp; j += blockDim.x) dst[j] = src[j];
@@ -780,7 +933,7 @@ cudaError_t exact_values_for_read(const RotHost& h, cudaStream_t s)
     clear_n2<<<1, 1, 0, s>>>(r.ctl);
     list_wide<<<(unsigned)std::min<long long>((h.N + 255) / 256, 1024), 256, 0, s>>>(r);
     rot_z64<<<h.z64_grid, 128, 0, s>>>(r, 4);
-    rot_fix<<<h.fix_grid, 256, 0, s>>>(r, 4);
+    rot_fix<<<h.fix_grid, 128, 0, s>>>(r, 4);
     clear_n2<<<1, 1, 0, s>>>(r.ctl);
     return cudaGetLastError();
 }
@@ -812,17 +965,17 @@ cudaError_t enqueue_generation_timed(const RotHost& h, cudaStream_t s, cudaEvent
     mark();
     rot_z32<<<h.z32_grid, 128, 0, s>>>(r);
     mark();
-    rot_fix32<<<h.fix_grid, 32 * wpb, 0, s>>>(r);
+    rot_fix32<<<h.fix_grid, 64, 0, s>>>(r);
     mark();
     rot_z64<<<h.z64_grid, 128, 0, s>>>(r, 1);
     mark();
-    rot_fix<<<h.fix_grid, 32 * wpb, 0, s>>>(r, 1);
+    rot_fix<<<h.fix_grid, 128, 0, s>>>(r, 1);
     mark();
     rot_argmin<<<1, 1024, 0, s>>>(r, 0);
     mark();
     rot_z64<<<h.z64_grid, 128, 0, s>>>(r, 2);
     mark();
-    rot_fix<<<h.fix_grid, 32 * wpb, 0, s>>>(r, 2);
+    rot_fix<<<h.fix_grid, 128, 0, s>>>(r, 2);
     mark();
     rot_argmin<<<1, 1024, 0, s>>>(r, 1);
     mark();
@@ -923,6 +1076,8 @@ cudaError_t build_constants(const RotHost& h, cudaStream_t s)
     split_m64<<<(unsigned)std::min<long long>((DD + 255) / 256, 4096), 256, 0, s>>>(h.M64, DD, h.Mh, h.Ml);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
+    const unsigned tiles = (unsigned)((r.D + 31) / 32);
+    transpose_m64<<<dim3(tiles, tiles), dim3(32, 8), 0, s>>>(h.M64, r.D, h.Mt);
     slice_matrix<<<r.Jp, 256, 0, s>>>(h.M64, r.D, r.Jp, r.Kp, h.B, r.mscale, r.ml1);
     return cudaGetLastError();
 }

@@ -46,8 +46,9 @@ struct RotDev {
     const float* Ml;
     float* z32;                    // [2N][Dp] refined z rows of list1 particles
     float* ez32;                   // [2N][Dp] their error bounds
-    double* zbuf;                  // [2N][Dp] FP64 z rows of listed particles
-    const double* zero64;          // [Dp] zeros
+    const double* Mt;              // [D][D] M^T (FP64 rotation: outputs side by side)
+    double* zbuf;                  // [2N][Dp] FP64 terms of listed particles (rot_z64)
+    double* sbuf;                  // [2N][Dp] Ackley's sines of the same rows (else null)
     RotCtl* ctl;
 };
 
@@ -57,6 +58,7 @@ struct RotHost {
     __nv_bfloat16* B;              // [4][Jp][Kp] integer slices of M32
     float* Mh;                     // float pair of M (refinement)
     float* Ml;
+    double* Mt;                    // M^T
     const float* M32;
     const double* M64;
     long long N;
