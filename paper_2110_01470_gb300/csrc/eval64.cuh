@@ -179,7 +179,8 @@ inline cudaError_t launch_fn(const Hot& in, const double* X, int64_t pitch, int6
 {
     const size_t smem = (size_t)WARPS * rows * row_pitch(in.nchunks) * sizeof(double) * (two_sums<FN> ? 2 : 1);
     if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(eval64<FN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        // an SM's whole 227 KB, whatever this call uses: calls on other threads share the kernel
+        const cudaError_t e = cudaFuncSetAttribute(eval64<FN>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
         if (e != cudaSuccess) return e;
     }
     const int64_t per_block = (int64_t)WARPS * rows;

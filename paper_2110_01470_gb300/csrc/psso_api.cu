@@ -390,7 +390,8 @@ psso_status plan(psso_ctx* h)
         }
         if (smem > (size_t)prop.sharedMemPerBlockOptin - 8192)
             return fail(PSSO_ERR_UNSUPPORTED, "per-block gBest rows exceed shared memory");
-        CUDA_TRY(set_smem_of(h->variant, h->mc_index, smem));
+        // the kernel's limit, not this handle's use: handles of other sizes share the kernel
+        CUDA_TRY(set_smem_of(h->variant, h->mc_index, (size_t)prop.sharedMemPerBlockOptin - 8192));
         int bps2 = 0;
         CUDA_TRY(occupancy_of(h->variant, h->mc_index, TB, smem, &bps2));
         if ((int64_t)bps2 * prop.multiProcessorCount >= nblocks) {
