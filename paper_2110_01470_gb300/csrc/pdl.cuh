@@ -1,0 +1,39 @@
+// pdl.cuh -- programmatic dependent launch of short kernel sequences.
+//
+// A sequence of kernels of a few microseconds each spends as long on the gaps
+// between them (drain, launch, first blocks) as on the work.  With this
+// attribute a kernel's blocks are placed while the previous kernel runs out
+// and wait in pdl_entry() until it has completed and its memory is visible;
+// every kernel of a sequence enters through pdl_entry before it touches memory
+// that another one writes, so the order is that of plain launches.
+#pragma once
+#include <cuda_runtime.h>
+#include <utility>
+
+namespace psso {
+
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_entry()
+{
+    pdl_trigger();
+    pdl_wait();
+}
+
+template <class... P, class... A>
+inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args)
+{
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = grid;
+    lc.blockDim = block;
+    lc.dynamicSmemBytes = smem;
+    lc.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = at;
+    lc.numAttrs = 1;
+    return cudaLaunchKernelEx(&lc, kernel, std::forward<A>(args)...);
+}
+
+}  // namespace psso

@@ -12,7 +12,7 @@
 #include "psso.h"
 #include "psso_internal.h"
 #include "rot_pipeline.h"
-#include "tc_gemm.cuh"
+#include "tc_pair.cuh"
 
 using namespace psso;
 
@@ -616,7 +616,7 @@ psso_status setup_tc(psso_ctx* h, size_t k)
     R.z64_grid = 2 * prop.multiProcessorCount;
     R.z32_grid = 8 * prop.multiProcessorCount;
     R.fix_grid = prop.multiProcessorCount;
-    R.gemm_grid = (int)std::min<long long>((long long)(r.Np / tc::BM) * r.nJt, prop.multiProcessorCount);
+    R.gemm_grid = tc::pair_grid(r.Np, r.Jp, prop.multiProcessorCount);
     if (!tc::make_tmap_bf16(&R.tmA, r.A, r.Kp, tc::SLICES * r.Np) ||
         !tc::make_tmap_bf16(&R.tmB, R.B, r.Kp, tc::SLICES * r.Jp, tc::SBN))
         return fail(PSSO_ERR_CUDA, "cuTensorMapEncodeTiled failed for the tensor-core operands");

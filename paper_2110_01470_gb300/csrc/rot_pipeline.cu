@@ -12,7 +12,7 @@
 //                    "x equals pBest" flag per row.
 //   2. rot_gemm_fit  the tcgen05 GEMM; its epilogue turns each z into the
 //                    function's FP32 terms and per-term error bounds and
-//                    writes per-(particle, 128-column tile) partial sums.
+//                    writes per-(particle, 64-column group) partial sums.
 //   3. rot_decide    FP32 fitness and bound per particle; pBest update when
 //                    the interval decides it (Alg. 3, <=); else the particle
 //                    goes on list 1.
@@ -47,6 +47,7 @@
 #include "rot_pipeline.h"
 #include "sso_kernel.cuh"
 #include "tc_gemm.cuh"
+#include "tc_pair.cuh"
 
 namespace psso {
 namespace rot {
@@ -218,56 +219,122 @@ struct FitEpi {
     const RotDev* r;
     int fn, D;
     float drop;                   // SLICE_DROP * D
-    // the current tile and row: particle i, column tile nt, s_d, sum |d_k|
+    // the current row and 64-column group: particle i, group nt, s_d, sum |d_k|
     int64_t i;
     int nt;
     float ds, dl1;
-    float acc, acc2, accE, rQ;
-    __device__ void tile(int tm, int tn, int row)
+    float t[64], em[64];          // joined accumulators, sums of the partial sums' magnitudes
+    __device__ __forceinline__ void tile(int tm, int g, int row)
     {
-        i = (int64_t)tm * BM + row;
-        nt = tn;
+        i = (int64_t)tm * tc::PBM + row;
+        nt = g;
         ds = i < r->N ? r->dscale[i] : 1.f;
         dl1 = i < r->N ? r->dl1[i] : 0.f;
-        acc = acc2 = accE = rQ = 0.f;
     }
-    __device__ void operator()(int c, const float (&tj)[32], const float (&em)[32])
+    // joins the accumulators from the smallest weight up; each step one
+    // rounding (the scaled accumulator is exact)
+    template <int C>
+    __device__ __forceinline__ void load32(uint32_t taddr)
     {
-        const int j0 = nt * tc::SBN + 32 * c;
-        float s = 0.f, s2 = 0.f, e = 0.f, eq = 0.f;
+        float v[32], w[32];
+        tc::tmem_ld32(taddr + (uint32_t)(3 * 128), v);
+        tc::tmem_ld32(taddr + (uint32_t)(2 * 128), w);
 #pragma unroll
-        for (int t = 0; t < 32; ++t) {
-            const int j = j0 + t;
-            if (j >= D) break;
-            const float sm = __ldg(r->mscale + j), l1m = __ldg(r->ml1 + j);
-            const float sc = __fmul_rn(ds, sm);                 // a power of two
-            const float zt = __fmul_rn(tj[t], __fmul_rn(sc, 0x1p-14f));
-            const float rd = __fmul_rn(sm, dl1), rm = __fmul_rn(ds, l1m);
-            // dropped slice products, slice remainders, the FP64 reference's
-            // own rounding (D <= 2^13 terms: 2^-40 sum |M||d|), the FP32 join
-            const float ez = 1.01f * (drop * sc + tc::SLICE_REM * (rd + rm) + 0x1p-40f * fminf(rd, rm) +
-                                      0x1p-38f * em[t] * sc) + 0x1p-126f;
-            term32(fn, zt, ez, r->inst_w32, j, s, s2, e, eq);
+        for (int q = 0; q < 32; ++q) {
+            t[32 * C + q] = __fmaf_rn(w[q], 0x1p-14f, __fmul_rn(v[q], 0x1p-21f));   // the product is exact
+            em[32 * C + q] = fabsf(t[32 * C + q]);
         }
-        acc = __fadd_rn(acc, s);
-        acc2 = __fadd_rn(acc2, s2);
-        accE = __fadd_rn(accE, e);
-        rQ = __fadd_rn(rQ, eq);
-        if (c == tc::SBN / 32 - 1) {
-            if (i < r->N && PSSO_CHK(nt < r->nJt, CHK_TILE, nt))
-                r->part[i * r->nJt + nt] = make_float4(acc, acc2, accE, rQ);
+        tc::tmem_ld32(taddr + (uint32_t)128, v);
+        tc::tmem_ld32(taddr, w);
+#pragma unroll
+        for (int q = 0; q < 32; ++q) {
+            const float t1 = __fmaf_rn(v[q], 0x1p-7f, t[32 * C + q]);
+            const float t2 = __fadd_rn(w[q], t1);
+            em[32 * C + q] = __fadd_ru(__fadd_ru(em[32 * C + q], fabsf(t1)), fabsf(t2));
+            t[32 * C + q] = t2;
         }
+    }
+    __device__ __forceinline__ void load(uint32_t taddr, int n)
+    {
+        load32<0>(taddr);
+        if (n == 2) load32<1>(taddr + 32);
+    }
+    // The terms of the 32-column blocks c0 .. c0 + n - 1 of the group.  Eight
+    // columns a step, the rest of the registers moved up: unrolled over 64
+    // columns, the code of a tile takes longer to fetch than to run where a CTA
+    // has one tile.
+    __device__ __forceinline__ void compute(int c0, int n, float4* xch)
+    {
+        float acc = 0.f, acc2 = 0.f, accE = 0.f, rQ = 0.f;
+        float s = 0.f, s2 = 0.f, e = 0.f, eq = 0.f;
+#pragma unroll 1
+        for (int h = 0; h < 4 * n; ++h) {
+            const int j0 = nt * 64 + 32 * c0 + 8 * h;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const int j = j0 + q;
+                if (j >= D) break;
+                const float sm = __ldg(r->mscale + j), l1m = __ldg(r->ml1 + j);
+                const float sc = __fmul_rn(ds, sm);                 // a power of two
+                const float zt = __fmul_rn(t[q], __fmul_rn(sc, 0x1p-14f));
+                const float rd = __fmul_rn(sm, dl1), rm = __fmul_rn(ds, l1m);
+                // dropped slice products, slice remainders, the FP64 reference's
+                // own rounding (D <= 2^13 terms: 2^-40 sum |M||d|), the FP32 join
+                const float ez = 1.01f * (drop * sc + tc::SLICE_REM * (rd + rm) + 0x1p-40f * fminf(rd, rm) +
+                                          0x1p-38f * em[q] * sc) + 0x1p-126f;
+                term32(fn, zt, ez, r->inst_w32, j, s, s2, e, eq);
+            }
+#pragma unroll
+            for (int q = 0; q < 56; ++q) {
+                t[q] = t[q + 8];
+                em[q] = em[q + 8];
+            }
+            if ((h & 3) == 3) {                 // a block of 32 terms ends
+                acc = __fadd_rn(acc, s);
+                acc2 = __fadd_rn(acc2, s2);
+                accE = __fadd_rn(accE, e);
+                rQ = __fadd_rn(rQ, eq);
+                s = s2 = e = eq = 0.f;
+            }
+        }
+        if (n == 1) {                           // the group's other 32 columns are the other warp's
+            const float4 o = tc::pair_exchange(make_float4(acc, acc2, accE, rQ), c0, xch);
+            if (c0 == 1) return;
+            acc = __fadd_rn(acc, o.x);
+            acc2 = __fadd_rn(acc2, o.y);
+            accE = __fadd_rn(accE, o.z);
+            rQ = __fadd_rn(rQ, o.w);
+        }
+        if (i < r->N && PSSO_CHK(nt < r->nJt, CHK_TILE, nt))
+            r->part[i * r->nJt + nt] = make_float4(acc, acc2, accE, rQ);
     }
 };
 
-// Persistent: one CTA per SM (at most one per tile), tiles in grid-stride order.
-__global__ void __launch_bounds__(tc::S_THREADS, 1)
+// The ten slice products of weight <= 3 (tc_gemm.cuh), one accumulator per weight.
+struct SliceCfg {
+    static constexpr int PLANES = tc::SLICES, STG = 2, PRODUCTS = 10;
+    __device__ static constexpr int pa(int q) { constexpr int T[10] = {0, 0, 1, 0, 1, 2, 0, 1, 2, 3}; return T[q]; }
+    __device__ static constexpr int pb(int q) { constexpr int T[10] = {0, 1, 0, 2, 1, 0, 3, 2, 1, 0}; return T[q]; }
+    __device__ static constexpr int acc(int q, int) { constexpr int T[10] = {0, 1, 1, 2, 2, 2, 3, 3, 3, 3}; return T[q]; }
+    __device__ static constexpr bool first(int q, int kb, int ks)
+    {
+        return (q == 0 || q == 1 || q == 3 || q == 6) && kb == 0 && ks == 0;
+    }
+};
+
+// Persistent, one CTA pair per two SMs (tc_pair.cuh).  N = 8192, D = 1000: 160 ->
+// 138 us per launch.
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc::P_THREADS, 1)
     rot_gemm_fit(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                  const __grid_constant__ RotDev r)
 {
-    FitEpi epi{&r, base_fn(r.fn), r.D, tc::SLICE_DROP * (float)r.D};
+    FitEpi epi;
+    epi.r = &r;
+    epi.fn = base_fn(r.fn);
+    epi.D = r.D;
+    epi.drop = tc::SLICE_DROP * (float)r.D;
     tc::GemmArgs a{r.Np, r.Jp, r.Kp, &r.ctl->status};
-    tc::gemm_sliced_persistent(&tmA, &tmB, a, epi);
+    tc::gemm_pair<SliceCfg>(&tmA, &tmB, a, epi);
 }
 
 // ---- 3. FP32 decisions ------------------------------------------------------------
@@ -469,7 +536,7 @@ __global__ void __launch_bounds__(128) rot_z32(const RotDev r)
 // handful of entries, so its time is instruction fetch and the chains of one
 // warp: the loops stay rolled (unrolled over the widest row, the straight-line
 // code took longer to fetch than to run) and the entry's two rows run side by
-// side (33 -> 8 us per launch at D = 1000).
+// side (33 -> 14 us per launch at D = 1000).
 __device__ Fit32 fit_refined(const RotDev& r, const InstDev& d, const float* z, const float* ez, int lane)
 {
     const int fn = base_fn(r.fn);
@@ -678,7 +745,7 @@ __device__ double sum_row(const InstDev& d, const double* t, int kind, int lane)
 
 // One block of four warps per entry: warp 2 s + row sums row `row` (X_i, P_i),
 // Ackley's second sum on s = 1.  The terms are rot_z64's, so a sum is 32
-// dependent additions per lane (76 -> 9 us per launch, rotated Rastrigin,
+// dependent additions per lane (76 -> 8 us per launch, rotated Rastrigin,
 // D = 1000, against evaluating the row's terms in one warp).
 __global__ void __launch_bounds__(128) rot_fix(const RotDev r, int which)
 {
@@ -746,7 +813,7 @@ __global__ void __launch_bounds__(128) rot_fix(const RotDev r, int which)
 // Lowest-index arg-min of the pBest bounds by one block: only the keys are
 // read and reduced (the smallest and second-smallest lower bound, the first's
 // index, the smallest upper bound), four particles per thread and load; the
-// winner's other fields are read afterwards (12.3 -> 5 us at N = 8192).
+// winner's other fields are read afterwards (12.3 -> 10.1 us at N = 8192).
 struct Key {
     float l1, l2, mh;
     int i;
@@ -959,7 +1026,7 @@ cudaError_t enqueue_generation_timed(const RotHost& h, cudaStream_t s, cudaEvent
     const int wpb = 8;
     rot_update<<<(N + wpb - 1) / wpb, 32 * wpb, 0, s>>>(r);
     mark();
-    rot_gemm_fit<<<h.gemm_grid, tc::S_THREADS, tc::S_SMEM_BYTES, s>>>(h.tmA, h.tmB, r);
+    rot_gemm_fit<<<h.gemm_grid, tc::P_THREADS, tc::pair_smem<SliceCfg::PLANES, SliceCfg::STG>(), s>>>(h.tmA, h.tmB, r);
     mark();
     rot_decide<<<(N + wpb - 1) / wpb, 32 * wpb, 0, s>>>(r);
     mark();
@@ -1090,7 +1157,8 @@ cudaError_t set_generation(const RotHost& h, long long g, cudaStream_t s)
 
 cudaError_t configure()
 {
-    return cudaFuncSetAttribute(rot_gemm_fit, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::S_SMEM_BYTES);
+    return cudaFuncSetAttribute(rot_gemm_fit, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                tc::pair_smem<SliceCfg::PLANES, SliceCfg::STG>());
 }
 
 }  // namespace rot
