@@ -13,7 +13,7 @@
 #include "psso.h"
 #include "rot_pipeline.h"
 #include "sso_kernel.cuh"
-#include "tc_gemm.cuh"
+#include "tc_pair.cuh"
 
 namespace psso {
 
@@ -342,97 +342,255 @@ cudaError_t launch_polish(const InstDev* inst, int k, int lattice, int owner_ran
 
 // ---------------------------------------------------------------------------
 // Rotated functions on the tensor cores (the *_ws entry points):
-//   forward   Z = (X - O) M^T        split-BF16 tcgen05 GEMM (tc_gemm.cuh)
-//             f_i from row Z_i       the unrotated function's FP32 kernel, o = 0
-//   backward  G_i = grad_f_i df/dz   from Z (same kernel, its z-gradient)
-//             grad_X = G M           second GEMM, B operand = the planes of M^T
-// Both GEMMs run the six split products of tc_gemm.cuh with FP32
+//   forward   planes of d = x - o and of M          prep_planes
+//             Z = (X - O) M^T, its epilogue the     pair GEMM, SumEpi
+//             terms of f summed per row and 64 columns
+//             f_i from the sums                     finish_rows
+//   backward  planes of d, M and M^T                prep_planes
+//             Z = (X - O) M^T                       pair GEMM, StoreEpi
+//             planes of G_i = grad_f_i df/dz        gz_rows
+//             grad_X = G M                          pair GEMM, StoreEpi
+// The GEMMs (tc_pair.cuh) run the six split products of tc_gemm.cuh with FP32
 // accumulation: each output carries an error below 2^-20 per MMA of
 // sum |A_ik| |B_jk| (tc_gemm.cuh), typically far less.
+//
+// Bound: the tensor pipe for large N D^2 (six products each), HBM for the
+// planes, launches for small ones.  Against one CTA per 128 x 128 tile with Z
+// stored a word at a time, a warp per row for f and for the planes of G, and
+// the outputs pre-filled with NaN (forward + backward): rotated Ackley, N =
+// 4096, D = 256: 123 -> 65 us; rotated Rastrigin, N = 8192, D = 1000: 568
+// -> 305 us.
 namespace gtc {
 
 using tc::BM;
 using tc::BN;
 using tc::BK;
 
-// B planes of M^T: row k of the [Jp][Kp] planes holds column k of M.
-__global__ void split_matrix_t(const float* __restrict__ M, int D, int Jp, int Kp, __nv_bfloat16* B)
+// Four consecutive values as the three planes' BF16 (8 bytes each at offset o).
+__device__ __forceinline__ void put_planes(const float (&v)[4], __nv_bfloat16* A, size_t plane, size_t o)
 {
-    const int k = blockIdx.x;
-    const size_t plane = (size_t)Jp * Kp;
-    for (int j = threadIdx.x; j < Kp; j += blockDim.x) {
-        const float v = (k < D && j < D) ? M[(size_t)j * D + k] : 0.f;
-        __nv_bfloat16 h, m, l;
-        tc::split3(v, h, m, l);
-        const size_t o = (size_t)k * Kp + j;
-        B[o] = h;
-        B[plane + o] = m;
-        B[2 * plane + o] = l;
+    uint32_t w[3][2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        __nv_bfloat16 a[3], b[3];
+        tc::split3(v[2 * h], a[0], a[1], a[2]);
+        tc::split3(v[2 * h + 1], b[0], b[1], b[2]);
+#pragma unroll
+        for (int p = 0; p < 3; ++p)
+            w[p][h] = (uint32_t)__bfloat16_as_ushort(a[p]) | ((uint32_t)__bfloat16_as_ushort(b[p]) << 16);
+    }
+#pragma unroll
+    for (int p = 0; p < 3; ++p) *reinterpret_cast<uint2*>(A + p * plane + o) = make_uint2(w[p][0], w[p][1]);
+}
+
+// Values 4 c .. 4 c + 3 of a row of D floats (zero beyond); vec: 16-byte loads.
+__device__ __forceinline__ void row4(const float* row, int c, int D, bool vec, float (&v)[4])
+{
+    if (vec && 4 * c + 4 <= D) {
+        ld4(row + 4 * c, v);
+        return;
+    }
+#pragma unroll
+    for (int m = 0; m < 4; ++m) v[m] = 4 * c + m < D ? __ldg(row + 4 * c + m) : 0.f;
+}
+
+// Operand planes of one call in one launch: a warp per row of X (d = x - o) and
+// per row of M, then 32 x 32 tiles of M^T.  Columns D .. Kp - 1 are zero; rows
+// beyond N and D are left as they are (an output element depends on its own
+// row and column only, and theirs are not stored).
+struct PrepArgs {
+    const float* X;
+    const float* o;
+    const float* M;
+    __nv_bfloat16 *A, *B, *Bt;      // Bt may be null
+    int* status;
+    int N, D, Np, Jp, Kp;
+    int row_blocks;                 // blocks of 8 rows of X and M together
+    bool vec_x, vec_m;
+};
+__global__ void __launch_bounds__(256) prep_planes(const PrepArgs a)
+{
+    __shared__ float tile[32][33];
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a.status = 0;
+    if ((int)blockIdx.x < a.row_blocks) {
+        const int lane = threadIdx.x & 31;
+        const int r = (int)blockIdx.x * 8 + (threadIdx.x >> 5);
+        if (r >= a.N + a.D) return;
+        const bool is_x = r < a.N;
+        const int i = is_x ? r : r - a.N;
+        const float* src = (is_x ? a.X : a.M) + (size_t)i * a.D;
+        __nv_bfloat16* dst = is_x ? a.A : a.B;
+        const size_t plane = (size_t)(is_x ? a.Np : a.Jp) * a.Kp;
+        const bool vec = is_x ? a.vec_x : a.vec_m;
+        for (int c = lane; c < a.Kp / 4; c += 32) {
+            float v[4];
+            row4(src, c, a.D, vec, v);
+            if (is_x) {
+#pragma unroll
+                for (int m = 0; m < 4; ++m)
+                    if (4 * c + m < a.D) v[m] = __fsub_rn(v[m], __ldg(a.o + 4 * c + m));
+            }
+            put_planes(v, dst, plane, (size_t)i * a.Kp + 4 * c);
+        }
+        return;
+    }
+    // Bt[k][j] = M[j][k]: tile (k0, j0)
+    const int t = (int)blockIdx.x - a.row_blocks, nt = a.Kp / 32;
+    const int k0 = (t / nt) * 32, j0 = (t % nt) * 32;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    for (int y = ty; y < 32; y += 8)
+        tile[y][tx] = (j0 + y < a.D && k0 + tx < a.D) ? __ldg(a.M + (size_t)(j0 + y) * a.D + k0 + tx) : 0.f;
+    __syncthreads();
+    const int k = k0 + (threadIdx.x >> 3), c = threadIdx.x & 7;
+    if (k < a.D) {
+        const float v[4] = {tile[4 * c][k - k0], tile[4 * c + 1][k - k0], tile[4 * c + 2][k - k0],
+                            tile[4 * c + 3][k - k0]};
+        put_planes(v, a.Bt, (size_t)a.Jp * a.Kp, (size_t)k * a.Kp + j0 + 4 * c);
     }
 }
 
-// C tile -> out[i * D + j] (rows < N, columns < D).
-struct StoreEpi {
-    float* out;
-    int N, D;
-    __device__ void operator()(int c, const float (&z)[32]) const
+// The terms of f summed over the 64 columns: part[i][g] = (s1, s2) (ellipsoid
+// sum w z^2, Rastrigin sum z^2 + 20 sin^2, Ackley sum z^2 and sum sin^2).
+struct SumEpi : tc::JoinEpi {
+    float2* part;
+    const float* w;
+    int fn, groups;
+    __device__ __forceinline__ void compute(int c0, int n, float4* xch)
     {
-        const int i = blockIdx.x * BM + threadIdx.x;
-        const int j0 = blockIdx.y * BN + 32 * c;
-        if (i >= N) return;
+        float s1 = 0.f, s2 = 0.f;
+#pragma unroll 1
+        for (int h = 0; h < 4 * n; ++h) {            // eight columns a step (short code)
 #pragma unroll
-        for (int t = 0; t < 32; ++t)
-            if (j0 + t < D) out[(size_t)i * D + j0 + t] = z[t];
+            for (int q = 0; q < 8; ++q) {
+                const int j = 64 * g + 32 * c0 + 8 * h + q;
+                if (j >= D) break;
+                const float zj = z[0][q];
+                if (fn == FN_ELLIPSOID) {
+                    s1 = __fmaf_rn(__fmul_rn(__ldg(w + j), zj), zj, s1);
+                } else {
+                    const float sn = sinpi_reduced_f32(__fsub_rn(zj, rint_f32(zj)));
+                    if (fn == FN_RASTRIGIN) {
+                        s1 = __fadd_rn(s1, __fmaf_rn(zj, zj, __fmul_rn(__fmul_rn(20.f, sn), sn)));
+                    } else {
+                        s1 = __fmaf_rn(zj, zj, s1);
+                        s2 = __fmaf_rn(sn, sn, s2);
+                    }
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 56; ++q) z[q >> 5][q & 31] = z[(q + 8) >> 5][(q + 8) & 31];
+        }
+        if (n == 1) {
+            const float4 o = tc::pair_exchange(make_float4(s1, s2, 0.f, 0.f), c0, xch);
+            if (c0 == 1) return;
+            s1 = __fadd_rn(s1, o.x);
+            s2 = __fadd_rn(s2, o.y);
+        }
+        if (i < N && g < groups) part[(size_t)i * groups + g] = make_float2(s1, s2);
     }
 };
 
-__global__ void __launch_bounds__(128, 1)
-    grad_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, tc::GemmArgs a,
-              StoreEpi epi)
+template <class Epi>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc::P_THREADS, 1)
+    pair_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const tc::GemmArgs a,
+              const __grid_constant__ Epi epi0)
 {
-    tc::gemm_tile(&tmA, &tmB, a, epi);
+    Epi epi = epi0;
+    epi.chains = a.Kp / BK < 3 ? a.Kp / BK : 3;
+    tc::gemm_pair<tc::SplitCfg>(&tmA, &tmB, a, epi);
 }
 
-// A planes of G = grad_f_i df/dz for the rows of Z (warp per row of the padded
-// Np x Kp planes; padding zero): the unrotated function's gradient at z.
-template <int MAXC>
-__global__ void gz_split(const Hot hz, const float* Z, int64_t N, const float* gf, int Np, int Kp,
-                         __nv_bfloat16* A)
+// f from the sums of its terms (a thread per row); NaN if a GEMM wait ran out.
+__global__ void finish_rows(const float2* part, int groups, int fn, int N, int D, const int* status, float* f)
 {
-    const int64_t i = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (i >= Np) return;
-    const int lane = threadIdx.x & 31;
-    const int D = hz.D;
-    float z[MAXC][4], g[MAXC][4];
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= N) return;
+    float s1 = 0.f, s2 = 0.f;
+    for (int t = 0; t < groups; ++t) {
+        const float2 p = part[(size_t)i * groups + t];
+        s1 = __fadd_rn(s1, p.x);
+        s2 = __fadd_rn(s2, p.y);
+    }
+    float v = s1;
+    if (fn == FN_ACKLEY)
+        v = -20.f * expm1f(-0.2f * sqrtf(s1 / (float)D)) - 2.7182818f * expm1f(-2.f * s2 / (float)D);
+    f[i] = *status ? __int_as_float(0x7fffffff) : v;
+}
+
+// Outputs of a backward pass whose GEMM wait ran out: NaN, never stale values.
+__global__ void poison(float* out, size_t n, const int* status)
+{
+    if (!*status) return;
+    for (size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (size_t)gridDim.x * blockDim.x)
+        out[q] = __int_as_float(0x7fffffff);
+}
+
+// A planes of G = grad_f_i df/dz for the rows of Z, a warp per row (the
+// functions' gradients as in grad32; Ackley's row sums first, the row kept in
+// registers).
+template <int FN, int MAXC>
+__global__ void __launch_bounds__(256) gz_rows(const float* __restrict__ Z, const float* __restrict__ w,
+                                               const float* __restrict__ gf, int N, int D, int Np, int Kp,
+                                               __nv_bfloat16* A)
+{
+    const int i = (int)blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (i >= N) return;
+    const int lane = threadIdx.x & 31, nc = Kp / 4;
+    const float* row = Z + (size_t)i * D;
+    const bool vec = (D & 3) == 0;
+    float z[MAXC][4];
 #pragma unroll
-    for (int q = 0; q < MAXC; ++q)
+    for (int q = 0; q < MAXC; ++q) row4(row, lane + 32 * q, D, vec, z[q]);
+    float c_lin = 0.f, c_sin = 0.f;
+    if constexpr (FN == FN_ACKLEY) {
+        float s1 = 0.f, s2 = 0.f;
 #pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            const int j = 4 * (lane + 32 * q) + m;
-            z[q][m] = (i < N && j < D) ? Z[i * D + j] : 0.f;
+        for (int q = 0; q < MAXC; ++q)
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {       // zero beyond D
+                s1 = __fmaf_rn(z[q][m], z[q][m], s1);
+                const float s = sinpi_reduced_f32(__fsub_rn(z[q][m], rint_f32(z[q][m])));
+                s2 = __fmaf_rn(s, s, s2);
+            }
+        for (int off = 16; off > 0; off >>= 1) {
+            s1 += __shfl_xor_sync(0xffffffffu, s1, off);
+            s2 += __shfl_xor_sync(0xffffffffu, s2, off);
         }
-    if (i < N) grad32<MAXC, true>(hz, z, g);
-    const float scale = i < N ? gf[i] : 0.f;
+        const float Av = sqrtf(s1 / (float)D);
+        c_lin = Av > 0.f ? 4.f * expf(-0.2f * Av) / (Av * (float)D) : 0.f;
+        c_sin = 6.28318548f * (2.7182818f * expf(-2.f * s2 / (float)D)) / (float)D;
+    }
+    const float scale = gf[i];
     const size_t plane = (size_t)Np * Kp;
 #pragma unroll
-    for (int q = 0; q < MAXC; ++q)
+    for (int q = 0; q < MAXC; ++q) {
+        const int c = lane + 32 * q;
+        if (c >= nc) break;
+        float g[4];
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
-            const int j = 4 * (lane + 32 * q) + m;
-            if (j >= Kp) continue;
-            const float v = (i < N && j < D) ? __fmul_rn(scale, g[q][m]) : 0.f;
-            __nv_bfloat16 h, mm, l;
-            tc::split3(v, h, mm, l);
-            const size_t o = (size_t)i * Kp + j;
-            A[o] = h;
-            A[plane + o] = mm;
-            A[2 * plane + o] = l;
+            const float zj = z[q][m];
+            float v;
+            if constexpr (FN == FN_ELLIPSOID) v = 4 * c + m < D ? 2.f * __ldg(w + 4 * c + m) * zj : 0.f;
+            else if constexpr (FN == FN_RASTRIGIN) v = __fmaf_rn(62.8318548f, sin2pi_f32(zj), 2.f * zj);
+            else v = __fmaf_rn(c_sin, sin2pi_f32(zj), c_lin * zj);
+            g[m] = __fmul_rn(scale, v);
+            if (4 * c + m >= D) g[m] = 0.f;      // (an infinite scale would make a NaN of 0)
         }
-    // columns beyond this lane layout's reach (Kp may exceed 4 * 32 * MAXC only
-    // when D does not fill the last 64-wide block): zero them
-    for (int j = 128 * MAXC + lane; j < Kp; j += 32) {
-        const size_t o = (size_t)i * Kp + j;
-        A[o] = A[plane + o] = A[2 * plane + o] = __float2bfloat16_rn(0.f);
+        put_planes(g, A, plane, (size_t)i * Kp + 4 * c);
+    }
+}
+
+template <int FN>
+inline void launch_gz(int maxc, const float* Z, const float* w, const float* gf, int N, int D, int Np, int Kp,
+                      __nv_bfloat16* A, cudaStream_t s)
+{
+    const unsigned grid = (unsigned)((N + 7) / 8);
+    switch (maxc) {
+    case 1: gz_rows<FN, 1><<<grid, 256, 0, s>>>(Z, w, gf, N, D, Np, Kp, A); break;
+    case 2: gz_rows<FN, 2><<<grid, 256, 0, s>>>(Z, w, gf, N, D, Np, Kp, A); break;
+    case 4: gz_rows<FN, 4><<<grid, 256, 0, s>>>(Z, w, gf, N, D, Np, Kp, A); break;
+    default: gz_rows<FN, 8><<<grid, 256, 0, s>>>(Z, w, gf, N, D, Np, Kp, A); break;
     }
 }
 
@@ -454,7 +612,7 @@ inline WsLayout ws_layout(int64_t N, int64_t D)
     w.b = take((size_t)3 * w.Jp * w.Kp * 2);
     w.bt = take((size_t)3 * w.Jp * w.Kp * 2);
     w.mn = take((size_t)w.Jp * 4);
-    w.z = take((size_t)N * D * 4);
+    w.z = take((size_t)N * D * 4);     // Z; a forward pass: the row sums (8 bytes per 64 columns)
     w.zero = take((size_t)(D + 4) * 4);
     w.status = take(4);
     w.total = off;
@@ -562,53 +720,78 @@ namespace {
 
 bool uses_tc(psso_fn fn, int64_t D) { return fn >= PSSO_ROT_ELLIPSOID && fn <= PSSO_ROT_ACKLEY && D >= 16; }
 
-psso::Hot base_hot(psso_fn fn, int64_t D, const float* zero, const float* weights)
+int plain_fn(psso_fn fn)
 {
-    psso::Hot h = fb_hot(fn, D, zero, weights, nullptr);
-    h.fn = fn == PSSO_ROT_ELLIPSOID ? PSSO_ELLIPSOID : fn == PSSO_ROT_RASTRIGIN ? PSSO_RASTRIGIN : PSSO_ACKLEY;
-    return h;
+    return fn == PSSO_ROT_ELLIPSOID ? psso::FN_ELLIPSOID : fn == PSSO_ROT_RASTRIGIN ? psso::FN_RASTRIGIN : psso::FN_ACKLEY;
 }
 
-// Operand planes of M (and of M^T for the backward pass), d = x - o, and Z.
-psso_status tc_forward_z(int64_t N, int64_t D, const float* X, const float* shift, const float* rotation,
-                         char* ws, const psso::gtc::WsLayout& L, bool transposed, cudaStream_t s,
-                         CUtensorMap* tb_t)
+// Number of SMs of the current device; sets the GEMM kernels' shared-memory
+// limit on the first call a thread makes on a device (the attribute is per device).
+int device_sms()
 {
     using namespace psso;
-    auto* A = reinterpret_cast<__nv_bfloat16*>(ws + L.a);
-    auto* B = reinterpret_cast<__nv_bfloat16*>(ws + L.b);
-    auto* Bt = reinterpret_cast<__nv_bfloat16*>(ws + L.bt);
-    CUtensorMap ta, tb;
-    if (!tc::make_tmap_bf16(&ta, A, L.Kp, 3 * L.Np) || !tc::make_tmap_bf16(&tb, B, L.Kp, 3 * L.Jp) ||
-        (transposed && !tc::make_tmap_bf16(tb_t, Bt, L.Kp, 3 * L.Jp))) {
+    static thread_local int dev_of = -1, sms = 0;
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    if (dev != dev_of) {
+        const int smem = tc::pair_smem<tc::SplitCfg::PLANES, tc::SplitCfg::STG>();
+        int n = 0;
+        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+            cudaFuncSetAttribute(gtc::pair_gemm<tc::StoreEpi>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
+                cudaSuccess ||
+            cudaFuncSetAttribute(gtc::pair_gemm<gtc::SumEpi>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
+                cudaSuccess)
+            return 0;
+        sms = n;
+        dev_of = dev;
+    }
+    return sms;
+}
+
+template <class Epi>
+void launch_gemm(const CUtensorMap& ta, const CUtensorMap& tb, const psso::gtc::WsLayout& L, int* status, Epi epi,
+                 int64_t N, int64_t D, int sms, cudaStream_t s)
+{
+    using namespace psso;
+    epi.N = (int)N;
+    epi.D = (int)D;
+    const tc::GemmArgs ga{L.Np, L.Jp, L.Kp, status};
+    gtc::pair_gemm<Epi><<<tc::pair_grid(L.Np, L.Jp, sms), tc::P_THREADS,
+                          tc::pair_smem<tc::SplitCfg::PLANES, tc::SplitCfg::STG>(), s>>>(ta, tb, ga, epi);
+}
+
+// Operand planes of d = x - o and M (and M^T), and the tensor maps of A and M.
+psso_status tc_prepare(int64_t N, int64_t D, const float* X, const float* shift, const float* rotation, char* ws,
+                       const psso::gtc::WsLayout& L, bool transposed, cudaStream_t s, CUtensorMap* ta, CUtensorMap* tb,
+                       CUtensorMap* tbt)
+{
+    using namespace psso;
+    gtc::PrepArgs a{};
+    a.X = X;
+    a.o = shift;
+    a.M = rotation;
+    a.A = reinterpret_cast<__nv_bfloat16*>(ws + L.a);
+    a.B = reinterpret_cast<__nv_bfloat16*>(ws + L.b);
+    a.Bt = transposed ? reinterpret_cast<__nv_bfloat16*>(ws + L.bt) : nullptr;
+    a.status = reinterpret_cast<int*>(ws + L.status);
+    a.N = (int)N;
+    a.D = (int)D;
+    a.Np = L.Np;
+    a.Jp = L.Jp;
+    a.Kp = L.Kp;
+    a.vec_x = D % 4 == 0 && tc::aligned(X, 16);
+    a.vec_m = D % 4 == 0 && tc::aligned(rotation, 16);
+    const int64_t rb = (N + D + 7) / 8;
+    const int64_t tiles = transposed ? (int64_t)((D + 31) / 32) * (L.Kp / 32) : 0;
+    a.row_blocks = (int)rb;
+    if (!tc::make_tmap_bf16(ta, a.A, L.Kp, 3 * L.Np) || !tc::make_tmap_bf16(tb, a.B, L.Kp, 3 * L.Jp, 64) ||
+        (transposed && !tc::make_tmap_bf16(tbt, a.Bt, L.Kp, 3 * L.Jp, 64))) {
         set_last_error("psso_fitness_*_ws: cuTensorMapEncodeTiled failed");
         return PSSO_ERR_CUDA;
     }
-    float* Z = reinterpret_cast<float*>(ws + L.z);
-    int* status = reinterpret_cast<int*>(ws + L.status);
-    if (cudaMemsetAsync(ws + L.zero, 0, (size_t)(D + 4) * 4, s) != cudaSuccess ||
-        cudaMemsetAsync(status, 0, 4, s) != cudaSuccess ||
-        // a GEMM whose wait runs out writes nothing: its outputs then read NaN
-        cudaMemsetAsync(Z, 0xff, (size_t)N * D * 4, s) != cudaSuccess ||
-        tc::launch_split_matrix(rotation, (int)D, L.Jp, L.Kp, B, reinterpret_cast<float*>(ws + L.mn), s) !=
-            cudaSuccess ||
-        tc::launch_split_rows(X, shift, (int)N, (int)D, L.Np, L.Kp, A, s) != cudaSuccess) {
-        set_last_error("psso_fitness_*_ws: operand preparation failed");
-        return PSSO_ERR_CUDA;
-    }
-    if (transposed) gtc::split_matrix_t<<<L.Jp, 256, 0, s>>>(rotation, (int)D, L.Jp, L.Kp, Bt);
-    static thread_local int smem_set_for = -1;   // the attribute is per device
-    int dev = -1;
-    cudaGetDevice(&dev);
-    if (smem_set_for != dev) {
-        cudaFuncSetAttribute(gtc::grad_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_BYTES);
-        smem_set_for = dev;
-    }
-    tc::GemmArgs ga{L.Np, L.Jp, L.Kp, status};
-    gtc::grad_gemm<<<dim3(L.Np / psso::tc::BM, L.Jp / psso::tc::BN), 128, tc::SMEM_BYTES, s>>>(ta, tb, ga,
-                                                                           gtc::StoreEpi{Z, (int)N, (int)D});
+    gtc::prep_planes<<<(unsigned)(rb + tiles), 256, 0, s>>>(a);
     if (cudaGetLastError() != cudaSuccess) {
-        set_last_error("psso_fitness_*_ws: GEMM launch failed");
+        set_last_error("psso_fitness_*_ws: operand preparation failed");
         return PSSO_ERR_CUDA;
     }
     return PSSO_OK;
@@ -643,12 +826,22 @@ extern "C" psso_status psso_fitness_forward_ws(psso_fn fn, int64_t N, int64_t D,
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     char* ws = static_cast<char*>(workspace);
-    st = tc_forward_z(N, D, X, shift, rotation, ws, L, false, s, nullptr);
+    const int sms = device_sms();
+    CUtensorMap ta, tb;
+    st = tc_prepare(N, D, X, shift, rotation, ws, L, false, s, &ta, &tb, nullptr);
     if (st != PSSO_OK) return st;
-    const Hot hz = base_hot(fn, D, reinterpret_cast<const float*>(ws + L.zero), weights);
-    const int wpb = 8;
-    fitness_fb<false><<<(unsigned)((N + wpb - 1) / wpb), 32 * wpb, 0, s>>>(
-        hz, reinterpret_cast<const float*>(ws + L.z), N, nullptr, f, nullptr);
+    if (sms < 2) {
+        set_last_error("psso_fitness_forward_ws: cannot configure the GEMM kernel");
+        return PSSO_ERR_CUDA;
+    }
+    int* status = reinterpret_cast<int*>(ws + L.status);
+    gtc::SumEpi epi{};
+    epi.part = reinterpret_cast<float2*>(ws + L.z);
+    epi.w = weights;
+    epi.fn = plain_fn(fn);
+    epi.groups = (int)((D + 63) / 64);
+    launch_gemm(ta, tb, L, status, epi, N, D, sms, s);
+    gtc::finish_rows<<<(unsigned)((N + 127) / 128), 128, 0, s>>>(epi.part, epi.groups, epi.fn, (int)N, (int)D, status, f);
     if (cudaGetLastError() != cudaSuccess) {
         set_last_error("psso_fitness_forward_ws: launch failed");
         return PSSO_ERR_CUDA;
@@ -674,32 +867,32 @@ extern "C" psso_status psso_fitness_backward_ws(psso_fn fn, int64_t N, int64_t D
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     char* ws = static_cast<char*>(workspace);
-    CUtensorMap tbt;
-    st = tc_forward_z(N, D, X, shift, rotation, ws, L, true, s, &tbt);
+    const int sms = device_sms();
+    CUtensorMap ta, tb, tbt;
+    st = tc_prepare(N, D, X, shift, rotation, ws, L, true, s, &ta, &tb, &tbt);
     if (st != PSSO_OK) return st;
-    const Hot hz = base_hot(fn, D, reinterpret_cast<const float*>(ws + L.zero), weights);
+    if (sms < 2) {
+        set_last_error("psso_fitness_backward_ws: cannot configure the GEMM kernel");
+        return PSSO_ERR_CUDA;
+    }
+    int* status = reinterpret_cast<int*>(ws + L.status);
+    float* Z = reinterpret_cast<float*>(ws + L.z);
+    tc::StoreEpi epi{};
+    epi.out = Z;
+    epi.vec = tc::store_width(Z, D);
+    launch_gemm(ta, tb, L, status, epi, N, D, sms, s);
     auto* A = reinterpret_cast<__nv_bfloat16*>(ws + L.a);   // reused: the planes of G
-    const int wpb = 8;
-    const unsigned grid = (unsigned)((L.Np + wpb - 1) / wpb);
-    const float* Z = reinterpret_cast<const float*>(ws + L.z);
-    switch (hz.maxc) {
-    case 1: gtc::gz_split<1><<<grid, 32 * wpb, 0, s>>>(hz, Z, N, grad_f, L.Np, L.Kp, A); break;
-    case 2: gtc::gz_split<2><<<grid, 32 * wpb, 0, s>>>(hz, Z, N, grad_f, L.Np, L.Kp, A); break;
-    case 4: gtc::gz_split<4><<<grid, 32 * wpb, 0, s>>>(hz, Z, N, grad_f, L.Np, L.Kp, A); break;
-    default: gtc::gz_split<8><<<grid, 32 * wpb, 0, s>>>(hz, Z, N, grad_f, L.Np, L.Kp, A); break;
+    int maxc = 1;                                            // chunks of 4 columns per lane, padding included
+    while (128 * maxc < L.Kp) maxc <<= 1;
+    switch (plain_fn(fn)) {
+    case FN_ELLIPSOID: gtc::launch_gz<FN_ELLIPSOID>(maxc, Z, weights, grad_f, (int)N, (int)D, L.Np, L.Kp, A, s); break;
+    case FN_RASTRIGIN: gtc::launch_gz<FN_RASTRIGIN>(maxc, Z, weights, grad_f, (int)N, (int)D, L.Np, L.Kp, A, s); break;
+    default: gtc::launch_gz<FN_ACKLEY>(maxc, Z, weights, grad_f, (int)N, (int)D, L.Np, L.Kp, A, s); break;
     }
-    CUtensorMap ta;
-    if (!tc::make_tmap_bf16(&ta, A, L.Kp, 3 * L.Np)) {
-        set_last_error("psso_fitness_backward_ws: cuTensorMapEncodeTiled failed");
-        return PSSO_ERR_CUDA;
-    }
-    if (cudaMemsetAsync(grad_X, 0xff, (size_t)N * D * 4, s) != cudaSuccess) {
-        set_last_error("psso_fitness_backward_ws: memset failed");
-        return PSSO_ERR_CUDA;
-    }
-    tc::GemmArgs ga{L.Np, L.Jp, L.Kp, reinterpret_cast<int*>(ws + L.status)};
-    gtc::grad_gemm<<<dim3(L.Np / psso::tc::BM, L.Jp / psso::tc::BN), 128, tc::SMEM_BYTES, s>>>(ta, tbt, ga,
-                                                                           gtc::StoreEpi{grad_X, (int)N, (int)D});
+    epi.out = grad_X;
+    epi.vec = tc::store_width(grad_X, D);
+    launch_gemm(ta, tbt, L, status, epi, N, D, sms, s);
+    gtc::poison<<<(unsigned)sms, 256, 0, s>>>(grad_X, (size_t)N * D, status);
     if (cudaGetLastError() != cudaSuccess) {
         set_last_error("psso_fitness_backward_ws: launch failed");
         return PSSO_ERR_CUDA;

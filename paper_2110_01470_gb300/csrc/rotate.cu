@@ -10,7 +10,7 @@
 #include "psso_internal.h"
 #include "sso_common.cuh"
 #include "rot_pipeline.h"
-#include "tc_gemm.cuh"
+#include "tc_pair.cuh"
 
 namespace psso {
 namespace tc {
@@ -85,39 +85,13 @@ __global__ void split_rows(const float* __restrict__ X, const float* __restrict_
     }
 }
 
-cudaError_t launch_split_matrix(const float* M32, int D, int Jp, int Kp, __nv_bfloat16* B, float* mnorm,
-                                cudaStream_t s)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_THREADS, 1)
+    rotate_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const GemmArgs a,
+                const __grid_constant__ StoreEpi epi0)
 {
-    split_matrix<<<Jp, 256, 0, s>>>(M32, D, Jp, Kp, B, mnorm);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_split_rows(const float* X, const float* o, int N, int D, int Np, int Kp, __nv_bfloat16* A,
-                              cudaStream_t s)
-{
-    split_rows<<<(Np + 7) / 8, 256, 0, s>>>(X, o, N, D, Np, Kp, A);
-    return cudaGetLastError();
-}
-
-struct ZEpi {
-    float* Z;
-    int N, D;
-    __device__ void operator()(int c, const float (&z)[32]) const
-    {
-        const int i = blockIdx.x * BM + threadIdx.x;
-        const int j0 = blockIdx.y * BN + 32 * c;
-        if (i >= N) return;
-#pragma unroll
-        for (int t = 0; t < 32; ++t)
-            if (j0 + t < D) Z[(size_t)i * D + j0 + t] = z[t];
-    }
-};
-
-__global__ void __launch_bounds__(128, 1)
-    rotate_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, GemmArgs a,
-                ZEpi epi)
-{
-    gemm_tile(&tmA, &tmB, a, epi);
+    StoreEpi epi = epi0;
+    epi.chains = a.Kp / BK < 3 ? a.Kp / BK : 3;
+    gemm_pair<SplitCfg>(&tmA, &tmB, a, epi);
 }
 
 }  // namespace tc
@@ -151,7 +125,7 @@ extern "C" psso_status psso_rotate(int64_t N, int64_t D, const float* X, const f
         return PSSO_ERR_OOM;
     }
     CUtensorMap ta, tb;
-    if (!make_tmap_bf16(&ta, A, Kp, 3 * Np) || !make_tmap_bf16(&tb, B, Kp, 3 * Jp)) {
+    if (!make_tmap_bf16(&ta, A, Kp, 3 * Np) || !make_tmap_bf16(&tb, B, Kp, 3 * Jp, 64)) {
         cleanup();
         set_last_error("psso_rotate: cuTensorMapEncodeTiled failed");
         return PSSO_ERR_CUDA;
@@ -159,9 +133,18 @@ extern "C" psso_status psso_rotate(int64_t N, int64_t D, const float* X, const f
     cudaMemsetAsync(status, 0, 4, s);
     split_matrix<<<Jp, 256, 0, s>>>(rotation, (int)D, Jp, Kp, B, mn);
     split_rows<<<(Np + 7) / 8, 256, 0, s>>>(X, shift, (int)N, (int)D, Np, Kp, A);
-    cudaFuncSetAttribute(rotate_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+    constexpr int smem = pair_smem<SplitCfg::PLANES, SplitCfg::STG>();
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaFuncSetAttribute(rotate_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     GemmArgs ga{Np, Jp, Kp, status};
-    rotate_gemm<<<dim3(Np / BM, Jp / BN), 128, SMEM_BYTES, s>>>(ta, tb, ga, ZEpi{Z, (int)N, (int)D});
+    StoreEpi epi{};
+    epi.N = (int)N;
+    epi.D = (int)D;
+    epi.out = Z;
+    epi.vec = store_width(Z, D);
+    if (sms >= 2) rotate_gemm<<<pair_grid(Np, Jp, sms), P_THREADS, smem, s>>>(ta, tb, ga, epi);
     cudaError_t e = cudaGetLastError();
     int st = 0;
     if (e == cudaSuccess) e = cudaMemcpyAsync(&st, status, 4, cudaMemcpyDeviceToHost, s);

@@ -224,132 +224,6 @@ struct GemmArgs {
     int* status;      // set to 1 when a wait ran out (device memory)
 };
 
-// The GEMM main loop for the tile (blockIdx.x, blockIdx.y); the epilogue
-// functor gets (row in tile = threadIdx.x, column block c of 32, z[32]).
-// Returns false (all threads) if a wait ran out.
-template <class Epi>
-__device__ __forceinline__ bool gemm_tile(const CUtensorMap* tmA, const CUtensorMap* tmB,
-                                          const GemmArgs& a, Epi& epi)
-{
-    extern __shared__ __align__(1024) unsigned char tc_smem_raw[];
-    __shared__ __align__(8) uint64_t bars[2 * STAGES + 1];
-    __shared__ uint32_t tmem_slot;
-    __shared__ int failed;
-    unsigned char* smem = reinterpret_cast<unsigned char*>(
-        (reinterpret_cast<uintptr_t>(tc_smem_raw) + 1023) & ~(uintptr_t)1023);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
-    const int nkb = a.Kp / BK;
-    const uint32_t sbase = smem_u32(smem);
-    auto full = [&](int s) { return smem_u32(&bars[s]); };
-    auto empty = [&](int s) { return smem_u32(&bars[STAGES + s]); };
-    const uint32_t done = smem_u32(&bars[2 * STAGES]);
-
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) {
-            mbar_init(full(s), 1);
-            mbar_init(empty(s), 1);
-        }
-        mbar_init(done, 1);
-        fence_mbar_init();
-        failed = 0;
-    }
-    if (warp == 0) {
-        tmem_alloc(smem_u32(&tmem_slot), TMEM_COLS);
-        tmem_relinquish();
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = tmem_slot;
-
-    if (warp == 0 && lane == 0) {
-        // TMA producer
-        for (int kb = 0; kb < nkb; ++kb) {
-            const int s = kb % STAGES;
-            if (kb >= STAGES && !mbar_wait(empty(s), (uint32_t)((kb / STAGES - 1) & 1))) {
-                failed = 1;
-                break;
-            }
-            mbar_expect_tx(full(s), STAGE_BYTES);
-            const uint32_t st = sbase + (uint32_t)(s * STAGE_BYTES);
-            for (int p = 0; p < 3; ++p) {
-                tma_load_2d(st + (uint32_t)(p * TILE_BYTES), tmA, kb * BK, p * a.Np + m0, full(s));
-                tma_load_2d(st + (uint32_t)((3 + p) * TILE_BYTES), tmB, kb * BK, p * a.Jp + n0, full(s));
-            }
-        }
-    } else if (warp == 1 && lane == 0) {
-        // MMA issuer
-        constexpr uint32_t idesc = idesc_bf16(BM, BN);
-        const uint32_t acc1 = tmem + NCHAIN * BN;
-        bool ok = true;
-        for (int kb = 0; kb < nkb && ok; ++kb) {
-            const int s = kb % STAGES;
-            if (!mbar_wait(full(s), (uint32_t)((kb / STAGES) & 1))) {
-                failed = 1;
-                ok = false;
-                break;
-            }
-            tc_fence_after();
-            const uint32_t st = sbase + (uint32_t)(s * STAGE_BYTES);
-            const uint32_t acc0 = tmem + (uint32_t)((kb % NCHAIN) * BN);
-#pragma unroll
-            for (int ks = 0; ks < BK / 16; ++ks) {
-                const uint32_t off = (uint32_t)(ks * 32);   // 16 bf16 along K
-                const uint64_t ah = sdesc_sw128(st + 0 * TILE_BYTES + off);
-                const uint64_t am = sdesc_sw128(st + 1 * TILE_BYTES + off);
-                const uint64_t al = sdesc_sw128(st + 2 * TILE_BYTES + off);
-                const uint64_t bh = sdesc_sw128(st + 3 * TILE_BYTES + off);
-                const uint64_t bm = sdesc_sw128(st + 4 * TILE_BYTES + off);
-                const uint64_t bl = sdesc_sw128(st + 5 * TILE_BYTES + off);
-                const uint32_t first0 = (kb < NCHAIN && ks == 0) ? 0u : 1u;   // chain's first MMA
-                const uint32_t first1 = (kb | ks) ? 1u : 0u;
-                mma_bf16(acc0, ah, bh, idesc, first0);
-                mma_bf16(acc1, ah, bm, idesc, first1);
-                mma_bf16(acc1, am, bh, idesc, 1u);
-                mma_bf16(acc1, ah, bl, idesc, 1u);
-                mma_bf16(acc1, al, bh, idesc, 1u);
-                mma_bf16(acc1, am, bm, idesc, 1u);
-            }
-            mma_commit(empty(s));      // the stage is free once these MMAs are done
-        }
-        mma_commit(done);              // all MMAs issued (possibly none if a wait failed)
-    }
-    __syncwarp();
-
-    bool ok = mbar_wait(done, 0u);
-    if (!ok) failed = 1;
-    tc_fence_after();
-    __syncthreads();
-    const bool good = !failed;
-    if (good) {
-        const uint32_t lane_base = (uint32_t)(32 * warp) << 16;
-        const int chains = nkb < NCHAIN ? nkb : NCHAIN;   // chains that received products
-#pragma unroll 1
-        for (int c = 0; c < BN / 32; ++c) {
-            float z0[32], z1[32];
-            tmem_ld32(tmem + lane_base + (uint32_t)(32 * c), z0);
-            for (int ch = 1; ch < chains; ++ch) {
-                tmem_ld32(tmem + lane_base + (uint32_t)(ch * BN + 32 * c), z1);
-#pragma unroll
-                for (int t = 0; t < 32; ++t) z0[t] = __fadd_rn(z0[t], z1[t]);
-            }
-            tmem_ld32(tmem + lane_base + (uint32_t)(NCHAIN * BN + 32 * c), z1);
-#pragma unroll
-            for (int t = 0; t < 32; ++t) z0[t] = __fadd_rn(z0[t], z1[t]);
-            epi(c, z0);
-        }
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 0) {
-        tc_fence_after();
-        tmem_dealloc(tmem, TMEM_COLS);
-    }
-    if (!good && threadIdx.x == 0 && a.status) atomicExch(a.status, 1);
-    return good;
-}
-
 // Host: tensor map of a [rows][Kp] bf16 matrix, boxes of 64 x box_rows,
 // 128-byte swizzle.
 bool make_tmap_bf16(CUtensorMap* map, const void* base, int Kp, int rows, int box_rows = BM);

@@ -317,6 +317,99 @@ __device__ __forceinline__ bool gemm_pair(const CUtensorMap* tmA, const CUtensor
     return good;
 }
 
+// The six split products: the main part in three accumulators (K blocks dealt
+// round robin), the corrections in a fourth.
+struct SplitCfg {
+    static constexpr int PLANES = 3, STG = 3, PRODUCTS = 6;
+    __device__ static constexpr int pa(int q) { constexpr int T[6] = {0, 0, 1, 0, 2, 1}; return T[q]; }
+    __device__ static constexpr int pb(int q) { constexpr int T[6] = {0, 1, 0, 2, 0, 1}; return T[q]; }
+    __device__ static constexpr int acc(int q, int kb) { return q == 0 ? kb % 3 : 3; }
+    __device__ static constexpr bool first(int q, int kb, int ks)
+    {
+        return ks == 0 && (q == 0 ? kb < 3 : q == 1 && kb == 0);
+    }
+};
+
+// 64 joined columns of one row: z = ((main 0 + main 1) + main 2) + corrections.
+struct JoinEpi {
+    int N, D, chains;             // chains: main accumulators that received products
+    int i, g;                     // row, 64-column group
+    float z[2][32];
+    __device__ __forceinline__ void tile(int tm, int g_, int row)
+    {
+        i = tm * PBM + row;
+        g = g_;
+    }
+    __device__ __forceinline__ void load(uint32_t taddr, int n)
+    {
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            if (c >= n) break;
+            float v[32];
+            tmem_ld32(taddr + (uint32_t)(32 * c), z[c]);
+            if (chains > 1) {
+                tmem_ld32(taddr + (uint32_t)(128 + 32 * c), v);
+#pragma unroll
+                for (int q = 0; q < 32; ++q) z[c][q] = __fadd_rn(z[c][q], v[q]);
+            }
+            if (chains > 2) {
+                tmem_ld32(taddr + (uint32_t)(256 + 32 * c), v);
+#pragma unroll
+                for (int q = 0; q < 32; ++q) z[c][q] = __fadd_rn(z[c][q], v[q]);
+            }
+            tmem_ld32(taddr + (uint32_t)(384 + 32 * c), v);
+#pragma unroll
+            for (int q = 0; q < 32; ++q) z[c][q] = __fadd_rn(z[c][q], v[q]);
+        }
+    }
+};
+
+// C -> out[i * D + j] (rows < N, columns < D).  vec: 8 (32-byte stores, the
+// row pitch and base are multiples of 32 bytes), 4 (16-byte) or 1.
+struct StoreEpi : JoinEpi {
+    float* out;
+    int vec;
+    __device__ __forceinline__ void compute(int c0, int nb, float4*)
+    {
+        if (i >= N) return;
+        float* row = out + (size_t)i * D + 64 * g + 32 * c0;
+        const int n = D - 64 * g - 32 * c0;   // columns left in the row
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+#pragma unroll
+            for (int q = 0; q < 32; q += 8) {
+                if (c >= nb) break;
+                const int j = 32 * c + q;
+                if (vec == 8 && j + 8 <= n) {
+                    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(row + j),
+                                 "f"(z[c][q]), "f"(z[c][q + 1]), "f"(z[c][q + 2]), "f"(z[c][q + 3]), "f"(z[c][q + 4]),
+                                 "f"(z[c][q + 5]), "f"(z[c][q + 6]), "f"(z[c][q + 7])
+                                 : "memory");
+                } else {
+#pragma unroll
+                    for (int h = 0; h < 8; h += 4) {
+                        if (vec >= 4 && j + h + 4 <= n) {
+                            *reinterpret_cast<float4*>(row + j + h) =
+                                make_float4(z[c][q + h], z[c][q + h + 1], z[c][q + h + 2], z[c][q + h + 3]);
+                        } else {
+#pragma unroll
+                            for (int m = 0; m < 4; ++m)
+                                if (j + h + m < n) row[j + h + m] = z[c][q + h + m];
+                        }
+                    }
+                }
+            }
+    }
+};
+
+inline bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; }
+
+// StoreEpi's store width for rows of D floats at out.
+inline int store_width(const float* out, int64_t D)
+{
+    return D % 8 == 0 && aligned(out, 32) ? 8 : D % 4 == 0 && aligned(out, 16) ? 4 : 1;
+}
+
 // CTAs of a pair GEMM's grid: one pair per two SMs, no more than work items.
 inline int pair_grid(int Np, int Jp, int sms)
 {
