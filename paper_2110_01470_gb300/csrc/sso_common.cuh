@@ -90,13 +90,19 @@ __device__ __forceinline__ bool same_bits(double a, double b)
 }
 
 // Order-preserving integer key of a double (sign-magnitude to two's complement,
-// so -0 and +0 are equal; a positive NaN is above everything).  Comparing two
-// keys is integer work, where comparing two doubles takes the FP64 unit: 64
-// clocks each, 19 clocks of the whole SM's unit.
+// so -0 and +0 are equal; a NaN is above everything).  Comparing two keys is
+// integer work, where comparing two doubles takes the FP64 unit: 64 clocks
+// each, 19 clocks of the whole SM's unit.
 __device__ __forceinline__ long long order_key(double v)
 {
-    const long long b = __double_as_longlong(v);
-    return b < 0 ? -(b & 0x7fffffffffffffffLL) : b;
+    const long long b = __double_as_longlong(v), mag = b & 0x7fffffffffffffffLL;
+    return mag > 0x7ff0000000000000LL ? 0x7fffffffffffffffLL : b < 0 ? -mag : mag;
+}
+// a <= b of doubles (false with a NaN), and a < b with a NaN above everything.
+__device__ __forceinline__ bool le_f64(double a, double b)
+{
+    const long long kb = order_key(b);
+    return order_key(a) <= kb && kb != 0x7fffffffffffffffLL;
 }
 
 // The per-particle fields of an instance descriptor, as a small value type
@@ -146,14 +152,20 @@ __device__ __forceinline__ float fresh_f32(uint32_t w, const Hot& in)
     x = (x > in.ubf) ? in.ubf : x;
     return x;
 }
+// The 53-bit uniform u = m 2^-53 without a conversion: the low 52 bits of m as
+// the mantissa of a double in [1/2, 1) are 1/2 + (m mod 2^52) 2^-53, which is u
+// when m's top bit is set and u + 1/2 (exactly) when it is not.  With lb <= x
+// by the rounding's monotony and the upper clamp on integer keys, a value takes
+// two FP64 instructions (31 ns each) instead of five.
 __device__ __forceinline__ double fresh_f64(uint32_t lo, uint32_t hi, const Hot& in)
 {
-    const uint64_t m = ((((uint64_t)hi) << 32) | lo) >> 11;
-    const double u = __dmul_rn(__ull2double_rn(m), 0x1p-53);
-    double x = __fma_rn(in.span, u, in.lb);
-    x = (x < in.lb) ? in.lb : x;
-    x = (x > in.ub) ? in.ub : x;
-    return x;
+    const uint32_t mh = hi >> 11, ml = __funnelshift_r(lo, hi, 11);       // m's high 21 and low 32 bits
+    const double half = __hiloint2double((int)(0x3fe00000u | (mh & 0xfffffu)), (int)ml);
+    const double u = __dadd_rn(half, (mh & 0x100000u) ? 0.0 : -0.5);
+    const double x = __fma_rn(in.span, u, in.lb);
+    // x > ub (a NaN, possible when ub - lb overflows, is kept)
+    const long long kx = order_key(x), ku = order_key(in.ub);
+    return (kx > ku && kx <= 0x7ff0000000000000LL) ? in.ub : x;
 }
 
 // Fresh values for the chunk's variables selected by `mask` (bit m = variable 4c+m).
