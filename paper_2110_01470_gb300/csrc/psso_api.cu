@@ -130,7 +130,7 @@ struct psso_ctx {
     size_t smem = 0;
     char* arena = nullptr;
     size_t arena_size = 0, state_off = 0;
-    size_t off_instdev = 0, off_units = 0, off_block_first = 0, off_status = 0;
+    size_t off_instdev = 0, off_units = 0, off_block_first = 0, off_status = 0, off_best = 0;
     int64_t gen = 0;
     int64_t evals = 0, updates = 0;
     int64_t h2d = 0, d2h = 0;
@@ -841,12 +841,9 @@ psso_status setup_async(psso_ctx* h)
     return PSSO_OK;
 }
 
-psso_status read_status(psso_ctx* h)
+// The device-side status words as read by the host.
+psso_status check_status(psso_ctx* h, const StatusDev& st)
 {
-    CUDA_TRY(cudaSetDevice(h->device));
-    CUDA_TRY(cudaStreamSynchronize(h->stream));
-    StatusDev st;
-    CUDA_TRY(cudaMemcpy(&st, h->arena + h->off_status, sizeof st, cudaMemcpyDeviceToHost));
     for (size_t k = 0; k < h->inst.size(); ++k) {
         if (!h->inst[k].tc) continue;
         int tst = 0;
@@ -863,6 +860,15 @@ psso_status read_status(psso_ctx* h)
                                              std::to_string(st.where & 0xffff) + ")");
     }
     return PSSO_OK;
+}
+
+psso_status read_status(psso_ctx* h)
+{
+    CUDA_TRY(cudaSetDevice(h->device));
+    CUDA_TRY(cudaStreamSynchronize(h->stream));
+    StatusDev st;
+    CUDA_TRY(cudaMemcpy(&st, h->arena + h->off_status, sizeof st, cudaMemcpyDeviceToHost));
+    return check_status(h, st);
 }
 
 }  // namespace
@@ -1003,10 +1009,13 @@ psso_status create_impl(const psso_problem* problems, int32_t count, const psso_
         off += bytes;
         return at;
     };
+    int max_dp = 0;
+    for (const auto& I : h->inst) max_dp = std::max(max_dp, I.Dp);
     h->off_instdev = take(sizeof(InstDev) * h->inst.size());
     h->off_units = take(sizeof(UnitDev) * h->units.size());
     h->off_block_first = take(sizeof(int32_t) * h->block_first.size());
     h->off_status = take(sizeof(StatusDev));
+    h->off_best = take(sizeof(BestPack) + (size_t)max_dp * h->pos_size);
     h->state_off = align_up(off, 256);
     const bool f32r = h->precision == PSSO_PREC_F32_RECHECK;
     const size_t logcap = c.log_stride > 0 ? (size_t)c.log_capacity : 0;
@@ -1171,13 +1180,10 @@ psso_status psso_reset(psso_handle h)
     if (!h) return fail(PSSO_ERR_ARG, "handle is NULL");
     CUDA_TRY(cudaSetDevice(h->device));
     const size_t logcap = h->cfg.log_stride > 0 ? (size_t)h->cfg.log_capacity : 0;
-    for (const auto& I : h->inst) {
-        const size_t rb = SLOTS * (size_t)I.R * REC_WORDS * 8;
-        CUDA_TRY(cudaMemsetAsync(h->arena + I.off_rec, 0xff, rb, h->stream));
-        CUDA_TRY(cudaMemsetAsync(h->arena + I.off_rec2, 0xff, rb, h->stream));
+    CUDA_TRY(launch_reset(reinterpret_cast<const InstDev*>(h->arena + h->off_instdev), (int)h->inst.size(), h->stream));
+    ++h->launches;
+    for (const auto& I : h->inst)
         if (logcap) CUDA_TRY(cudaMemsetAsync(h->arena + I.off_log, 0xff, logcap * sizeof(LogDev), h->stream));
-        CUDA_TRY(cudaMemsetAsync(h->arena + I.off_gb, 0, sizeof(GBestDev), h->stream));
-    }
     CUDA_TRY(cudaMemsetAsync(h->arena + h->off_status, 0, sizeof(StatusDev), h->stream));
     for (auto& I : h->inst)
         if (I.tc) CUDA_TRY(cudaMemsetAsync(&I.rh.dev.ctl->status, 0, sizeof(int), h->stream));
@@ -1220,20 +1226,27 @@ psso_status psso_best(psso_handle h, int32_t instance, double* value, int64_t* i
     const Range range("psso_best");
     if (!h) return fail(PSSO_ERR_ARG, "handle is NULL");
     if (instance < 0 || instance >= (int32_t)h->inst.size()) return fail(PSSO_ERR_ARG, "instance out of range");
-    psso_status st = read_status(h);
-    if (st != PSSO_OK) return st;
-    if (h->precision == PSSO_PREC_F32_RECHECK) {
-        CUDA_TRY(launch_best_f64(reinterpret_cast<const InstDev*>(h->arena + h->off_instdev),
-                                 (int)h->inst.size(), h->lattice, h->stream));
-        CUDA_TRY(cudaStreamSynchronize(h->stream));
-    }
+    CUDA_TRY(cudaSetDevice(h->device));
     const HostInst& I = h->inst[instance];
-    GBestDev gb;
-    CUDA_TRY(cudaMemcpy(&gb, h->arena + I.off_gb, sizeof gb, cudaMemcpyDeviceToHost));
-    h->d2h += (int64_t)sizeof gb;
-    if (value) *value = gb.f64;
-    if (index) *index = gb.idx;
-    if (row) return copy_row(h, I, I.off_gbrow, 1, row);
+    alignas(16) char buf[sizeof(BestPack) + 32 * MAX_CHUNKS_PER_LANE * 4 * sizeof(double)];
+    const size_t n = sizeof(BestPack) + (row ? (size_t)I.Dp * h->pos_size : 0);
+    CUDA_TRY(launch_best(reinterpret_cast<const InstDev*>(h->arena + h->off_instdev), instance, h->lattice,
+                         reinterpret_cast<const StatusDev*>(h->arena + h->off_status),
+                         reinterpret_cast<BestPack*>(h->arena + h->off_best), h->stream));
+    CUDA_TRY(cudaMemcpyAsync(buf, h->arena + h->off_best, n, cudaMemcpyDeviceToHost, h->stream));
+    CUDA_TRY(cudaStreamSynchronize(h->stream));
+    BestPack pk;
+    std::memcpy(&pk, buf, sizeof pk);
+    const psso_status st = check_status(h, pk.status);
+    if (st != PSSO_OK) return st;
+    h->d2h += (int64_t)n;
+    if (value) *value = pk.gb.f64;
+    if (index) *index = pk.gb.idx;
+    if (row) {
+        const char* r = buf + sizeof pk;
+        for (int64_t j = 0; j < I.pr.D; ++j)
+            row[j] = h->pos_size == 8 ? reinterpret_cast<const double*>(r)[j] : (double)reinterpret_cast<const float*>(r)[j];
+    }
     return PSSO_OK;
 }
 

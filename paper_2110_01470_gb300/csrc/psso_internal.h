@@ -157,7 +157,16 @@ struct KParams {
 // limit, 3 = maximum threads per block into *out.
 cudaError_t gen_call(int variant, int op, int mc_index, const KParams* p, int grid, int block,
                      size_t smem, cudaStream_t s, int* out);
-cudaError_t launch_best_f64(const InstDev* inst, int n_inst, int lattice, cudaStream_t s);
+// What psso_best reads, packed for one copy: followed by the gBest row.
+struct BestPack {
+    GBestDev gb;
+    StatusDev status;
+};
+// Instance k's gBest (its FP64 value computed if only bounds are known), the
+// launch status and the row into out.
+cudaError_t launch_best(const InstDev* inst, int k, int lattice, const StatusDev* status, BestPack* out, cudaStream_t s);
+// Empties every instance's exchange records and clears its gBest record.
+cudaError_t launch_reset(const InstDev* inst, int n_inst, cudaStream_t s);
 
 // Batched throughput pipeline: one generation of many independent swarms as
 // one kernel per class of equal lane-group width G and chunks per lane (each

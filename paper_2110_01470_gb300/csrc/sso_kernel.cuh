@@ -1531,21 +1531,6 @@ __global__ void __launch_bounds__(GenBound<MC>::threads) sso_generations(const K
     }
 }
 
-// FP64 fitness of every instance's gBest row (used when only FP32 bounds are known).
-template <class Pos>
-__global__ void best_f64_kernel(const InstDev* inst, int n_inst)
-{
-    const int k = blockIdx.x;
-    if (k >= n_inst) return;
-    const InstDev& in = inst[k];
-    if (in.gb->has64) return;
-    const double f = fit64_row<Pos>(hot_of(in), static_cast<const Pos*>(in.gbrow), true);
-    if (threadIdx.x == 0) {
-        in.gb->f64 = f;
-        in.gb->has64 = 1;
-    }
-}
-
 template <class Pos, bool F32R, int MC>
 inline cudaError_t launch_generations(const KParams& p, int grid, int block, size_t smem, cudaStream_t s)
 {
