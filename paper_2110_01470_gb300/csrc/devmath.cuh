@@ -71,11 +71,14 @@ __device__ __forceinline__ double sinpi_sq_f64(double z)
 }
 
 // sin(pi x) with its sign: x = n + r, n the nearest integer (half even),
-// sin(pi x) = (-1)^n sin(pi r); n is odd iff n / 2 is not an integer.
+// sin(pi x) = (-1)^n sin(pi r); n's parity is the last bit of n + 1.5 2^52 (one
+// FP64 instruction), or, beyond 2^51, whether n / 2 is an integer.
 __device__ __forceinline__ double sinpi_f64(double x)
 {
     const double n = rint(x);
     const double s = sinpi_reduced_f64(__dsub_rn(x, n));
+    if (((uint32_t)__double2hiint(n) & 0x7fffffffu) < 0x43200000u)
+        return (__double2loint(__dadd_rn(n, 0x1.8p52)) & 1) ? -s : s;
     const double h = __dmul_rn(n, 0.5);
     return (h != rint(h)) ? -s : s;
 }
@@ -90,7 +93,8 @@ __device__ __forceinline__ double sin_rad_f64(double a)
 }
 __device__ __forceinline__ double cos_rad_f64(double a)
 {
-    const double s = sinpi_f64(__dmul_rn(a, 0x1.45f306dc9c883p-3));
+    const double q = __dmul_rn(a, 0x1.45f306dc9c883p-3);
+    const double s = sinpi_reduced_f64(__dsub_rn(q, rint(q)));      // the sign cancels in the square
     return __fma_rn(__dmul_rn(-2.0, s), s, 1.0);
 }
 

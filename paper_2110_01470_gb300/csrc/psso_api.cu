@@ -75,6 +75,9 @@ struct HostInst {
     size_t off_X = 0, off_P = 0, off_pf64 = 0, off_plo = 0, off_phi = 0, off_pver = 0,
            off_pflag = 0, off_grow = 0, off_rec = 0, off_rec2 = 0, off_gb = 0, off_gbrow = 0,
            off_log = 0, off_o64 = 0, off_o32 = 0, off_w64 = 0, off_w32 = 0, off_M64 = 0, off_M32 = 0;
+    size_t off_tab = 0;           // Griewank: sqrt(j + 1), j < D (a constant, not part of the saved state)
+    bool one_block = false;       // at most four passes of a default block: psso_set_gbest takes it
+                                  // whether it runs in one block or, pipelined, in several
     int64_t i_base = 0;           // shard of a larger swarm: index of its first particle
     bool tc = false;              // generations run by the tensor-core pipeline
     bool bp = false;              // generations run by the batched throughput pipeline
@@ -213,6 +216,16 @@ psso_status check_problem(const psso_problem& pr, int precision, int idx)
     return PSSO_OK;
 }
 
+// A single swarm of more warps (of 32 / G particles) than this, no block limit
+// given, is spread over pipelined blocks of one compute warp each instead of
+// running its up to four passes in one block.  Measured (us per generation,
+// one block / spread), sphere: FP64 N = 8, D = 30 (2 warps) 6.1 / 3.6, N = 100,
+// D = 30 (25 warps) 16.7 / 3.9; Ackley: FP64 N = 16, D = 10 (2) 11.3 / 11.2, N =
+// 100, D = 30 51.6 / 9.8; FP32 N = 16, D = 10 (2) 11.3 / 11.7, N = 32, D = 10 (4)
+// 14.4 / 13.5, N = 100, D = 30 15.5 / 7.9.  One block needs no exchange, but its
+// SM's FP64 unit (or issue slots) serves every particle.
+constexpr int ONE_BLOCK_WARPS_F64 = 1, ONE_BLOCK_WARPS_F32 = 2;
+
 // Picks blocks per instance and assigns units to blocks.
 psso_status plan(psso_ctx* h)
 {
@@ -257,12 +270,18 @@ psso_status plan(psso_ctx* h)
     // One multi-block swarm: a control warp plus enough compute warps for one
     // particle per compute group and about one block per SM (pipelined blocks).
     bool pipe = false;
+    if (n_kernel == 1) {
+        HostInst& I = h->inst[only];
+        const int gpw = 32 / I.G;
+        I.one_block = (I.pr.N + (int64_t)nw * gpw - 1) / ((int64_t)nw * gpw) <= sbm;
+    }
     if (n_kernel == 1 && h->cfg.pipeline != 2) {
         const HostInst& I = h->inst[only];
         const int gpw = 32 / I.G;
         const int64_t groups = (I.pr.N + gpw - 1) / gpw;
-        const int64_t single_passes = (I.pr.N + (int64_t)nw * gpw - 1) / ((int64_t)nw * gpw);
-        if (single_passes > sbm) {
+        const bool spread = h->cfg.single_block_max == 0 &&
+                            groups > (h->variant == V_F32R ? ONE_BLOCK_WARPS_F32 : ONE_BLOCK_WARPS_F64);
+        if (!I.one_block || spread) {
             // at most 128 blocks: each lane of the control warp then polls <= 4
             // records, all in flight at once
             const int64_t blocks_cap = std::min<int64_t>(prop.multiProcessorCount, 128);
@@ -411,6 +430,82 @@ psso_status plan(psso_ctx* h)
     return fail(PSSO_ERR_UNSUPPORTED, "could not find a co-resident launch shape");
 }
 
+// Offsets of instance I's saved state from `off` on, for R blocks; returns the end.
+size_t layout_state(const psso_ctx* h, HostInst& I, int R, size_t off)
+{
+    auto take = [&](size_t bytes) {
+        off = align_up(off, 256);
+        const size_t at = off;
+        off += bytes;
+        return at;
+    };
+    const bool f32r = h->precision == PSSO_PREC_F32_RECHECK;
+    const size_t N = (size_t)I.pr.N, row = (size_t)I.Dp * h->pos_size;
+    I.off_X = take(N * row);
+    I.off_P = take(N * row);
+    I.off_pf64 = take(N * 8);
+    I.off_plo = take(f32r ? N * 4 : 0);
+    I.off_phi = take(f32r ? N * 4 : 0);
+    I.off_pver = take(N * 4);
+    I.off_pflag = take(f32r ? N * 4 : 0);
+    I.off_grow = take(SLOTS * (size_t)R * I.Dp * (h->pos_size / 4) * 8);   // tagged words
+    I.off_rec = take(SLOTS * (size_t)R * REC_WORDS * 8);
+    I.off_rec2 = take(SLOTS * (size_t)R * REC_WORDS * 8);
+    I.off_gb = take(sizeof(GBestDev));
+    I.off_gbrow = take(row);
+    I.off_log = take((h->cfg.log_stride > 0 ? (size_t)h->cfg.log_capacity : 0) * sizeof(LogDev));
+    I.off_o64 = take((size_t)I.Dp * 8);
+    I.off_o32 = take((size_t)I.Dp * 4);
+    I.off_w64 = take(I.w.empty() ? 0 : (size_t)I.Dp * 8);
+    I.off_w32 = take(I.w.empty() ? 0 : (size_t)I.Dp * 4);
+    I.off_M64 = take(I.M.size() * 8);
+    I.off_M32 = take(I.M.size() * 8);   // float(M), then float(M - float(M))
+    return off;
+}
+
+// Several blocks: the exchange records and row of generation g rewritten so
+// that the next launch's first step A finds this gBest (rank 0 carries it; the
+// other ranks' records lose against every value).
+psso_status publish_gbest(psso_ctx* h, const HostInst& I, int64_t g, const GBestDev& gb, const char* row)
+{
+    const uint64_t tag = (uint64_t)(g & 0xffff) << 48;
+    const size_t slot = (size_t)(g % SLOTS), R = (size_t)I.R, wpe = h->pos_size / 4;
+    auto u64 = [](double v) {
+        uint64_t b;
+        std::memcpy(&b, &v, 8);
+        return b;
+    };
+    auto u32 = [](float v) {
+        uint32_t b;
+        std::memcpy(&b, &v, 4);
+        return (uint64_t)b;
+    };
+    std::vector<uint64_t> rec(R * REC_WORDS), words((size_t)I.Dp * wpe);
+    for (size_t r = 0; r < R; ++r) {
+        // a losing record: a NaN with FP64 fitness, infinite bounds with FP32
+        const bool has64 = r == 0 ? gb.has64 != 0 : h->variant != V_F32R;
+        const uint64_t v = !has64 ? (r == 0 ? u32(gb.lo) | (u32(gb.hi) << 32) : 0x7f8000007f800000ull)
+                                  : r == 0 ? u64(gb.f64) : 0x7ff8000000000000ull;
+        const uint64_t idx = r == 0 ? (uint64_t)(uint32_t)gb.idx : 0x7ffffffeull;
+        uint64_t* w = rec.data() + r * REC_WORDS;
+        w[RW_IDX] = tag | ((uint64_t)has64 << 32) | idx;
+        w[RW_VER] = tag | (r == 0 ? gb.ver : 0u);
+        w[RW_V0] = tag | (v & 0xffffffffull);
+        w[RW_V1] = tag | (v >> 32);
+        w[RW_ACC] = w[RW_RCK] = tag;
+    }
+    for (size_t q = 0; q < words.size(); ++q) {
+        uint32_t part;
+        std::memcpy(&part, row + 4 * q, 4);
+        words[q] = tag | part;
+    }
+    CUDA_TRY(cudaMemcpy(h->arena + I.off_rec + slot * R * REC_WORDS * 8, rec.data(), rec.size() * 8,
+                        cudaMemcpyHostToDevice));
+    CUDA_TRY(cudaMemcpy(h->arena + I.off_grow + slot * R * words.size() * 8, words.data(), words.size() * 8,
+                        cudaMemcpyHostToDevice));
+    return PSSO_OK;
+}
+
 void fill_instdev(psso_ctx* h, std::vector<InstDev>& out)
 {
     char* A = h->arena;
@@ -445,7 +540,9 @@ void fill_instdev(psso_ctx* h, std::vector<InstDev>& out)
         d.ubf = float_at_or_below(I.pr.ub);
         d.o64 = reinterpret_cast<const double*>(A + I.off_o64);
         d.o32 = reinterpret_cast<const float*>(A + I.off_o32);
-        d.w64 = I.w.empty() ? nullptr : reinterpret_cast<const double*>(A + I.off_w64);
+        d.w64 = I.pr.fn == PSSO_GRIEWANK ? reinterpret_cast<const double*>(A + I.off_tab)
+                : I.w.empty()            ? nullptr
+                                         : reinterpret_cast<const double*>(A + I.off_w64);
         d.w32 = I.w.empty() ? nullptr : reinterpret_cast<const float*>(A + I.off_w32);
         d.M64 = I.M.empty() ? nullptr : reinterpret_cast<const double*>(A + I.off_M64);
         d.M32 = I.M.empty() ? nullptr : reinterpret_cast<const float*>(A + I.off_M32);
@@ -1016,31 +1113,11 @@ psso_status create_impl(const psso_problem* problems, int32_t count, const psso_
     h->off_block_first = take(sizeof(int32_t) * h->block_first.size());
     h->off_status = take(sizeof(StatusDev));
     h->off_best = take(sizeof(BestPack) + (size_t)max_dp * h->pos_size);
+    for (auto& I : h->inst)
+        if (I.pr.fn == PSSO_GRIEWANK) I.off_tab = take((size_t)I.Dp * 8);
     h->state_off = align_up(off, 256);
-    const bool f32r = h->precision == PSSO_PREC_F32_RECHECK;
     const size_t logcap = c.log_stride > 0 ? (size_t)c.log_capacity : 0;
-    for (auto& I : h->inst) {
-        const size_t N = (size_t)I.pr.N, row = (size_t)I.Dp * h->pos_size;
-        I.off_X = take(N * row);
-        I.off_P = take(N * row);
-        I.off_pf64 = take(N * 8);
-        I.off_plo = take(f32r ? N * 4 : 0);
-        I.off_phi = take(f32r ? N * 4 : 0);
-        I.off_pver = take(N * 4);
-        I.off_pflag = take(f32r ? N * 4 : 0);
-        I.off_grow = take(SLOTS * (size_t)I.R * I.Dp * (h->pos_size / 4) * 8);   // tagged words
-        I.off_rec = take(SLOTS * (size_t)I.R * REC_WORDS * 8);
-        I.off_rec2 = take(SLOTS * (size_t)I.R * REC_WORDS * 8);
-        I.off_gb = take(sizeof(GBestDev));
-        I.off_gbrow = take(row);
-        I.off_log = take(logcap * sizeof(LogDev));
-        I.off_o64 = take((size_t)I.Dp * 8);
-        I.off_o32 = take((size_t)I.Dp * 4);
-        I.off_w64 = take(I.w.empty() ? 0 : (size_t)I.Dp * 8);
-        I.off_w32 = take(I.w.empty() ? 0 : (size_t)I.Dp * 4);
-        I.off_M64 = take(I.M.size() * 8);
-        I.off_M32 = take(I.M.size() * 8);   // float(M), then float(M - float(M))
-    }
+    for (auto& I : h->inst) off = layout_state(h, I, I.R, off);
     h->arena_size = align_up(off, 256);
     cudaError_t e = cudaMalloc(&h->arena, h->arena_size);
     if (e != cudaSuccess) {
@@ -1073,6 +1150,13 @@ psso_status create_impl(const psso_problem* problems, int32_t count, const psso_
             e = cudaMemsetAsync(h->arena + I.off_log, 0xff, logcap * sizeof(LogDev), h->stream);
         const size_t nd = (size_t)I.pr.D;
         const bool hw = !I.w.empty();
+        if (I.pr.fn == PSSO_GRIEWANK) {
+            staging.emplace_back(nd * 8);
+            double* tab = reinterpret_cast<double*>(staging.back().data());
+            for (size_t j = 0; j < nd; ++j) tab[j] = std::sqrt((double)(j + 1));
+            if (e == cudaSuccess) e = cudaMemcpyAsync(h->arena + I.off_tab, tab, nd * 8, cudaMemcpyHostToDevice, h->stream);
+            h->h2d += (int64_t)(nd * 8);
+        }
         staging.emplace_back(nd * (hw ? 24 : 12));
         char* b = staging.back().data();
         double* o64 = reinterpret_cast<double*>(b);
@@ -1257,7 +1341,7 @@ psso_status psso_set_gbest(psso_handle h, int32_t instance, double value, int64_
     if (!std::isfinite(value)) return fail(PSSO_ERR_ARG, "psso_set_gbest: value must be finite");
     if (h->failed) return fail(PSSO_ERR_STATE, "the handle failed earlier");
     const HostInst& I = h->inst[instance];
-    if (h->async || (!I.tc && !I.bp && I.R != 1))
+    if (h->async || (!I.tc && !I.bp && I.R != 1 && !I.one_block))
         return fail(PSSO_ERR_UNSUPPORTED,
                     "psso_set_gbest: the instance's gBest comes from a cross-block exchange or the "
                     "asynchronous flow (create it with psso_create_shard)");
@@ -1287,6 +1371,7 @@ psso_status psso_set_gbest(psso_handle h, int32_t instance, double value, int64_
     CUDA_TRY(cudaMemcpy(h->arena + I.off_gbrow, buf.data(), (size_t)I.Dp * h->pos_size, cudaMemcpyHostToDevice));
     CUDA_TRY(cudaMemcpy(h->arena + I.off_gb, &gb, sizeof gb, cudaMemcpyHostToDevice));
     h->h2d += (int64_t)((size_t)I.Dp * h->pos_size + sizeof gb);
+    if (I.R > 1) return publish_gbest(h, I, h->gen, gb, buf.data());
     return PSSO_OK;
 }
 
@@ -1514,21 +1599,54 @@ psso_status psso_save(psso_handle h, void* buf, size_t cap, size_t* n)
     return PSSO_OK;
 }
 
+// A state saved by a one-block run of a swarm that this handle spreads over
+// several blocks: everything but the exchange records is copied
+// by field, the records are made from the gBest.
+static psso_status load_one_block(psso_ctx* h, const SaveHeader& hd, const char* state)
+{
+    const HostInst& I = h->inst[0];
+    HostInst J = I;
+    layout_state(h, J, 1, h->state_off);
+    auto src = [&](size_t off) { return state + (off - h->state_off); };
+    auto put = [&](size_t to, size_t from, size_t bytes) {
+        return cudaMemcpy(h->arena + to, src(from), bytes, cudaMemcpyHostToDevice);
+    };
+    const size_t row = (size_t)I.Dp * h->pos_size;
+    CUDA_TRY(put(h->state_off, h->state_off, I.off_grow - h->state_off));
+    CUDA_TRY(put(I.off_gb, J.off_gb, sizeof(GBestDev)));
+    CUDA_TRY(put(I.off_gbrow, J.off_gbrow, row));
+    CUDA_TRY(put(I.off_log, J.off_log, J.off_o64 - J.off_log));
+    GBestDev gb;
+    std::memcpy(&gb, src(J.off_gb), sizeof gb);
+    return publish_gbest(h, I, hd.gen, gb, src(J.off_gbrow));
+}
+
 psso_status psso_load(psso_handle h, const void* buf, size_t n)
 {
     if (!h || !buf) return fail(PSSO_ERR_ARG, "handle or buf is NULL");
     if (n < sizeof(SaveHeader)) return fail(PSSO_ERR_ARG, "buffer too small");
     SaveHeader hd;
     std::memcpy(&hd, buf, sizeof hd);
+    const char* data = static_cast<const char*>(buf) + sizeof hd;
     const size_t state = h->arena_size - h->state_off;
-    if (std::memcmp(hd.magic, "PSSOST01", 8) != 0 || hd.state_bytes != (int64_t)state ||
-        n != sizeof hd + state || hd.grid != h->grid || hd.block != h->block ||
-        hd.n_inst != (int32_t)h->inst.size() || hd.variant != h->variant)
+    const bool same = hd.state_bytes == (int64_t)state && hd.grid == h->grid && hd.block == h->block;
+    bool one_block = false;
+    if (!same && h->inst.size() == 1 && h->inst[0].one_block && h->inst[0].R > 1 && hd.grid == 1 &&
+        hd.block == (h->cfg.threads_per_block ? h->cfg.threads_per_block : 256)) {
+        HostInst J = h->inst[0];
+        one_block = hd.state_bytes == (int64_t)(align_up(layout_state(h, J, 1, h->state_off), 256) - h->state_off);
+    }
+    if (std::memcmp(hd.magic, "PSSOST01", 8) != 0 || !(same || one_block) ||
+        n != sizeof hd + (size_t)hd.state_bytes || hd.n_inst != (int32_t)h->inst.size() || hd.variant != h->variant)
         return fail(PSSO_ERR_ARG, "state was saved from a handle with other problems or launch shape");
     CUDA_TRY(cudaSetDevice(h->device));
     CUDA_TRY(cudaStreamSynchronize(h->stream));
-    CUDA_TRY(cudaMemcpy(h->arena + h->state_off, static_cast<const char*>(buf) + sizeof hd, state,
-                        cudaMemcpyHostToDevice));
+    if (one_block) {
+        const psso_status st = load_one_block(h, hd, data);
+        if (st != PSSO_OK) return st;
+    } else {
+        CUDA_TRY(cudaMemcpy(h->arena + h->state_off, data, state, cudaMemcpyHostToDevice));
+    }
     CUDA_TRY(cudaMemset(h->arena + h->off_status, 0, sizeof(StatusDev)));
     for (auto& I : h->inst)
         if (I.tc) CUDA_TRY(cudaMemset(&I.rh.dev.ctl->status, 0, sizeof(int)));

@@ -476,8 +476,9 @@ __device__ __forceinline__ void particle_compute(const Hot& in, const View<Pos>&
     s.cachef = 0.0;
     s.undecided = false;
     if constexpr (!F32R) {
-        const double f = fit64<Pos, MAXC>(in, s.x, lane_g, gmask, in.G);
-        const double pf = (g == 0) ? f : v.pf64[e];
+        const double cut = (g == 0) ? DBL_MAX : v.pf64[e];
+        const double f = fit64<Pos, MAXC>(in, s.x, lane_g, gmask, in.G, cut);
+        const double pf = (g == 0) ? f : cut;
         s.accept = (g == 0) || le_f64(f, pf);
         s.wstate = s.accept;
         s.f64v = s.accept ? f : pf;
