@@ -2,6 +2,7 @@
 // the on-demand FP64 evaluation of gBest rows.
 #include <climits>
 
+#include "bat_rows.cuh"
 #include "sso_kernel.cuh"
 
 namespace psso {
@@ -71,7 +72,8 @@ cudaError_t bat_rows_call(int variant, int fn, bool wide, int op, const BatRowsP
 // key and the index -- and the winner's other fields afterwards.  The
 // candidates of the exact pass are first collected by a scan over all
 // threads: one warp walking the particles one load at a time cost a load
-// latency per particle and warp.  40 swarms, FP64: 17 -> 10 us per launch.
+// latency per particle and warp.  40 swarms, FP64: 17 -> 10 us per launch; 512
+// swarms, FP32, generations 20-60: 171-308 -> 111-188 us.
 constexpr int ARGMIN_LIST = 2048;
 
 struct BatKey {
@@ -127,8 +129,35 @@ __device__ __forceinline__ BatKey key_block(BatKey k, BatKey* sh)
     return k;
 }
 
+// The rotated functions' rows, out of line (the whole-row code needs 255
+// registers, which left an SM one block of the arg-min).
+template <class Pos>
+__device__ __noinline__ double exact_row_general(const Hot& in, const Pos* row)
+{
+    return fit64_row<Pos>(in, row, false);
+}
+
+// FP64 fitness of a row by one warp; the plain functions in rolled code (the
+// unrolled whole-row code takes longer to fetch than to run once).
+template <class Pos>
+__device__ double exact_row(const Hot& in, const Pos* row)
+{
+    const int lane = threadIdx.x & 31, nq = (in.nchunks + 31) >> 5;
+    switch (in.fn) {
+#define PSSO_ROW_FN(F) \
+    case F: return row_f64<F, Pos>(row + 4 * lane, true, lane, 32, in.nchunks, nq, in.D, in.o64, in.w64)
+    PSSO_ROW_FN(FN_SPHERE);
+    PSSO_ROW_FN(FN_ELLIPSOID);
+    PSSO_ROW_FN(FN_RASTRIGIN);
+    PSSO_ROW_FN(FN_ROSENBROCK);
+    PSSO_ROW_FN(FN_ACKLEY);
+#undef PSSO_ROW_FN
+    default: return exact_row_general<Pos>(in, row);
+    }
+}
+
 template <class Pos, bool F32R>
-__global__ void __launch_bounds__(256) bat_argmin(const InstDev* inst, const int32_t* ids, long long* gen,
+__global__ void __launch_bounds__(256, 4) bat_argmin(const InstDev* inst, const int32_t* ids, long long* gen,
                                                   unsigned* ticket, BatCounters* cnt)
 {
     __shared__ BatKey sh[8];
@@ -159,9 +188,15 @@ __global__ void __launch_bounds__(256) bat_argmin(const InstDev* inst, const int
         if (b.l2 <= b.mh) {
             // every pBest that can be the minimum gets its FP64 value, a list of
             // candidates at a time, a warp per candidate
+            // (a converged swarm's candidates are mostly copies of the gBest row, whose
+            // value is known: they take it; a gBest put there by psso_set_gbest has a
+            // value of the caller's)
             const Hot hin = hot_of(d);
             const int lane = threadIdx.x & 31;
             const float m = b.mh;
+            const Pos* const gr = static_cast<const Pos*>(d.gbrow);
+            const bool known = g > 0 && d.gb->has64 && d.gb->ver != 0xffffffffu;
+            const double gf = d.gb->f64;
             for (int base = 0; base < N; base += ARGMIN_LIST) {
                 __syncthreads();
                 if (threadIdx.x == 0) n_list = 0;
@@ -172,7 +207,17 @@ __global__ void __launch_bounds__(256) bat_argmin(const InstDev* inst, const int
                 __syncthreads();
                 for (int e = threadIdx.x >> 5; e < n_list; e += 8) {
                     const int i = list[e];
-                    const double f = fit64_row<Pos>(hin, static_cast<const Pos*>(d.P) + (int64_t)i * d.Dp, false);
+                    const Pos* const row = static_cast<const Pos*>(d.P) + (int64_t)i * d.Dp;
+                    bool copy = known;
+                    for (int q = lane; q < d.nchunks && copy; q += 32) {
+                        Pos u[4], v[4];
+                        ld4(row + 4 * q, u);
+                        ld4(gr + 4 * q, v);
+#pragma unroll
+                        for (int t = 0; t < 4; ++t) copy = copy && same_bits(u[t], v[t]);
+                    }
+                    copy = __all_sync(0xffffffffu, copy);
+                    const double f = copy ? gf : exact_row<Pos>(hin, row);
                     if (lane == 0) {
                         d.pf64[i] = f;
                         d.pflag[i] = 1u;
