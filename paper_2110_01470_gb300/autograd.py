@@ -11,7 +11,8 @@ from __future__ import annotations
 
 import torch
 
-from . import FN, psso_fitness_backward_ws, psso_fitness_forward_ws, psso_fitness_workspace_size
+from . import (FN, PSSO_ROT_ACKLEY, PSSO_ROT_ELLIPSOID, PSSO_ROT_RASTRIGIN,
+               psso_fitness_backward_ws, psso_fitness_forward_ws, psso_fitness_workspace_size)
 
 
 def _ptr(t):
@@ -22,7 +23,15 @@ def _stream(device):
     return torch.cuda.current_stream(device).cuda_stream
 
 
+try:  # the stream's handle without a torch.cuda.Stream object around it
+    from torch._C import _cuda_getCurrentRawStream as _raw_stream
+except ImportError:
+    _raw_stream = None
+
+
 def _workspace(fn, N, D, device):
+    if fn not in _ROTATED:      # no call needed: the other functions use no workspace
+        return None, 0
     n = psso_fitness_workspace_size(fn, N, D)
     if n == 0:
         return None, 0
@@ -30,21 +39,31 @@ def _workspace(fn, N, D, device):
     return torch.empty(n, dtype=torch.uint8, device=device), n
 
 
+_ROTATED = (PSSO_ROT_ELLIPSOID, PSSO_ROT_RASTRIGIN, PSSO_ROT_ACKLEY)
+
+
+def _data(t, device):
+    """t as a contiguous float32 tensor on the device (itself if it is one)."""
+    if t is None or (t.dtype is torch.float32 and t.device == device and t.is_contiguous()):
+        return t
+    return t.to(device, torch.float32).contiguous()
+
+
 class Fitness(torch.autograd.Function):
     @staticmethod
     def forward(ctx, X, fn, shift, weights=None, rotation=None):
-        if not (X.is_cuda and X.dtype == torch.float32 and X.dim() == 2):
+        if not (X.is_cuda and X.dtype is torch.float32 and X.dim() == 2):
             raise TypeError("X must be a 2-D float32 CUDA tensor")
+        device = X.device
         X = X.contiguous()
         N, D = X.shape
-        shift = shift.to(X.device, torch.float32).contiguous()
-        weights = None if weights is None else weights.to(X.device, torch.float32).contiguous()
-        rotation = None if rotation is None else rotation.to(X.device, torch.float32).contiguous()
-        f = torch.empty(N, device=X.device, dtype=torch.float32)
+        shift, weights, rotation = _data(shift, device), _data(weights, device), _data(rotation, device)
+        f = torch.empty(N, device=device, dtype=torch.float32)
         fn = FN[fn] if isinstance(fn, str) else int(fn)
-        ws, nws = _workspace(fn, N, D, X.device)
+        ws, nws = _workspace(fn, N, D, device)
+        stream = _raw_stream(device.index) if _raw_stream else _stream(device)
         psso_fitness_forward_ws(fn, N, D, X.data_ptr(), shift.data_ptr(), _ptr(weights),
-                                _ptr(rotation), f.data_ptr(), _ptr(ws), nws, _stream(X.device))
+                                _ptr(rotation), f.data_ptr(), _ptr(ws), nws, stream)
         ctx.save_for_backward(X, shift, weights, rotation)
         ctx.fn = fn
         return f
@@ -53,12 +72,14 @@ class Fitness(torch.autograd.Function):
     def backward(ctx, grad_f):
         X, shift, weights, rotation = ctx.saved_tensors
         N, D = X.shape
-        grad_f = grad_f.to(torch.float32).contiguous()
+        device = X.device
+        grad_f = _data(grad_f, grad_f.device)
         gX = torch.empty_like(X)
-        ws, nws = _workspace(ctx.fn, N, D, X.device)
+        ws, nws = _workspace(ctx.fn, N, D, device)
+        stream = _raw_stream(device.index) if _raw_stream else _stream(device)
         psso_fitness_backward_ws(ctx.fn, N, D, X.data_ptr(), shift.data_ptr(), _ptr(weights),
                                  _ptr(rotation), grad_f.data_ptr(), gX.data_ptr(), _ptr(ws), nws,
-                                 _stream(X.device))
+                                 stream)
         return gX, None, None, None, None
 
 
