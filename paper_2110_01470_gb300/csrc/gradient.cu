@@ -358,8 +358,8 @@ cudaError_t launch_polish(const InstDev* inst, int k, int lattice, int owner_ran
 // planes, launches for small ones.  Against one CTA per 128 x 128 tile with Z
 // stored a word at a time, a warp per row for f and for the planes of G, and
 // the outputs pre-filled with NaN (forward + backward): rotated Ackley, N =
-// 4096, D = 256: 123 -> 65 us; rotated Rastrigin, N = 8192, D = 1000: 568
-// -> 305 us.
+// 4096, D = 256: 123 -> 63 us; rotated Rastrigin, N = 8192, D = 1000: 568
+// -> 303 us; with the sequence's launches overlapped (pdl.cuh) 51 and 288 us.
 namespace gtc {
 
 using tc::BM;
@@ -410,6 +410,7 @@ struct PrepArgs {
 };
 __global__ void __launch_bounds__(256) prep_planes(const PrepArgs a)
 {
+    pdl_trigger();
     __shared__ float tile[32][33];
     if (blockIdx.x == 0 && threadIdx.x == 0) *a.status = 0;
     if ((int)blockIdx.x < a.row_blocks) {
@@ -503,6 +504,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc::P_THREADS, 1)
 // f from the sums of its terms (a thread per row); NaN if a GEMM wait ran out.
 __global__ void finish_rows(const float2* part, int groups, int fn, int N, int D, const int* status, float* f)
 {
+    pdl_entry();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
     float s1 = 0.f, s2 = 0.f;
@@ -520,6 +522,7 @@ __global__ void finish_rows(const float2* part, int groups, int fn, int N, int D
 // Outputs of a backward pass whose GEMM wait ran out: NaN, never stale values.
 __global__ void poison(float* out, size_t n, const int* status)
 {
+    pdl_entry();
     if (!*status) return;
     for (size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x; q < n; q += (size_t)gridDim.x * blockDim.x)
         out[q] = __int_as_float(0x7fffffff);
@@ -533,6 +536,7 @@ __global__ void __launch_bounds__(256) gz_rows(const float* __restrict__ Z, cons
                                                const float* __restrict__ gf, int N, int D, int Np, int Kp,
                                                __nv_bfloat16* A)
 {
+    pdl_entry();
     const int i = (int)blockIdx.x * 8 + (threadIdx.x >> 5);
     if (i >= N) return;
     const int lane = threadIdx.x & 31, nc = Kp / 4;
@@ -587,10 +591,10 @@ inline void launch_gz(int maxc, const float* Z, const float* w, const float* gf,
 {
     const unsigned grid = (unsigned)((N + 7) / 8);
     switch (maxc) {
-    case 1: gz_rows<FN, 1><<<grid, 256, 0, s>>>(Z, w, gf, N, D, Np, Kp, A); break;
-    case 2: gz_rows<FN, 2><<<grid, 256, 0, s>>>(Z, w, gf, N, D, Np, Kp, A); break;
-    case 4: gz_rows<FN, 4><<<grid, 256, 0, s>>>(Z, w, gf, N, D, Np, Kp, A); break;
-    default: gz_rows<FN, 8><<<grid, 256, 0, s>>>(Z, w, gf, N, D, Np, Kp, A); break;
+    case 1: launch_pdl(gz_rows<FN, 1>, dim3(grid), dim3(256), 0, s, Z, w, gf, N, D, Np, Kp, A); break;
+    case 2: launch_pdl(gz_rows<FN, 2>, dim3(grid), dim3(256), 0, s, Z, w, gf, N, D, Np, Kp, A); break;
+    case 4: launch_pdl(gz_rows<FN, 4>, dim3(grid), dim3(256), 0, s, Z, w, gf, N, D, Np, Kp, A); break;
+    default: launch_pdl(gz_rows<FN, 8>, dim3(grid), dim3(256), 0, s, Z, w, gf, N, D, Np, Kp, A); break;
     }
 }
 
@@ -756,8 +760,8 @@ void launch_gemm(const CUtensorMap& ta, const CUtensorMap& tb, const psso::gtc::
     epi.N = (int)N;
     epi.D = (int)D;
     const tc::GemmArgs ga{L.Np, L.Jp, L.Kp, status};
-    gtc::pair_gemm<Epi><<<tc::pair_grid(L.Np, L.Jp, sms), tc::P_THREADS,
-                          tc::pair_smem<tc::SplitCfg::PLANES, tc::SplitCfg::STG>(), s>>>(ta, tb, ga, epi);
+    launch_pdl(gtc::pair_gemm<Epi>, dim3(tc::pair_grid(L.Np, L.Jp, sms)), dim3(tc::P_THREADS),
+               tc::pair_smem<tc::SplitCfg::PLANES, tc::SplitCfg::STG>(), s, ta, tb, ga, epi);
 }
 
 // Operand planes of d = x - o and M (and M^T), and the tensor maps of A and M.
@@ -841,7 +845,8 @@ extern "C" psso_status psso_fitness_forward_ws(psso_fn fn, int64_t N, int64_t D,
     epi.fn = plain_fn(fn);
     epi.groups = (int)((D + 63) / 64);
     launch_gemm(ta, tb, L, status, epi, N, D, sms, s);
-    gtc::finish_rows<<<(unsigned)((N + 127) / 128), 128, 0, s>>>(epi.part, epi.groups, epi.fn, (int)N, (int)D, status, f);
+    launch_pdl(gtc::finish_rows, dim3((unsigned)((N + 127) / 128)), dim3(128), 0, s, (const float2*)epi.part, epi.groups,
+               epi.fn, (int)N, (int)D, (const int*)status, f);
     if (cudaGetLastError() != cudaSuccess) {
         set_last_error("psso_fitness_forward_ws: launch failed");
         return PSSO_ERR_CUDA;
@@ -892,7 +897,7 @@ extern "C" psso_status psso_fitness_backward_ws(psso_fn fn, int64_t N, int64_t D
     epi.out = grad_X;
     epi.vec = tc::store_width(grad_X, D);
     launch_gemm(ta, tbt, L, status, epi, N, D, sms, s);
-    gtc::poison<<<(unsigned)sms, 256, 0, s>>>(grad_X, (size_t)N * D, status);
+    launch_pdl(gtc::poison, dim3((unsigned)sms), dim3(256), 0, s, grad_X, (size_t)N * D, (const int*)status);
     if (cudaGetLastError() != cudaSuccess) {
         set_last_error("psso_fitness_backward_ws: launch failed");
         return PSSO_ERR_CUDA;

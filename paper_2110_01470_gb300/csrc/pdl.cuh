@@ -6,6 +6,10 @@
 // and wait in pdl_entry() until it has completed and its memory is visible;
 // every kernel of a sequence enters through pdl_entry before it touches memory
 // that another one writes, so the order is that of plain launches.
+// Rotated Ackley with its gradient, N = 4096, D = 256: 63 -> 51 us.  Not for
+// sequences that run beside others on the same GPU: the waiting blocks hold the
+// places that the other sequence's kernels want (two swarms of the rotated
+// pipeline, N = 8192, D = 1000: 54.3 -> 57.5 ms per 100 generations).
 #pragma once
 #include <cuda_runtime.h>
 #include <utility>

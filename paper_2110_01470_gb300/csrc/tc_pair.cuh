@@ -29,6 +29,7 @@
 // the leader's MMAs), tfull (both CTAs: a tile's MMAs are complete), tempty
 // (leader: the 16 epilogue warps of the pair).  Every wait is bounded.
 #pragma once
+#include "pdl.cuh"
 #include "tc_gemm.cuh"
 
 namespace psso {
@@ -195,6 +196,7 @@ __device__ __forceinline__ bool gemm_pair(const CUtensorMap* tmA, const CUtensor
     __syncthreads();
     cluster_sync();               // the peer's barriers exist
     tc_fence_after();
+    pdl_entry();                  // the operands are the previous kernel's
     const uint32_t tmem = tmem_slot;
 
     if (warp == 0) {
