@@ -75,110 +75,165 @@ __global__ void set_gen(RotCtl* ctl, long long g)
 }
 
 // ---- 1. update --------------------------------------------------------------
-template <int MAXC>
-__device__ void update_row(const RotDev& r, const Hot& in, int64_t i, int64_t g)
+// A warp per row, in grid-stride order, the row staged in the warp's shared
+// memory: the interval draws; the fresh-value blocks of the chunks that need
+// one (about a third), 32 a round; X and the row's scale and norm; the slices.
+// Bound: instruction issue (Philox 56 of about 130 lane-operations a variable)
+// close to HBM (28 bytes a variable: X, P read, X and four BF16 planes written;
+// 34 us at N = 8192, D = 1000).  With the row held in registers (64 of them at D =
+// 1000) an SM ran 8 to 16 warps, both Philox blocks of every chunk, and the
+// slices one rounding after the other: 54 -> 47 us per launch; N = 4096,
+// D = 256: 13 -> 13 us.
+constexpr int UPDATE_WARPS = 8;
+__global__ void __launch_bounds__(32 * UPDATE_WARPS, 4) rot_update(const RotDev r)
 {
-    const int lane = threadIdx.x & 31;
+    __shared__ __align__(16) float stage[UPDATE_WARPS][1024];
+    __shared__ uint32_t reqs[UPDATE_WARPS][256];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float* const row = stage[warp];
+    uint32_t* const req = reqs[warp];
+    const unsigned lt_mask = (1u << lane) - 1u;
     const InstDev& d = *r.inst;
-    float* xr = static_cast<float*>(d.X) + i * in.Dp;
-    const float* pr = static_cast<const float*>(d.P) + i * in.Dp;
-    const float* gs = static_cast<const float*>(d.gbrow);
+    const long long g = r.ctl->gen;
     const uint32_t gg = (uint32_t)g;
-    const uint32_t ctr3r = TAG_RHO | (in.sid << 8), ctr3f = TAG_FRESH | (in.sid << 8);
-    bool eqp = true;
-    float dmax = 0.f, l1 = 0.f;
-    float dv[MAXC][4], dl[MAXC][4];    // d = x - o exactly, as a float pair
+    const int nch = d.nchunks, D = d.D, Dp = d.Dp, nq = (nch + 31) >> 5;
+    if (!PSSO_CHK(Dp <= 1024, CHK_ROT_ROW, Dp)) return;
+    const uint32_t k0 = d.k0, k1 = d.k1;
+    const float* const o32 = as_global(d.o32);
+    const size_t plane = (size_t)r.Np * r.Kp;
+    const int nwarps = (int)gridDim.x * UPDATE_WARPS, N = (int)d.N;
+    for (int i = (int)blockIdx.x * UPDATE_WARPS + warp; i < N; i += nwarps) {
+        float* const xr = as_global(static_cast<float*>(d.X)) + (int64_t)i * Dp;
+        const float* const pr = as_global(static_cast<const float*>(d.P)) + (int64_t)i * Dp;
+        const uint32_t ii = (uint32_t)i + d.i_base;
+        __syncwarp();                    // the previous row's stage is consumed
+        bool eqp = true;
+        int nreq = 0;
+        {
+            const uint32_t Tg = d.Tg > 0xffffffffull ? 0xffffffffu : (uint32_t)d.Tg;
+            const uint32_t Tp = d.Tp > 0xffffffffull ? 0xffffffffu : (uint32_t)d.Tp;
+            const uint32_t Tw = d.Tw > 0xffffffffull ? 0xffffffffu : (uint32_t)d.Tw;
+            const bool fg = d.Tg > 0xffffffffull, fp = d.Tp > 0xffffffffull, fw = d.Tw > 0xffffffffull;
+            const uint32_t ctr3 = TAG_RHO | (d.sid << 8);
+            const float* const gs = as_global(static_cast<const float*>(d.gbrow));
+            // sources of the first and third interval (Eq. 2.1 as printed keeps x first
+            // and takes gBest third)
+            const float* const src1 = d.order ? xr : gs;
+            const float* const src3 = d.order ? gs : xr;
+#pragma unroll 2
+            for (int q = 0; q < nq; ++q) {
+                const int c = lane + 32 * q;
+                uint32_t nf = 0;
+                if (c < nch) {
+                    const uint32_t valid = 4 * c + 4 <= D ? 15u : (1u << (D - 4 * c)) - 1u;
+                    float x[4] = {0.f, 0.f, 0.f, 0.f};
+                    if (g == 0) {
+                        nf = valid;
+                    } else {
+                        float v1[4], v2[4], v3[4];
+                        ld4_cg(src1 + 4 * c, v1);
+                        ld4_cg(pr + 4 * c, v2);
+                        ld4_cg(src3 + 4 * c, v3);
+                        const uint4 rb = philox10(make_uint4((uint32_t)c, ii, gg, ctr3), k0, k1);
 #pragma unroll
-    for (int q = 0; q < MAXC; ++q) {
-        const int c = lane + 32 * q;
+                        for (int m = 0; m < 4; ++m) {
+                            const uint32_t w = word_of(rb, m);
+                            const bool lg = w < Tg || fg, lp = w < Tp || fp, lw = w < Tw || fw;
+                            // a variable of the last interval holds its pBest value until it is
+                            // drawn (beyond D every source is 0)
+                            x[m] = lg ? v1[m] : (lp || !lw) ? v2[m] : v3[m];
+                            if (!lw) nf |= 1u << m;
+                            eqp = eqp && same_bits(x[m], v2[m]);
+                        }
+                        nf &= valid;
+                    }
+                    st4(row + 4 * c, x);
+                }
+                const unsigned want = __ballot_sync(0xffffffffu, nf != 0u);
+                if (nf) req[nreq + __popc(want & lt_mask)] = (uint32_t)c | (nf << 8);
+                nreq += __popc(want);
+            }
+        }
+        __syncwarp();
+        {
+            Hot fh;                      // the fields fresh_chunk reads
+            fh.sid = d.sid;
+            fh.k0 = k0;
+            fh.k1 = k1;
+            fh.S32 = d.S32;
+            fh.L32 = d.L32;
+            fh.lbf = d.lbf;
+            fh.ubf = d.ubf;
+            for (int base = 0; base < nreq; base += 32) {
+                const int e = base + lane;
+                if (e < nreq) {
+                    const uint32_t rq = req[e], c = rq & 0xffu, nf = rq >> 8;
+                    float fv[4], pv[4];
+                    ld4(row + 4 * c, pv);
+                    fresh_chunk(fv, nf, c, ii, gg, g == 0 ? TAG_INIT : TAG_FRESH, fh);
 #pragma unroll
-        for (int m = 0; m < 4; ++m) dv[q][m] = dl[q][m] = 0.f;
-        if (c >= in.nchunks) continue;
-        const int nvalid = min(4, in.D - 4 * c);
-        const uint32_t valid = (1u << nvalid) - 1u;
-        float x[4] = {0.f, 0.f, 0.f, 0.f};
-        if (g == 0) {
-            fresh_chunk(x, valid, (uint32_t)c, (uint32_t)i + in.i_base, 0u, TAG_INIT, in);
-        } else {
-            const uint4 rb = philox10(make_uint4((uint32_t)c, (uint32_t)i + in.i_base, gg, ctr3r), in.k0, in.k1);
-            const uint4 fb = philox10(make_uint4((uint32_t)c, (uint32_t)i + in.i_base, gg, ctr3f), in.k0, in.k1);
-            float xo[4], po[4], go[4];
-            // xo: the third interval's source, go: the first's (Eq. 2.1 as printed
-            // swaps them: keep x first, gBest third)
-            ld4((in.order ? gs : xr) + 4 * c, xo);
-            ld4(pr + 4 * c, po);
-            ld4((in.order ? xr : gs) + 4 * c, go);
+                    for (int m = 0; m < 4; ++m)
+                        if (nf & (1u << m)) {
+                            eqp = eqp && same_bits(fv[m], pv[m]);
+                            pv[m] = fv[m];
+                        }
+                    st4(row + 4 * c, pv);
+                }
+            }
+        }
+        __syncwarp();
+        eqp = __all_sync(0xffffffffu, eqp);
+        // X, the row maximum and the L1 norm of d = x - o (exactly a float pair, TwoSum)
+        float dmax = 0.f, l1 = 0.f;
+        for (int q = 0; q < nq; ++q) {
+            const int c = lane + 32 * q;
+            if (c >= nch) continue;
+            float x[4], o[4];
+            ld4(row + 4 * c, x);
+            ld4_nc(o32 + 4 * c, o);
+            st4(xr + 4 * c, x);
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {            // beyond D: x = o = 0
+                const float ad = fabsf(__fsub_rn(x[m], o[m]));
+                dmax = fmaxf(dmax, ad);
+                l1 = __fadd_ru(l1, ad);
+            }
+        }
+        for (int off = 16; off > 0; off >>= 1) {
+            dmax = fmaxf(dmax, __shfl_xor_sync(0xffffffffu, dmax, off));
+            l1 = __fadd_ru(l1, __shfl_xor_sync(0xffffffffu, l1, off));
+        }
+        // |d| <= |fl(d)| (1 + 2^-24): the scale and the L1 norm cover the exact d
+        l1 = __fmul_ru(l1, 1.f + 0x1p-22f);
+        // the 7-bit integer slices of d / s_d (tc_gemm.cuh), four planes
+        const float sd = tc::slice_scale(dmax), inv = 1.f / sd;   // powers of two: exact
+        // differences whose scale leaves the range of a float: no bound holds
+        if (!(dmax < 0x1p120f) || sd < 0x1p-120f) l1 = INFINITY;
+        __nv_bfloat16* const arow = r.A + (size_t)i * r.Kp;
+        for (int q = 0; q < nq; ++q) {
+            const int c = lane + 32 * q;
+            if (c >= nch) continue;
+            float x[4], o[4];
+            ld4(row + 4 * c, x);
+            ld4_nc(o32 + 4 * c, o);
+            uint32_t u[4];
 #pragma unroll
             for (int m = 0; m < 4; ++m) {
-                const uint32_t w = word_of(rb, m);
-                const bool lg = (w < in.Tg32) || (in.tfull & 1u);
-                const bool lp = (w < in.Tp32) || (in.tfull & 2u);
-                const bool lw = (w < in.Tw32) || (in.tfull & 4u);
-                x[m] = lg ? go[m] : lp ? po[m] : lw ? xo[m] : fresh_f32(word_of(fb, m), in);
-                if (m >= nvalid) x[m] = 0.f;
-                eqp = eqp && same_bits(x[m], po[m]);
+                const float v = x[m], w = -o[m];
+                const float sum = __fadd_rn(v, w), bb = __fsub_rn(sum, v);   // TwoSum
+                const float lo = __fadd_rn(__fsub_rn(v, __fsub_rn(sum, bb)), __fsub_rn(w, bb));
+                u[m] = tc::slice_fields(__fmul_rn(sum, inv), __fmul_rn(lo, inv));
             }
+#pragma unroll
+            for (int p = 0; p < tc::SLICES; ++p)     // 4 consecutive bf16 (8 bytes) per plane
+                *reinterpret_cast<uint2*>(arow + p * plane + 4 * c) =
+                    make_uint2(tc::slice_pack(u[0], u[1], p), tc::slice_pack(u[2], u[3], p));
         }
-        st4(xr + 4 * c, x);
-#pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            const int j = 4 * c + m;
-            if (j < in.D) {
-                const float a = x[m], b = -__ldg(in.o32 + j);
-                const float sum = __fadd_rn(a, b), bb = __fsub_rn(sum, a);   // TwoSum
-                dv[q][m] = sum;
-                dl[q][m] = __fadd_rn(__fsub_rn(a, __fsub_rn(sum, bb)), __fsub_rn(b, bb));
-            }
-            dmax = fmaxf(dmax, fabsf(dv[q][m]));
-            l1 = __fadd_ru(l1, fabsf(dv[q][m]));
+        if (lane == 0) {
+            r.dscale[i] = sd;
+            r.dl1[i] = l1;
+            r.same[i] = (g > 0 && eqp) ? 1u : 0u;
         }
-    }
-    for (int off = 16; off > 0; off >>= 1) {
-        dmax = fmaxf(dmax, __shfl_xor_sync(0xffffffffu, dmax, off));
-        l1 = __fadd_ru(l1, __shfl_xor_sync(0xffffffffu, l1, off));
-    }
-    eqp = __all_sync(0xffffffffu, eqp);
-    // |d| <= |fl(d)| (1 + 2^-24): the scale and the L1 norm cover the exact d
-    l1 = __fmul_ru(l1, 1.f + 0x1p-22f);
-    // the 7-bit integer slices of d / s_d (tc_gemm.cuh), four planes
-    const float sd = tc::slice_scale(dmax), inv = 1.f / sd;   // powers of two: exact
-    const size_t plane = (size_t)r.Np * r.Kp;
-    __nv_bfloat16* arow = r.A + (size_t)i * r.Kp;
-#pragma unroll
-    for (int q = 0; q < MAXC; ++q) {
-        const int c = lane + 32 * q;
-        if (c >= in.nchunks) continue;
-        __nv_bfloat16 sl[4][tc::SLICES];
-#pragma unroll
-        for (int m = 0; m < 4; ++m) tc::slice4_pair(__fmul_rn(dv[q][m], inv), __fmul_rn(dl[q][m], inv), sl[m]);
-#pragma unroll
-        for (int p = 0; p < tc::SLICES; ++p) {
-            // 4 consecutive bf16 (8 bytes) per plane
-            uint2 u;
-            u.x = (uint32_t)__bfloat16_as_ushort(sl[0][p]) | ((uint32_t)__bfloat16_as_ushort(sl[1][p]) << 16);
-            u.y = (uint32_t)__bfloat16_as_ushort(sl[2][p]) | ((uint32_t)__bfloat16_as_ushort(sl[3][p]) << 16);
-            *reinterpret_cast<uint2*>(arow + p * plane + 4 * c) = u;
-        }
-    }
-    if (lane == 0) {
-        r.dscale[i] = sd;
-        r.dl1[i] = l1;
-        r.same[i] = (g > 0 && eqp) ? 1u : 0u;
-    }
-}
-
-__global__ void rot_update(const RotDev r)
-{
-    const int64_t i = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const InstDev& d = *r.inst;
-    if (i >= d.N) return;
-    const Hot in = hot_of(d);
-    const int64_t g = r.ctl->gen;
-    switch (in.maxc) {
-    case 1: update_row<1>(r, in, i, g); break;
-    case 2: update_row<2>(r, in, i, g); break;
-    case 4: update_row<4>(r, in, i, g); break;
-    default: update_row<8>(r, in, i, g); break;
     }
 }
 
@@ -1024,7 +1079,7 @@ cudaError_t enqueue_generation_timed(const RotHost& h, cudaStream_t s, cudaEvent
     const RotDev& r = h.dev;
     const int N = (int)h.N;
     const int wpb = 8;
-    rot_update<<<(N + wpb - 1) / wpb, 32 * wpb, 0, s>>>(r);
+    rot_update<<<std::min(4 * h.fix_grid, (N + UPDATE_WARPS - 1) / UPDATE_WARPS), 32 * UPDATE_WARPS, 0, s>>>(r);
     mark();
     rot_gemm_fit<<<h.gemm_grid, tc::P_THREADS, tc::pair_smem<SliceCfg::PLANES, SliceCfg::STG>(), s>>>(h.tmA, h.tmB, r);
     mark();

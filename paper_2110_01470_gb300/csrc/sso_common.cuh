@@ -62,6 +62,20 @@ __device__ __forceinline__ void ld4_cg(const double* p, double (&v)[4])
     const double2 b = __ldcg(reinterpret_cast<const double2*>(p) + 1);
     v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
 }
+// Read-only for the whole kernel.
+__device__ __forceinline__ void ld4_nc(const float* p, float (&v)[4])
+{
+    const float4 t = __ldg(reinterpret_cast<const float4*>(p));
+    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+}
+// A pointer read from memory, known to be global: its accesses then need not
+// keep their order with those of shared memory.
+template <class T>
+__device__ __forceinline__ T* as_global(T* p)
+{
+    __builtin_assume(__isGlobal(p));
+    return p;
+}
 __device__ __forceinline__ void st4(float* p, const float (&v)[4])
 {
     *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
