@@ -487,11 +487,15 @@ __global__ void rot_decide(const RotDev r)
 // g = gamma_n: |z~ - z| <= 1.01 u |z~| + (2 g^2 + 4 u g + 2^-42) S, where
 // S = sum |M||d| <= S~ (1 + 2 gamma_D)(1 + 2^-22) from the FP32 sum S~ of
 // |Mh||d_h|; 2^-42 S also covers the oracle's own FP64 rounding of z.
-// A block takes Z32_OUT outputs of one listed row; each warp keeps Z32_NJ
-// outputs in flight (independent chains sharing the loads of d), so a short
-// list still spreads over many blocks and the loads of M overlap.
-constexpr int Z32_NJ = 4;                       // outputs per warp in flight
-constexpr int Z32_OUT = 32;                     // outputs per block
+// A block takes Z32_OUT outputs of one listed row, each warp Z32_NJ of them
+// (independent chains sharing the loads of d).  The lists are short (about ten
+// rows), so a launch is one block's chain of loads, and M has left L2 since the
+// last generation: Z32_AHEAD steps' loads of M travel together, and a warp has
+// one group of outputs (one step's loads at a time and two groups a warp: 52 ->
+// 36 us per launch, rotated Rastrigin, N = 8192, D = 1000; ellipsoid 31 -> 12).
+constexpr int Z32_NJ = 4;                       // outputs per warp
+constexpr int Z32_OUT = 4 * Z32_NJ;             // outputs per block
+constexpr int Z32_AHEAD = 4;                    // steps of 32 k
 __global__ void __launch_bounds__(128) rot_z32(const RotDev r)
 {
     __shared__ float dh[1024], dl[1024];
@@ -525,62 +529,73 @@ __global__ void __launch_bounds__(128) rot_z32(const RotDev r)
         }
         __syncthreads();
         const size_t o = (size_t)(2 * e + row) * d.Dp;
-#pragma unroll 1
-        for (int pass = 0; pass < Z32_OUT / (4 * Z32_NJ); ++pass) {
-            const int j0 = jb * Z32_OUT + pass * 4 * Z32_NJ + warp * Z32_NJ;   // warp-uniform
-            int nv = D - j0;                     // outputs of this group inside the row
-            nv = nv < 0 ? 0 : nv > Z32_NJ ? Z32_NJ : nv;
-            if (lane == 0)
-                for (int t = nv; t < Z32_NJ; ++t)
-                    if (j0 + t < d.Dp) {
-                        r.z32[o + j0 + t] = 0.f;
-                        r.ez32[o + j0 + t] = 0.f;
-                    }
-            if (nv == 0) continue;
-            const float* mh[Z32_NJ];
-            const float* ml[Z32_NJ];
-            float p[Z32_NJ], sc[Z32_NJ], S[Z32_NJ];
+        const int j0 = jb * Z32_OUT + warp * Z32_NJ;   // warp-uniform
+        int nv = D - j0;                               // outputs of this group inside the row
+        nv = nv < 0 ? 0 : nv > Z32_NJ ? Z32_NJ : nv;
+        if (lane == 0)
+            for (int t = nv; t < Z32_NJ; ++t)
+                if (j0 + t < d.Dp) {
+                    r.z32[o + j0 + t] = 0.f;
+                    r.ez32[o + j0 + t] = 0.f;
+                }
+        if (nv == 0) continue;
+        const float* mh[Z32_NJ];
+        const float* ml[Z32_NJ];
+        float p[Z32_NJ], sc[Z32_NJ], S[Z32_NJ];
 #pragma unroll
-            for (int t = 0; t < Z32_NJ; ++t) {
-                const int j = t < nv ? j0 + t : j0;   // rows past the end repeat a valid one, unused
-                mh[t] = r.Mh + (size_t)j * D;
-                ml[t] = r.Ml + (size_t)j * D;
-                p[t] = sc[t] = S[t] = 0.f;
-            }
-            for (int k = lane; k < D; k += 32) {
-                const float b = dh[k], bl = dl[k];
+        for (int t = 0; t < Z32_NJ; ++t) {
+            const int j = t < nv ? j0 + t : j0;        // rows past the end repeat a valid one, unused
+            mh[t] = r.Mh + (size_t)j * D;
+            ml[t] = r.Ml + (size_t)j * D;
+            p[t] = sc[t] = S[t] = 0.f;
+        }
+#pragma unroll 1
+        for (int k0 = lane; k0 < D; k0 += 32 * Z32_AHEAD) {
+            float ah[Z32_AHEAD][Z32_NJ], al[Z32_AHEAD][Z32_NJ];
+#pragma unroll
+            for (int s = 0; s < Z32_AHEAD; ++s)
 #pragma unroll
                 for (int t = 0; t < Z32_NJ; ++t) {
-                    const float a = __ldg(mh[t] + k);
+                    const int k = k0 + 32 * s;
+                    ah[s][t] = k < D ? __ldg(mh[t] + k) : 0.f;
+                    al[s][t] = k < D ? __ldg(ml[t] + k) : 0.f;
+                }
+#pragma unroll
+            for (int s = 0; s < Z32_AHEAD; ++s) {
+                const int k = k0 + 32 * s;
+                const float b = k < D ? dh[k] : 0.f, bl = k < D ? dl[k] : 0.f;   // beyond D: adds nothing
+#pragma unroll
+                for (int t = 0; t < Z32_NJ; ++t) {
+                    const float a = ah[s][t];
                     const float h = __fmul_rn(a, b);
                     const float rr = __fmaf_rn(a, b, -h);                 // a b = h + rr exactly
                     const float tt = __fadd_rn(p[t], h);
                     const float bb = __fsub_rn(tt, p[t]);
                     const float q = __fadd_rn(__fsub_rn(p[t], __fsub_rn(tt, bb)), __fsub_rn(h, bb));   // p + h = tt + q
                     p[t] = tt;
-                    const float cross = __fmaf_rn(a, bl, __fmul_rn(__ldg(ml[t] + k), b));
+                    const float cross = __fmaf_rn(a, bl, __fmul_rn(al[s][t], b));
                     sc[t] = __fadd_rn(sc[t], __fadd_rn(__fadd_rn(q, rr), cross));
                     S[t] = __fmaf_rn(fabsf(a), fabsf(b), S[t]);
                 }
             }
+        }
 #pragma unroll
-            for (int t = 0; t < Z32_NJ; ++t) {
-                for (int off = 16; off > 0; off >>= 1) {       // every lane ends with the same values
-                    const float po = __shfl_xor_sync(0xffffffffu, p[t], off);
-                    const float so = __shfl_xor_sync(0xffffffffu, sc[t], off);
-                    const float Sq = __shfl_xor_sync(0xffffffffu, S[t], off);
-                    const float tt = __fadd_rn(p[t], po);
-                    const float bb = __fsub_rn(tt, p[t]);
-                    const float q = __fadd_rn(__fsub_rn(p[t], __fsub_rn(tt, bb)), __fsub_rn(po, bb));
-                    p[t] = tt;
-                    sc[t] = __fadd_rn(__fadd_rn(sc[t], so), q);
-                    S[t] = __fadd_rn(S[t], Sq);
-                }
-                if (lane == 0 && t < nv) {
-                    const float z = __fadd_rn(p[t], sc[t]);
-                    r.z32[o + j0 + t] = z;
-                    r.ez32[o + j0 + t] = __fmaf_ru(cS, S[t], 1.01f * U * fabsf(z));
-                }
+        for (int t = 0; t < Z32_NJ; ++t) {
+            for (int off = 16; off > 0; off >>= 1) {           // every lane ends with the same values
+                const float po = __shfl_xor_sync(0xffffffffu, p[t], off);
+                const float so = __shfl_xor_sync(0xffffffffu, sc[t], off);
+                const float Sq = __shfl_xor_sync(0xffffffffu, S[t], off);
+                const float tt = __fadd_rn(p[t], po);
+                const float bb = __fsub_rn(tt, p[t]);
+                const float q = __fadd_rn(__fsub_rn(p[t], __fsub_rn(tt, bb)), __fsub_rn(po, bb));
+                p[t] = tt;
+                sc[t] = __fadd_rn(__fadd_rn(sc[t], so), q);
+                S[t] = __fadd_rn(S[t], Sq);
+            }
+            if (lane == 0 && t < nv) {
+                const float z = __fadd_rn(p[t], sc[t]);
+                r.z32[o + j0 + t] = z;
+                r.ez32[o + j0 + t] = __fmaf_ru(cS, S[t], 1.01f * U * fabsf(z));
             }
         }
     }
