@@ -36,6 +36,11 @@
 // the whole-row code for narrow rows), whole runs with their arg-mins and
 // read-backs: 512 swarms, 1.19e8 variables, 150 generations, FP32 223 -> 167
 // ms; 40 swarms, 7.6e6 variables, 50 generations, FP64 21.9 -> 13.6 ms.
+// The interval's three sources chosen as pointers by the order, and FP32 terms
+// without a range check (a variable beyond D, where x = o = w = 0, adds zero; FP64 terms keep theirs,
+// the FP64 unit would work for the padding): 118.8 -> 111.2 ms of the FP32 run's
+// generations.  Loads of the next task's rows to L2 ahead, a slice loop unrolled
+// by 2 or 4, and 3 or 5 blocks an SM instead of 4 gained nothing.
 #pragma once
 #include <type_traits>
 
@@ -266,44 +271,42 @@ __global__ void __launch_bounds__(256, RowsBound<Pos, F32R>::min_blocks) bat_row
             const bool fg = d.Tg > 0xffffffffull, fp = d.Tp > 0xffffffffull, fw = d.Tw > 0xffffffffull;
             const uint32_t ctr3 = TAG_RHO | (d.sid << 8);
             const bool paper = d.order != 0;
-            const Pos* const gs = static_cast<const Pos*>(d.gbrow);
+            const Pos* const gs = static_cast<const Pos*>(d.gbrow) + 4 * lane_g;
             int s = 0;
             for (int r = 0; r < rounds; ++r) {
                 const int pi = r * gpw + sub;
+                // sources of the first, second and third interval (Eq. 2.1 as printed
+                // keeps x first and takes gBest third)
+                const Pos* const own = X + (int64_t)pi * Dp + 4 * lane_g;
+                const Pos* const src1 = paper ? own : gs;
+                const Pos* const src2 = P + (int64_t)pi * Dp + 4 * lane_g;
+                const Pos* const src3 = paper ? gs : own;
                 for (int q = 0; q < nq; ++q, ++s) {
                     const int c = lane_g + 32 * q;
                     uint32_t nf = 0;
                     if (c < nch && pi < np) {
-                        const int nvalid = min(4, D - 4 * c);
+                        const uint32_t valid = 4 * c + 4 <= D ? 15u : (1u << (D - 4 * c)) - 1u;
                         Pos x[4] = {Pos(0), Pos(0), Pos(0), Pos(0)};
                         if (g == 0) {
-                            nf = (1u << nvalid) - 1u;
+                            nf = valid;
                         } else {
-                            Pos xo[4], po[4], go[4];
-                            ld4(X + (int64_t)pi * Dp + 4 * c, xo);
-                            ld4(P + (int64_t)pi * Dp + 4 * c, po);
-                            ld4(gs + 4 * c, go);
-                            if (paper) {       // Eq. 2.1 as printed: keep x first, gBest third
-#pragma unroll
-                                for (int m = 0; m < 4; ++m) {
-                                    const Pos v = xo[m];
-                                    xo[m] = go[m];
-                                    go[m] = v;
-                                }
-                            }
+                            Pos v1[4], v2[4], v3[4];
+                            ld4(src1 + 128 * q, v1);
+                            ld4(src2 + 128 * q, v2);
+                            ld4(src3 + 128 * q, v3);
                             const uint4 rb = philox10(make_uint4((uint32_t)c, ibase + (uint32_t)pi, gg, ctr3), k0, k1);
                             bool ne = false;
 #pragma unroll
                             for (int m = 0; m < 4; ++m) {
                                 const uint32_t w = word_of(rb, m);
                                 const bool lg = w < Tg || fg, lp = w < Tp || fp, lw = w < Tw || fw;
-                                // a variable of the last interval holds its pBest value
-                                x[m] = lg ? go[m] : (lp || !lw) ? po[m] : xo[m];
+                                // a variable of the last interval holds its pBest value (beyond
+                                // D every source is 0)
+                                x[m] = lg ? v1[m] : (lp || !lw) ? v2[m] : v3[m];
                                 if (!lw) nf |= 1u << m;
-                                if (m >= nvalid) x[m] = Pos(0);   // padding (P holds 0 there)
-                                ne = ne || !same_bits(x[m], po[m]);
+                                ne = ne || !same_bits(x[m], v2[m]);
                             }
-                            nf &= (1u << nvalid) - 1u;
+                            nf &= valid;
                             if (ne || nf) neq |= 1u << r;
                         }
                         st4(stage + 4 * (32 * s + lane), x);
@@ -388,6 +391,7 @@ __global__ void __launch_bounds__(256, RowsBound<Pos, F32R>::min_blocks) bat_row
         };
         int n_acc = 0;          // warp-uniform
         const float* const o32 = d.o32;
+        const float* const w32 = d.w32;
         const double* const o64 = d.o64;
         double* const pf64 = d.pf64 + task.i0;
         uint32_t* const pver = d.pver + task.i0;
@@ -434,10 +438,7 @@ __global__ void __launch_bounds__(256, RowsBound<Pos, F32R>::min_blocks) bat_row
                             next = to_f32_trunc(__dsub_rn((double)stage[4 * slot + 4], __ldg(o64 + 4 * c + 4)));
                     }
 #pragma unroll
-                    for (int m = 0; m < 4; ++m) {
-                        if (4 * c + m >= D) break;
-                        rs.term(d.w32, D, 4 * c + m, z[m], m < 3 ? z[(m + 1) & 3] : next);
-                    }
+                    for (int m = 0; m < 4; ++m) rs.term(w32, D, 4 * c + m, z[m], m < 3 ? z[(m + 1) & 3] : next);
                 }
                 const Fit32 fr = rs.finish(G, D, nq);
                 const bool same = same_row(r, pi, valid);
