@@ -61,21 +61,20 @@ cudaError_t bat_rows_call(int variant, int fn, bool wide, int op, const BatRowsP
     return table[variant](fn, wide, op, p, grid, s, out);
 }
 
-// gBest of one instance per block: the lowest-index arg-min of the pBests
-// (FP32 mode: certain from the bounds, else the pBests that may be the
-// minimum made exact in FP64 and the exact arg-min taken), then the record,
-// log and gBest row; the last block advances the generation.
+// gBest of one instance per block: the lowest-index arg-min of the pBests, then
+// the record, log and gBest row.  FP32 bounds that leave more than one candidate
+// queue the candidates without an FP64 value for bat_exact, which evaluates those
+// of every swarm and finishes the swarm with its last one.  The last kernel's
+// last block advances the generation.
 //
 // Bound: latency (a few loads and block reductions per swarm).  Only the keys
 // are read and reduced -- FP32: the smallest and second-smallest lower bound,
 // the first's index, the smallest upper bound; FP64: the value as an integer
-// key and the index -- and the winner's other fields afterwards.  The
-// candidates of the exact pass are first collected by a scan over all
-// threads: one warp walking the particles one load at a time cost a load
-// latency per particle and warp.  40 swarms, FP64: 17 -> 10 us per launch; 512
-// swarms, FP32, generations 20-60: 171-308 -> 111-188 us.
-constexpr int ARGMIN_LIST = 2048;
-
+// key and the index -- and the winner's other fields afterwards: 40 swarms,
+// FP64, 17 -> 10 us per launch.  A swarm's candidates evaluated by its own block
+// kept one SM's FP64 unit busy (6 us a row of 1000 variables) and most others
+// idle: 512 swarms, FP32, generations 20-60: 111-188 -> 45-48 us for both
+// kernels, 118.8 -> 101.5 ms per 150 generations (1 to 2 candidates a swarm).
 struct BatKey {
     long long v;      // FP64: order_key of the value
     float l1, l2, mh; // FP32
@@ -156,19 +155,44 @@ __device__ double exact_row(const Hot& in, const Pos* row)
     }
 }
 
+// Copies the winner's row to the gBest row and writes the record and the log
+// (threads tid of nt); value: the winner's FP64 value when `exact`.
 template <class Pos, bool F32R>
-__global__ void __launch_bounds__(256, 4) bat_argmin(const InstDev* inst, const int32_t* ids, long long* gen,
-                                                  unsigned* ticket, BatCounters* cnt)
+__device__ __forceinline__ void finish_swarm(const InstDev& d, BatCounters& cnt, long long g, int wi, bool exact,
+                                             double value, unsigned extra, int tid, int nt)
+{
+    const Pos* src = static_cast<const Pos*>(d.P) + (int64_t)wi * d.Dp;
+    Pos* dst = static_cast<Pos*>(d.gbrow);
+    for (int q = tid; q < d.nchunks; q += nt) {
+        Pos v[4];
+        ld4(src + 4 * q, v);
+        st4(dst + 4 * q, v);
+    }
+    if (tid != 0) return;
+    Winner w;
+    w.idx = wi;
+    w.ver = d.pver[wi];
+    w.acc = cnt.acc;
+    w.rck = cnt.rck + extra;
+    const bool has = exact || (F32R && (d.pflag[wi] & 1u));
+    w.has64 = has ? 1 : 0;
+    w.f64 = exact ? value : has ? d.pf64[wi] : 0.0;
+    w.lo = exact ? f64_to_f32_rd(w.f64) : d.plo[wi];
+    w.hi = exact ? f64_to_f32_ru(w.f64) : d.phi[wi];
+    write_gbest(d, w, g);
+    cnt.acc = 0;
+    cnt.rck = 0;
+}
+
+template <class Pos, bool F32R>
+__global__ void __launch_bounds__(256) bat_argmin(const InstDev* inst, const int32_t* ids, BatCtl* ctl, BatCounters* cnt)
 {
     __shared__ BatKey sh[8];
-    __shared__ int list[F32R ? ARGMIN_LIST : 1];
-    __shared__ int n_list;
-    __shared__ unsigned long long extra;
+    __shared__ unsigned n_list, n_placed, first;
     const int k = ids[blockIdx.x];
     const InstDev& d = inst[k];
-    const long long g = *gen;
+    const long long g = ctl->gen;
     const int N = (int)d.N;
-    if (threadIdx.x == 0) extra = 0;
     const BatKey none = {LLONG_MAX, FLT_MAX, FLT_MAX, FLT_MAX, INT_MAX};
     BatKey c = none;
     for (int i = threadIdx.x; i < N; i += 256) {
@@ -184,99 +208,136 @@ __global__ void __launch_bounds__(256, 4) bat_argmin(const InstDev* inst, const 
     }
     BatKey b = key_block<F32R>(c, sh);
     bool exact = !F32R;
+    unsigned todo = 0;
     if constexpr (F32R) {
         if (b.l2 <= b.mh) {
-            // every pBest that can be the minimum gets its FP64 value, a list of
-            // candidates at a time, a warp per candidate
-            // (a converged swarm's candidates are mostly copies of the gBest row, whose
-            // value is known: they take it; a gBest put there by psso_set_gbest has a
-            // value of the caller's)
-            const Hot hin = hot_of(d);
-            const int lane = threadIdx.x & 31;
+            // the best of the FP64 values that are known, and the pBests without one
+            // that can be the minimum
             const float m = b.mh;
-            const Pos* const gr = static_cast<const Pos*>(d.gbrow);
-            const bool known = g > 0 && d.gb->has64 && d.gb->ver != 0xffffffffu;
-            const double gf = d.gb->f64;
-            for (int base = 0; base < N; base += ARGMIN_LIST) {
-                __syncthreads();
-                if (threadIdx.x == 0) n_list = 0;
-                __syncthreads();
-                const int top = min(N, base + ARGMIN_LIST);
-                for (int i = base + threadIdx.x; i < top; i += 256)
-                    if (d.plo[i] <= m && !(d.pflag[i] & 1u)) list[atomicAdd(&n_list, 1)] = i;
-                __syncthreads();
-                for (int e = threadIdx.x >> 5; e < n_list; e += 8) {
-                    const int i = list[e];
-                    const Pos* const row = static_cast<const Pos*>(d.P) + (int64_t)i * d.Dp;
-                    bool copy = known;
-                    for (int q = lane; q < d.nchunks && copy; q += 32) {
-                        Pos u[4], v[4];
-                        ld4(row + 4 * q, u);
-                        ld4(gr + 4 * q, v);
-#pragma unroll
-                        for (int t = 0; t < 4; ++t) copy = copy && same_bits(u[t], v[t]);
-                    }
-                    copy = __all_sync(0xffffffffu, copy);
-                    const double f = copy ? gf : exact_row<Pos>(hin, row);
-                    if (lane == 0) {
-                        d.pf64[i] = f;
-                        d.pflag[i] = 1u;
-                        d.plo[i] = f64_to_f32_rd(f);
-                        d.phi[i] = f64_to_f32_ru(f);
-                        atomicAdd(&extra, 1ull);
-                    }
-                }
-            }
+            if (threadIdx.x == 0) n_list = n_placed = 0;
             __syncthreads();
             BatKey e = none;
-            for (int i = threadIdx.x; i < N; i += 256)
+            unsigned mine = 0;
+            for (int i = threadIdx.x; i < N; i += 256) {
                 if (d.pflag[i] & 1u) {
                     BatKey q = none;
                     q.i = i;
                     q.v = order_key(d.pf64[i]);
                     e = key_merge<false>(e, q);
+                } else if (d.plo[i] <= m) {
+                    ++mine;
                 }
+            }
+            if (mine) atomicAdd(&n_list, mine);
             b = key_block<false>(e, sh);
             exact = true;
+            todo = n_list;
+            if (todo > 0) {
+                if (threadIdx.x == 0) {
+                    first = atomicAdd(&ctl->n_queue, todo);
+                    BatPend& pd = ctl->pend[blockIdx.x];
+                    pd.inst = k;
+                    pd.first = first;
+                    pd.n = todo;
+                    pd.left = todo;
+                    pd.key = b.v;
+                    pd.i = b.i;
+                }
+                __syncthreads();
+                for (int i = threadIdx.x; i < N; i += 256)
+                    if (!(d.pflag[i] & 1u) && d.plo[i] <= m)
+                        ctl->queue[first + atomicAdd(&n_placed, 1u)] = make_int2((int)blockIdx.x, i);
+            }
         }
     }
-    const int wi = b.i < N ? b.i : 0;        // no finite value at all: the first particle
-    const Pos* src = static_cast<const Pos*>(d.P) + (int64_t)wi * d.Dp;
-    Pos* dst = static_cast<Pos*>(d.gbrow);
-    for (int q = threadIdx.x; q < d.nchunks; q += 256) {
-        Pos v[4];
-        ld4(src + 4 * q, v);
-        st4(dst + 4 * q, v);
+    if (todo == 0) {
+        const int wi = b.i < N ? b.i : 0;    // no finite value at all: the first particle
+        finish_swarm<Pos, F32R>(d, cnt[k], g, wi, exact, exact ? d.pf64[wi] : 0.0, 0u, (int)threadIdx.x, 256);
     }
-    if (threadIdx.x == 0) {
-        Winner w;
-        w.idx = wi;
-        w.ver = d.pver[wi];
-        w.acc = cnt[k].acc;
-        w.rck = cnt[k].rck + extra;
-        const bool has = exact || (F32R && (d.pflag[wi] & 1u));
-        w.has64 = has ? 1 : 0;
-        w.f64 = has ? d.pf64[wi] : 0.0;
-        w.lo = exact ? f64_to_f32_rd(w.f64) : d.plo[wi];
-        w.hi = exact ? f64_to_f32_ru(w.f64) : d.phi[wi];
-        write_gbest(d, w, g);
-        cnt[k].acc = 0;
-        cnt[k].rck = 0;
+    if constexpr (!F32R) {
         // every block has read the generation before it takes a ticket
+        if (threadIdx.x == 0) {
+            __threadfence();
+            if (atomicInc(&ctl->ticket, gridDim.x - 1) == gridDim.x - 1) ctl->gen = g + 1;
+        }
+    }
+}
+
+// The queued candidates' FP64 values, a warp per candidate; neighbours in the
+// queue (one swarm's) go to different SMs.  The warp that completes a swarm's
+// last candidate takes the exact arg-min.
+template <class Pos>
+__global__ void __launch_bounds__(256, 4) bat_exact(const InstDev* inst, BatCtl* ctl, BatCounters* cnt)
+{
+    const int lane = threadIdx.x & 31;
+    const long long g = ctl->gen;
+    const unsigned n = ctl->n_queue;
+    for (unsigned e = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; e < n; e += 8 * gridDim.x) {
+        const int2 entry = ctl->queue[e];
+        BatPend& pd = ctl->pend[entry.x];
+        const int k = pd.inst, i = entry.y;
+        const InstDev& d = inst[k];
+        if (!PSSO_CHK(i >= 0 && i < d.N, CHK_BAT_ROW, i)) continue;
+        const Pos* const row = static_cast<const Pos*>(d.P) + (int64_t)i * d.Dp;
+        // (a converged swarm's candidates are mostly copies of the gBest row, whose
+        // value is known: they take it; a gBest put there by psso_set_gbest has a
+        // value of the caller's)
+        bool copy = g > 0 && d.gb->has64 && d.gb->ver != 0xffffffffu;
+        const double gf = d.gb->f64;
+        const Pos* const gr = static_cast<const Pos*>(d.gbrow);
+        for (int q = lane; q < d.nchunks && copy; q += 32) {
+            Pos u[4], v[4];
+            ld4(row + 4 * q, u);
+            ld4(gr + 4 * q, v);
+#pragma unroll
+            for (int t = 0; t < 4; ++t) copy = copy && same_bits(u[t], v[t]);
+        }
+        copy = __all_sync(0xffffffffu, copy);
+        const double f = copy ? gf : exact_row<Pos>(hot_of(d), row);
+        unsigned left = 0;
+        if (lane == 0) {
+            d.pf64[i] = f;
+            d.pflag[i] = 1u;
+            d.plo[i] = f64_to_f32_rd(f);
+            d.phi[i] = f64_to_f32_ru(f);
+            __threadfence();
+            left = atomicSub(&pd.left, 1u);
+        }
+        left = __shfl_sync(0xffffffffu, left, 0);
+        if (left != 1u) continue;
+        __threadfence();                     // the swarm's other values are visible
+        BatKey w = {pd.key, 0.f, 0.f, 0.f, pd.i};
+        for (unsigned q = lane; q < pd.n; q += 32) {
+            BatKey o = w;
+            o.i = ctl->queue[pd.first + q].y;
+            o.v = order_key(__ldcg(d.pf64 + o.i));
+            w = key_merge<false>(w, o);
+        }
+        w = key_warp<false>(w);
+        const int wi = w.i < (int)d.N ? w.i : 0;
+        finish_swarm<Pos, true>(d, cnt[k], g, wi, true, __ldcg(d.pf64 + wi), pd.n, lane, 32);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
         __threadfence();
-        if (atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1) *gen = g + 1;
+        if (atomicInc(&ctl->ticket, gridDim.x - 1) == gridDim.x - 1) {
+            ctl->n_queue = 0;
+            ctl->gen = g + 1;
+        }
     }
 }
 
 __global__ void bat_set(long long* gen, long long g) { *gen = g; }
 
-cudaError_t launch_bat_argmin(int variant, const InstDev* inst, const int32_t* ids, int n_ids, long long* gen,
-                              BatCounters* cnt, cudaStream_t s)
+cudaError_t launch_bat_argmin(int variant, const InstDev* inst, const int32_t* ids, int n_ids, BatCtl* ctl,
+                              BatCounters* cnt, int exact_grid, cudaStream_t s)
 {
-    unsigned* ticket = reinterpret_cast<unsigned*>(gen + 1);
-    if (variant == 0) bat_argmin<double, false><<<n_ids, 256, 0, s>>>(inst, ids, gen, ticket, cnt);
-    else if (variant == 1) bat_argmin<float, false><<<n_ids, 256, 0, s>>>(inst, ids, gen, ticket, cnt);
-    else bat_argmin<float, true><<<n_ids, 256, 0, s>>>(inst, ids, gen, ticket, cnt);
+    if (variant == 0) bat_argmin<double, false><<<n_ids, 256, 0, s>>>(inst, ids, ctl, cnt);
+    else if (variant == 1) bat_argmin<float, false><<<n_ids, 256, 0, s>>>(inst, ids, ctl, cnt);
+    else {
+        bat_argmin<float, true><<<n_ids, 256, 0, s>>>(inst, ids, ctl, cnt);
+        bat_exact<float><<<exact_grid, 256, 0, s>>>(inst, ctl, cnt);
+    }
     return cudaGetLastError();
 }
 

@@ -101,7 +101,8 @@ struct BatHost {
     int32_t* all_ids = nullptr;   // every batched instance (arg-min blocks)
     int32_t n_all = 0;
     BatCounters* cnt = nullptr;
-    long long* gen = nullptr;     // generation, then the arg-min's ticket word
+    BatCtl* ctl = nullptr;        // its first word is the generation
+    int exact_grid = 0;
     void* mem = nullptr;
     cudaGraphExec_t graph1 = nullptr, graphG = nullptr;
     static constexpr int GRAPH_GENS = 16;
@@ -599,12 +600,12 @@ psso_status launch(psso_ctx* h, int64_t g_begin, int64_t g_end)
         ++h->launches;
     }
     if (h->bat.n_all > 0) {
-        CUDA_TRY(launch_bat_set_gen(h->bat.gen, g_begin, h->stream));
+        CUDA_TRY(launch_bat_set_gen(&h->bat.ctl->gen, g_begin, h->stream));
         int64_t count = g_end - g_begin + 1;
         for (; count >= BatHost::GRAPH_GENS; count -= BatHost::GRAPH_GENS)
             CUDA_TRY(cudaGraphLaunch(h->bat.graphG, h->stream));
         for (; count > 0; --count) CUDA_TRY(cudaGraphLaunch(h->bat.graph1, h->stream));
-        h->launches += 1 + (int64_t)(h->bat.classes.size() + 1) * (g_end - g_begin + 1);
+        h->launches += 1 + (int64_t)(h->bat.classes.size() + bat_argmin_kernels(h->variant)) * (g_end - g_begin + 1);
     }
     // tensor-pipeline swarms: forked after everything above in stream order,
     // one side stream each (the handle's stream when there is no side stream)
@@ -731,10 +732,10 @@ cudaError_t enqueue_bat_generation(psso_ctx* h, cudaStream_t s, cudaEvent_t* ev 
     BatHost& B = h->bat;
     auto step = [&](const BatHost::Class& c, cudaStream_t st) {
         if (c.fn >= 0) {
-            BatRowsParams p{inst, c.tasks, c.n_tasks, B.gen, B.cnt};
+            BatRowsParams p{inst, c.tasks, c.n_tasks, &B.ctl->gen, B.cnt};
             return bat_rows_call(h->variant, c.fn, c.wide, 0, &p, c.grid, st, nullptr);
         }
-        BatParams p{inst, c.ids, c.first, c.n, c.G, c.total, B.gen, B.cnt};
+        BatParams p{inst, c.ids, c.first, c.n, c.G, c.total, &B.ctl->gen, B.cnt};
         return bat_call(h->variant, c.mc_index, 0, &p, c.grid, 256, st, nullptr);
     };
     int q = 0;
@@ -757,7 +758,7 @@ cudaError_t enqueue_bat_generation(psso_ctx* h, cudaStream_t s, cudaEvent_t* ev 
     for (size_t k = 0; branch && k + 1 < B.classes.size() && e == cudaSuccess; ++k)
         e = cudaStreamWaitEvent(s, B.join[k], 0);
     if (e != cudaSuccess) return e;
-    e = launch_bat_argmin(h->variant, inst, B.all_ids, B.n_all, B.gen, B.cnt, s);
+    e = launch_bat_argmin(h->variant, inst, B.all_ids, B.n_all, B.ctl, B.cnt, B.exact_grid, s);
     if (ev) cudaEventRecord(ev[q++], s);
     return e;
 }
@@ -836,8 +837,12 @@ psso_status setup_bat(psso_ctx* h)
         }
     }
     const size_t oall = take(all.size() * 4), ocnt = take(h->inst.size() * sizeof(BatCounters)),
-                 ogen = take(2 * sizeof(long long));
-    CUDA_TRY(cudaMalloc(&B.mem, bytes));
+                 octl = take(sizeof(BatCtl));
+    // the arg-min's queue, written before it is read: every particle at most once
+    int64_t particles = 0;
+    for (int32_t k : all) particles += h->inst[k].pr.N;
+    const size_t opend = align_up(bytes, 256), oqueue = align_up(opend + all.size() * sizeof(BatPend), 256);
+    CUDA_TRY(cudaMalloc(&B.mem, h->variant == V_F32R ? oqueue + (size_t)particles * sizeof(int2) : bytes));
     std::vector<char> host(bytes, 0);
     char* base = static_cast<char*>(B.mem);
     for (size_t c = 0; c < keys.size(); ++c) {
@@ -874,7 +879,12 @@ psso_status setup_bat(psso_ctx* h)
     std::memcpy(host.data() + oall, all.data(), all.size() * 4);
     B.all_ids = reinterpret_cast<int32_t*>(base + oall);
     B.cnt = reinterpret_cast<BatCounters*>(base + ocnt);
-    B.gen = reinterpret_cast<long long*>(base + ogen);
+    B.ctl = reinterpret_cast<BatCtl*>(base + octl);
+    BatCtl ctl{};
+    ctl.pend = reinterpret_cast<BatPend*>(base + opend);
+    ctl.queue = reinterpret_cast<int2*>(base + oqueue);
+    std::memcpy(host.data() + octl, &ctl, sizeof ctl);
+    B.exact_grid = 2 * prop.multiProcessorCount;
     CUDA_TRY(cudaMemcpy(B.mem, host.data(), bytes, cudaMemcpyHostToDevice));
     h->h2d += (int64_t)bytes;
     // side streams of the classes after the first (released by psso_destroy)
@@ -1506,7 +1516,7 @@ static psso_status time_bat_kernels(psso_ctx* h, int32_t generations, float* ms,
     std::vector<cudaEvent_t> ev(K + 1);
     for (auto& x : ev) CUDA_TRY(cudaEventCreate(&x));
     double acc[3] = {0.0, 0.0, 0.0};
-    cudaError_t e = launch_bat_set_gen(h->bat.gen, h->gen + 1, h->stream);
+    cudaError_t e = launch_bat_set_gen(&h->bat.ctl->gen, h->gen + 1, h->stream);
     for (int32_t g = 0; g < generations && e == cudaSuccess; ++g) {
         e = enqueue_bat_generation(h, h->stream, ev.data());
         if (e == cudaSuccess) e = cudaEventSynchronize(ev[K]);
@@ -1524,7 +1534,7 @@ static psso_status time_bat_kernels(psso_ctx* h, int32_t generations, float* ms,
         h->evals += I.pr.N * generations;
         h->updates += I.pr.N * I.pr.D * generations;
     }
-    h->launches += 1 + (int64_t)K * generations;
+    h->launches += 1 + (int64_t)(h->bat.classes.size() + bat_argmin_kernels(h->variant)) * generations;
     for (int q = 0; q < n; ++q) ms[q] = q < 3 ? (float)(acc[q] / generations) : 0.f;
     return PSSO_OK;
 }

@@ -206,11 +206,27 @@ struct BatRowsParams {
 // into *out); wide: rows of more than 128 variables.
 cudaError_t bat_rows_call(int variant, int fn, bool wide, int op, const BatRowsParams* p, int grid, cudaStream_t s,
                           int* out);
-// One block per listed instance: gBest arg-min (exact lowest index), record,
-// log, gBest row; the last block adds 1 to the generation counter (last kernel
-// of a generation).  gen: the counter, followed by a ticket word (zero).
-cudaError_t launch_bat_argmin(int variant, const InstDev* inst, const int32_t* ids, int n_ids, long long* gen,
-                              BatCounters* cnt, cudaStream_t s);
+// A swarm whose FP32 bounds leave several candidates: its entries of the queue,
+// and the best FP64 value that was known (integer key, particle).
+struct BatPend {
+    int32_t inst;
+    uint32_t first, n, left;
+    long long key;
+    int32_t i;
+};
+struct BatCtl {
+    long long gen;                 // generation being run
+    uint32_t ticket, n_queue;      // zero between generations
+    BatPend* pend;                 // [arg-min blocks]
+    int2* queue;                   // arg-min block, particle: [particles]
+};
+// gBest arg-min (exact lowest index), record, log and gBest row of every listed
+// instance, a block each; FP32 fitness: a second kernel (exact_grid blocks) for
+// the candidates that the bounds leave.  Then adds 1 to the generation (last
+// kernels of a generation).
+inline int bat_argmin_kernels(int variant) { return variant == 2 ? 2 : 1; }
+cudaError_t launch_bat_argmin(int variant, const InstDev* inst, const int32_t* ids, int n_ids, BatCtl* ctl,
+                              BatCounters* cnt, int exact_grid, cudaStream_t s);
 cudaError_t launch_bat_set_gen(long long* gen, long long g, cudaStream_t s);
 
 // Asynchronous flow (Alg. 1): control words of the grid barrier and of the
