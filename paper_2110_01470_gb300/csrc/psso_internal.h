@@ -157,7 +157,7 @@ struct KParams {
 // limit, 3 = maximum threads per block into *out.
 cudaError_t gen_call(int variant, int op, int mc_index, const KParams* p, int grid, int block,
                      size_t smem, cudaStream_t s, int* out);
-// What psso_best reads, packed for one copy: followed by the gBest row.
+// What psso_best reads, in one buffer: followed by the gBest row.
 struct BestPack {
     GBestDev gb;
     StatusDev status;
