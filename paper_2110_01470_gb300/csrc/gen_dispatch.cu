@@ -349,16 +349,16 @@ cudaError_t launch_bat_set_gen(long long* gen, long long g, cudaStream_t s)
 
 // One block: psso_best's answer in one buffer.  Reading the status, the record
 // and the row one by one, after a kernel and a synchronisation of its own for
-// the FP64 value, took 43 us a call; one copy of a packed answer 32 us; `out`, pinned
-// host memory that this kernel writes, 24 us.
+// the FP64 value, took 43 us a call; one kernel and one copy take 32 us.
+// (Written to pinned host memory by the kernel it is 24 us, but the memory costs
+// 150-400 us at psso_create.)
 template <class Pos>
-__global__ void __launch_bounds__(128) best_pack(const InstDev* inst, int k, const StatusDev* status, BestPack* out,
-                                                 int with_row)
+__global__ void __launch_bounds__(128) best_pack(const InstDev* inst, int k, const StatusDev* status, BestPack* out)
 {
     const InstDev& in = inst[k];
     const Pos* row = static_cast<const Pos*>(in.gbrow);
     Pos* dst = reinterpret_cast<Pos*>(out + 1);
-    for (int j = threadIdx.x; with_row && j < in.Dp; j += blockDim.x) dst[j] = row[j];
+    for (int j = threadIdx.x; j < in.Dp; j += blockDim.x) dst[j] = row[j];
     if (threadIdx.x >= 32) return;
     if (!in.gb->has64) {
         const double f = fit64_row<Pos>(hot_of(in), row, true);
@@ -374,11 +374,10 @@ __global__ void __launch_bounds__(128) best_pack(const InstDev* inst, int k, con
     }
 }
 
-cudaError_t launch_best(const InstDev* inst, int k, int lattice, const StatusDev* status, BestPack* out, int with_row,
-                        cudaStream_t s)
+cudaError_t launch_best(const InstDev* inst, int k, int lattice, const StatusDev* status, BestPack* out, cudaStream_t s)
 {
-    if (lattice == 1) best_pack<float><<<1, 128, 0, s>>>(inst, k, status, out, with_row);
-    else best_pack<double><<<1, 128, 0, s>>>(inst, k, status, out, with_row);
+    if (lattice == 1) best_pack<float><<<1, 128, 0, s>>>(inst, k, status, out);
+    else best_pack<double><<<1, 128, 0, s>>>(inst, k, status, out);
     return cudaGetLastError();
 }
 

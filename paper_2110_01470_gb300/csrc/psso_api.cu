@@ -134,8 +134,7 @@ struct psso_ctx {
     size_t smem = 0;
     char* arena = nullptr;
     size_t arena_size = 0, state_off = 0;
-    size_t off_instdev = 0, off_units = 0, off_block_first = 0, off_status = 0;
-    void* best = nullptr;           // pinned host memory: psso_best's answer (BestPack and the row)
+    size_t off_instdev = 0, off_units = 0, off_block_first = 0, off_status = 0, off_best = 0;
     int64_t gen = 0;
     int64_t evals = 0, updates = 0;
     int64_t h2d = 0, d2h = 0;
@@ -1127,16 +1126,15 @@ psso_status create_impl(const psso_problem* problems, int32_t count, const psso_
     h->off_units = take(sizeof(UnitDev) * h->units.size());
     h->off_block_first = take(sizeof(int32_t) * h->block_first.size());
     h->off_status = take(sizeof(StatusDev));
+    h->off_best = take(sizeof(BestPack) + (size_t)max_dp * h->pos_size);
     for (auto& I : h->inst)
         if (I.pr.fn == PSSO_GRIEWANK) I.off_tab = take((size_t)I.Dp * 8);
     h->state_off = align_up(off, 256);
     const size_t logcap = c.log_stride > 0 ? (size_t)c.log_capacity : 0;
     for (auto& I : h->inst) off = layout_state(h, I, I.R, off);
     h->arena_size = align_up(off, 256);
-    cudaError_t e = cudaHostAlloc(&h->best, sizeof(BestPack) + (size_t)max_dp * h->pos_size, cudaHostAllocDefault);
-    if (e == cudaSuccess) e = cudaMalloc(&h->arena, h->arena_size);
+    cudaError_t e = cudaMalloc(&h->arena, h->arena_size);
     if (e != cudaSuccess) {
-        if (h->best) cudaFreeHost(h->best);
         delete h;
         return fail(PSSO_ERR_OOM, std::string("cudaMalloc of the state arena: ") + cudaGetErrorString(e));
     }
@@ -1328,20 +1326,22 @@ psso_status psso_best(psso_handle h, int32_t instance, double* value, int64_t* i
     if (instance < 0 || instance >= (int32_t)h->inst.size()) return fail(PSSO_ERR_ARG, "instance out of range");
     CUDA_TRY(cudaSetDevice(h->device));
     const HostInst& I = h->inst[instance];
+    alignas(16) char buf[sizeof(BestPack) + 32 * MAX_CHUNKS_PER_LANE * 4 * sizeof(double)];
     const size_t n = sizeof(BestPack) + (row ? (size_t)I.Dp * h->pos_size : 0);
     CUDA_TRY(launch_best(reinterpret_cast<const InstDev*>(h->arena + h->off_instdev), instance, h->lattice,
                          reinterpret_cast<const StatusDev*>(h->arena + h->off_status),
-                         static_cast<BestPack*>(h->best), row ? 1 : 0, h->stream));
+                         reinterpret_cast<BestPack*>(h->arena + h->off_best), h->stream));
+    CUDA_TRY(cudaMemcpyAsync(buf, h->arena + h->off_best, n, cudaMemcpyDeviceToHost, h->stream));
     CUDA_TRY(cudaStreamSynchronize(h->stream));
     BestPack pk;
-    std::memcpy(&pk, h->best, sizeof pk);
+    std::memcpy(&pk, buf, sizeof pk);
     const psso_status st = check_status(h, pk.status);
     if (st != PSSO_OK) return st;
     h->d2h += (int64_t)n;
     if (value) *value = pk.gb.f64;
     if (index) *index = pk.gb.idx;
     if (row) {
-        const char* r = static_cast<const char*>(h->best) + sizeof pk;
+        const char* r = buf + sizeof pk;
         for (int64_t j = 0; j < I.pr.D; ++j)
             row[j] = h->pos_size == 8 ? reinterpret_cast<const double*>(r)[j] : (double)reinterpret_cast<const float*>(r)[j];
     }
@@ -1678,7 +1678,6 @@ void psso_destroy(psso_handle h)
     if (h->arena) {
         cudaSetDevice(h->device);
         cudaStreamSynchronize(h->stream);
-        cudaFreeHost(h->best);
         cudaFree(h->arena);
     }
     for (auto& I : h->inst) {

@@ -164,8 +164,7 @@ struct BestPack {
 };
 // Instance k's gBest (its FP64 value computed if only bounds are known), the
 // launch status and the row into out.
-cudaError_t launch_best(const InstDev* inst, int k, int lattice, const StatusDev* status, BestPack* out, int with_row,
-                        cudaStream_t s);
+cudaError_t launch_best(const InstDev* inst, int k, int lattice, const StatusDev* status, BestPack* out, cudaStream_t s);
 // Empties every instance's exchange records and clears its gBest record.
 cudaError_t launch_reset(const InstDev* inst, int n_inst, cudaStream_t s);
 
