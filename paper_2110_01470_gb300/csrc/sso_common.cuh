@@ -385,9 +385,9 @@ __device__ __forceinline__ double fit64_impl(const Hot& in, const Pos (&x)[MAXC]
 // once S / 4000 exceeds cut by more than that, f does, and S / 4000 is returned
 // without the product -- most of its 27 FP64 instructions per variable, and
 // most particles do not beat their pBest.
-template <class Pos, int MAXC>
-__device__ __noinline__ double fit64_extra(const Hot& in, const RowBuf<Pos, MAXC>& xb, int lane_g,
-                                           unsigned gmask, int G, double cut)
+template <class Pos, int MAXC, bool CUT>
+__device__ __forceinline__ double fit64_extra_impl(const Hot& in, const RowBuf<Pos, MAXC>& xb, int lane_g,
+                                                   unsigned gmask, int G, double cut)
 {
     const auto& x = xb.v;
     const int D = in.D, nch = in.nchunks, fn = in.fn;
@@ -449,7 +449,7 @@ __device__ __noinline__ double fit64_extra(const Hot& in, const RowBuf<Pos, MAXC
         const double low = __ddiv_rn(acc, 4000.0);
         // 1 - P >= -2^-40 for D <= 1024 factors of at most 1 + 2^-51 each; the
         // relative margin covers the last rounding (uniform over the group)
-        if (low > __fma_rn(fabs(cut), 0x1p-40, __dadd_rn(cut, 0x1p-30))) return low;
+        if (CUT && low > __fma_rn(fabs(cut), 0x1p-40, __dadd_rn(cut, 0x1p-30))) return low;
 #pragma unroll
         for (int q = 0; q < MAXC; ++q) {
             const int c = lane_g + 32 * q;
@@ -470,16 +470,29 @@ __device__ __noinline__ double fit64_extra(const Hot& in, const RowBuf<Pos, MAXC
 }
 
 template <class Pos, int MAXC>
+__device__ __noinline__ double fit64_extra(const Hot& in, const RowBuf<Pos, MAXC>& xb, int lane_g,
+                                           unsigned gmask, int G)
+{
+    return fit64_extra_impl<Pos, MAXC, false>(in, xb, lane_g, gmask, G, 0.0);
+}
+template <class Pos, int MAXC>
+__device__ __noinline__ double fit64_extra_cut(const Hot& in, const RowBuf<Pos, MAXC>& xb, int lane_g,
+                                               unsigned gmask, int G, double cut)
+{
+    return fit64_extra_impl<Pos, MAXC, true>(in, xb, lane_g, gmask, G, cut);
+}
+
+template <class Pos, int MAXC>
 __device__ __noinline__ double fit64_rotated(const Hot& in, const RowBuf<Pos, MAXC>& xb, int lane_g,
                                              unsigned gmask, int G)
 {
     return fit64_impl<Pos, MAXC, true>(in, xb.v, lane_g, gmask, G);
 }
 
-// cut: see fit64_extra (infinite: the value is needed).
-template <class Pos, int MAXC>
+// CUT, cut: see fit64_extra_impl.
+template <class Pos, int MAXC, bool CUT = false>
 __device__ __forceinline__ double fit64(const Hot& in, const Pos (&x)[MAXC][4], int lane_g, unsigned gmask,
-                                        int G, double cut = DBL_MAX)
+                                        int G, double cut = 0.0)
 {
     if (is_rotated(in.fn) || is_fp64_only(in.fn)) {
         RowBuf<Pos, MAXC> xb;
@@ -487,7 +500,10 @@ __device__ __forceinline__ double fit64(const Hot& in, const Pos (&x)[MAXC][4], 
         for (int q = 0; q < MAXC; ++q)
 #pragma unroll
             for (int m = 0; m < 4; ++m) xb.v[q][m] = x[q][m];
-        if (is_fp64_only(in.fn)) return fit64_extra<Pos, MAXC>(in, xb, lane_g, gmask, G, cut);
+        if (is_fp64_only(in.fn)) {
+            if constexpr (CUT) return fit64_extra_cut<Pos, MAXC>(in, xb, lane_g, gmask, G, cut);
+            else return fit64_extra<Pos, MAXC>(in, xb, lane_g, gmask, G);
+        }
         return fit64_rotated<Pos, MAXC>(in, xb, lane_g, gmask, G);
     }
     return fit64_impl<Pos, MAXC, false>(in, x, lane_g, gmask, G);
