@@ -68,3 +68,39 @@ def test_gradients_at_tile_edges(lib, fn, N, D):
     assert np.all(np.abs(f1 - f0) <= 1e-4 * np.maximum(np.abs(f0), 1e-3))
     big = np.abs(g0).max(axis=1, keepdims=True)
     assert np.all(np.abs(g1 - g0) <= 2e-4 * big + 1e-30)
+
+
+def test_gradients_under_capture(lib):
+    """The overlapped launches in a CUDA graph, replayed on new inputs: the same
+    bits as the calls."""
+    torch = pytest.importorskip("torch")
+    N, D = 700, 130
+    p = workload.problem("rot_ackley", 4, D, seed=3, lattice="f32", shift_range=(-1.0, 1.0))
+    dev = lambda a: torch.tensor(a, dtype=torch.float32, device="cuda")  # noqa: E731
+    rng = np.random.default_rng(1)
+    X, o, M, gf = dev(rng.uniform(-2, 2, (N, D))), dev(p["o"]), dev(p["M"]), dev(rng.standard_normal(N))
+    n = lib.psso_fitness_workspace_size("rot_ackley", N, D)
+    ws = torch.empty(n, dtype=torch.uint8, device="cuda")
+    f, g = torch.empty(N, device="cuda"), torch.empty(N, D, device="cuda")
+
+    def call():
+        s = torch.cuda.current_stream().cuda_stream
+        args = ("rot_ackley", N, D, X.data_ptr(), o.data_ptr(), None, M.data_ptr())
+        lib.psso_fitness_forward_ws(*args, f.data_ptr(), ws.data_ptr(), n, s)
+        lib.psso_fitness_backward_ws(*args, gf.data_ptr(), g.data_ptr(), ws.data_ptr(), n, s)
+
+    call()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        call()
+    for k in range(3):
+        X.copy_(dev(rng.uniform(-2, 2, (N, D))))
+        gf.copy_(dev(rng.standard_normal(N)))
+        graph.replay()
+        torch.cuda.synchronize()
+        got = f.clone(), g.clone()
+        f.zero_(), g.zero_()
+        call()
+        torch.cuda.synchronize()
+        assert torch.equal(got[0], f) and torch.equal(got[1], g), k
