@@ -148,9 +148,11 @@ typedef struct {
 typedef struct {
     int32_t precision;          /* psso_precision                                   */
     int32_t threads_per_block;  /* 0 = 256; a multiple of 32 in [64, 512]           */
-    int32_t single_block_max;   /* 0 = auto: swarms of at most this many particle
-                                   passes run in one block with no cross-block
-                                   exchange; -1 = never                            */
+    int32_t single_block_max;   /* swarms of at most this many particle passes run
+                                   in one block with no cross-block exchange; 0 =
+                                   auto: 4 passes, but a single swarm of more than
+                                   one warp (FP64 fitness; FP32: two) runs as
+                                   pipelined blocks; -1 = never                     */
     int32_t log_stride;         /* log every log_stride-th generation (0 = off)     */
     int64_t log_capacity;       /* log entries kept per instance (ring)             */
     int64_t spin_limit;         /* polls of a cross-block wait before the run fails
@@ -176,11 +178,12 @@ typedef struct {
                                    fails with PSSO_ERR_UNSUPPORTED (always)        */
     int32_t batch_stream;       /* handles of many swarms: 0 = auto (16 or more
                                    swarms that are not on the tensor-core pipeline
-                                   run each generation as one kernel per row-width
-                                   class over every particle of every swarm, then
-                                   one block per swarm for the gBest, replayed as
-                                   CUDA graphs); 1 = always; -1 = never (the
-                                   persistent kernel)                              */
+                                   run each generation as one kernel per class of
+                                   swarms (function, row width) over every particle
+                                   of the class, then one block per swarm for the
+                                   gBest (FP32: and a kernel for the candidates that
+                                   need FP64), replayed as CUDA graphs); 1 = always;
+                                   -1 = never (the persistent kernel)               */
     int32_t batch_blocks_per_sm;/* batched pipeline: resident blocks per SM of each
                                    step kernel's grid (0 = the occupancy maximum;
                                    larger values are clamped to it)                 */
@@ -289,9 +292,10 @@ psso_status psso_best(psso_handle h, int32_t instance, double* value, int64_t* i
  * psso_set_gbest replaces the gBest the next generation searches with: FP64
  * value, an index (stored as given; any label), and the row (host, D values
  * inside [lb, ub]; floats for the F32 lattice).  Synchronises.  Valid for
- * shard handles and single-block, tensor-pipeline or batched-pipeline
- * instances; PSSO_ERR_UNSUPPORTED for an instance spread over several blocks
- * or the asynchronous flow. */
+ * shard handles and for instances that fit one block (also when they run as
+ * pipelined blocks) or run on the tensor or batched pipeline;
+ * PSSO_ERR_UNSUPPORTED for a larger instance spread over several blocks or the
+ * asynchronous flow. */
 psso_status psso_create_shard(const psso_problem* problem, int64_t first, int64_t count,
                               const psso_config* cfg, psso_handle* out);
 psso_status psso_set_gbest(psso_handle h, int32_t instance, double value, int64_t index, const double* row);
@@ -454,8 +458,8 @@ psso_status psso_rotate(int64_t N, int64_t D, const float* X, const float* shift
  * decisions, arg-min, FP64 rotation and decisions of arg-min candidates,
  * gBest); n >= 11.  On a handle whose swarms all run on the batched
  * pipeline it times that pipeline instead, writing the mean per-generation
- * duration of its streaming step kernels (rows over 128 variables), of its
- * other step kernels and of its arg-min kernel to ms[0..2] (n >= 3; instance
+ * duration of its step kernels for rows over 128 variables, of its other step
+ * kernels and of its arg-min kernels to ms[0..2] (n >= 3; instance
  * is ignored).  The paper has no counterpart.  Synchronises.
  * PSSO_ERR_UNSUPPORTED for a swarm on the persistent kernel. */
 psso_status psso_time_kernels(psso_handle h, int32_t instance, int32_t generations, float* ms, int32_t n);
