@@ -108,8 +108,9 @@ extern "C" psso_status psso_evaluate(psso_fn fn, int64_t N, int64_t D, const dou
         if (f32 && (double)(float)o64[j] != o64[j])
             return bad(PSSO_ERR_ARG, "psso_evaluate: FP32 needs a float-exact shift");
         o32[j] = (float)o64[j];
-        // Griewank: the divisors of its cosines (eval64)
-        w64[j] = weights ? weights[j] : fn == PSSO_GRIEWANK ? std::sqrt((double)(j + 1)) : 0.0;
+        // Griewank: the divisors of its cosines (eval64); weights given to it are ignored,
+        // as every function but the ellipsoids does
+        w64[j] = fn == PSSO_GRIEWANK ? std::sqrt((double)(j + 1)) : weights ? weights[j] : 0.0;
         w32[j] = (float)w64[j];
     }
     const size_t nM = rot ? (size_t)D * D : 0;
