@@ -226,6 +226,15 @@ __host__ __device__ constexpr size_t rows_smem_per_warp()
     return (size_t)ROWS_SLICES * 128 * sizeof(Pos) + ROWS_SLICES * 32 * sizeof(uint32_t);
 }
 
+// The FP32 filter decides only above this lower bound.  E is relative to the
+// sums, so each sum must stand clear of the denormal floats, where a square or a
+// partial sum errs by up to 2^-149 absolutely.  Rastrigin and Rosenbrock: the
+// value is the sum itself; 1024 such errors are below 2^-39 of 1e-30.  Ackley's
+// value is at most 4 sqrt(s / D) + 54 s / D in s = sum z^2, so above 1e-16 s / D
+// exceeds 6e-34: an error of 2^-149 a term is below 2^-38 of it.  (With 1e-30 for
+// Ackley too, s of 1e-40 passed, whose squares had lost most of their bits.)
+template <int FN> constexpr float FILTER_MIN = FN == FN_ACKLEY ? 1e-16f : 1e-30f;
+
 // Blocks of 8 warps per SM the kernel is compiled for.
 template <class Pos, bool F32R> struct RowsBound { static constexpr int min_blocks = F32R ? 4 : 3; };
 
@@ -468,7 +477,7 @@ __global__ void __launch_bounds__(256, RowsBound<Pos, F32R>::min_blocks) bat_row
                     // f32 - E above the pBest's value: rejected.  A NaN bound, and
                     // sums so small that the floats' range ends, go to FP64.
                     const bool keep = valid && same && !is_nan_bits(pf);
-                    const bool reject = g > 0 && lo0 > 1e-30f && (double)lo0 > pf;
+                    const bool reject = g > 0 && lo0 > FILTER_MIN<FN> && (double)lo0 > pf;
                     const bool need = valid && !keep && !reject;
                     if (keep && lane_g == 0) pver[pi] = gg;
                     n_acc += __popc(__ballot_sync(0xffffffffu, keep && lane_g == 0));
