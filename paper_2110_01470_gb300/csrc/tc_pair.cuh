@@ -27,7 +27,9 @@
 // owns the tensor memory, warps 2..9 run the epilogue.  Barriers: full[s]
 // (leader: one arrival and both CTAs' bytes), empty[s] (both CTAs: committed by
 // the leader's MMAs), tfull (both CTAs: a tile's MMAs are complete), tempty
-// (leader: the 16 epilogue warps of the pair).  Every wait is bounded.
+// (leader: the 16 epilogue warps of the pair).  Every wait on them is bounded;
+// the barriers without a limit (the two warps of a lane quarter, the block, the
+// cluster) are reached by all their threads whether a wait ran out or not.
 #pragma once
 #include "pdl.cuh"
 #include "tc_gemm.cuh"
@@ -107,6 +109,24 @@ __device__ __forceinline__ float4 pair_exchange(float4 v, int c0, float4* xch)
     if (c0 == 0) o = *xch;
     asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory");
     return o;
+}
+
+// Whether ok holds in all threads of the two warps of a lane quarter (the same
+// barrier; both warps come here for every tile, after a wait with a limit).
+__device__ __forceinline__ bool quarter_all(bool ok)
+{
+    const int id = 1 + ((threadIdx.x >> 5) & 3);
+    uint32_t r;
+    __syncwarp();
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.u32 q, %1, 0;\n\t"
+        "bar.red.and.pred p, %2, 64, q;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(r)
+        : "r"((uint32_t)ok), "r"(id)
+        : "memory");
+    return r != 0;
 }
 
 // The tile walk of one pair.
@@ -286,9 +306,11 @@ __device__ __forceinline__ bool gemm_pair(const CUtensorMap* tmA, const CUtensor
             int tm, g0, ng;
             tiles.item(k, tm, g0, ng);
             if (ng == 0) continue;
+            // the two warps of a lane quarter go on or leave together: each times its
+            // own wait, and pair_exchange waits for the other warp without a limit
             const bool ok = mbar_wait(tfull, (uint32_t)(tl & 1));
             ++tl;
-            if (!__all_sync(0xffffffffu, ok)) {
+            if (!quarter_all(ok)) {
                 failed = 1;
                 break;
             }
