@@ -293,8 +293,6 @@ __device__ __forceinline__ bool gemm_pair(const CUtensorMap* tmA, const CUtensor
             // every MMA issued by this thread has completed once `done` fires
             mma_commit_pair(done);
         }
-        // both CTAs: the leader's commits have all arrived here
-        if (lane == 0 && !mbar_wait(done, 0u)) failed = 1;
     } else {
         // epilogue: warp w reads tensor-memory lanes 32 (w % 4) .. + 31 (one row
         // per lane), the 64-column group (w - 2) / 4 of the tile
@@ -324,6 +322,12 @@ __device__ __forceinline__ bool gemm_pair(const CUtensorMap* tmA, const CUtensor
             epi.compute(ng == 2 ? 0 : half, ng, &xch[32 * qtr + lane]);
         }
     }
+    __syncwarp();
+    __syncthreads();              // the CTA's roles have ended: each has waited for one step at a time
+    // both CTAs: the leader's commits have all arrived here.  Waited for from here on
+    // only: from the start of the kernel, the limit of this one wait would bound the
+    // peer CTA's whole GEMM.
+    if (warp == 1 && lane == 0 && !mbar_wait(done, 0u)) failed = 1;
     __syncwarp();
     if (vload(failed)) {          // let this CTA's copies in flight land before it gives up its memory
         const long long t0 = clock64();

@@ -6,7 +6,8 @@ to exchange sums, so neither may reach it when the other has left.  Each times
 its own wait for a tile: near the limit one may run out while the other's
 succeeds.  The model gives every wait a random outcome and checks that both
 warps always finish, whatever the interleaving and the kinds of the items
-(128 columns: no exchange; 64 columns: two barriers)."""
+(128 columns: no exchange; 64 columns: two barriers).  The second model looks at how long a
+correct run waits."""
 import random
 
 import pytest
@@ -84,3 +85,24 @@ def test_the_model_sees_a_warp_that_leaves_alone():
     with pytest.raises(AssertionError):
         for _ in range(500):
             run_quarter([2, 1, 1], rng, agree=False)
+
+
+def longest_wait(ntiles, tile_time, after_roles):
+    """Longest wait of the peer CTA in a run whose tiles complete every
+    `tile_time`: its epilogue waits tile by tile, its warp 1 for the leader's
+    last commit, from the end of the CTA's roles or from the kernel's start."""
+    finished = [(t + 1) * tile_time for t in range(ntiles)]
+    waits, now = [], 0.0
+    for t in finished:
+        waits.append(t - now)
+        now = max(now, t)
+    last_commit = finished[-1]
+    waits.append(max(0.0, last_commit - (now if after_roles else 0.0)))
+    return max(waits)
+
+
+@pytest.mark.parametrize("ntiles", [1, 7, 1000])
+def test_no_wait_spans_more_than_one_tile(ntiles):
+    """The limit of a wait is one for a step, however many tiles a call has."""
+    assert longest_wait(ntiles, 0.25, after_roles=True) <= 0.25
+    assert longest_wait(1000, 0.25, after_roles=False) > 2.0
