@@ -150,9 +150,9 @@ typedef struct {
     int32_t threads_per_block;  /* 0 = 256; a multiple of 32 in [64, 512]           */
     int32_t single_block_max;   /* swarms of at most this many particle passes run
                                    in one block with no cross-block exchange; 0 =
-                                   auto: 4 passes, but a single swarm of more than
-                                   one warp (FP64 fitness; FP32: two) runs as
-                                   pipelined blocks; -1 = never                     */
+                                   auto: 4 passes, but a single swarm may run as
+                                   pipelined blocks where that is faster, unless
+                                   threads_per_block is given; -1 = never           */
     int32_t log_stride;         /* log every log_stride-th generation (0 = off)     */
     int64_t log_capacity;       /* log entries kept per instance (ring)             */
     int64_t spin_limit;         /* polls of a cross-block wait before the run fails

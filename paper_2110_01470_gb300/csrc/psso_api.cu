@@ -217,15 +217,26 @@ psso_status check_problem(const psso_problem& pr, int precision, int idx)
     return PSSO_OK;
 }
 
-// A single swarm of more warps (of 32 / G particles) than this, no block limit
-// given, is spread over pipelined blocks of one compute warp each instead of
-// running its up to four passes in one block.  Measured (us per generation,
-// one block / spread), sphere: FP64 N = 8, D = 30 (2 warps) 6.1 / 3.6, N = 100,
-// D = 30 (25 warps) 16.7 / 3.9; Ackley: FP64 N = 16, D = 10 (2) 11.3 / 11.2, N =
-// 100, D = 30 51.6 / 9.8; FP32 N = 16, D = 10 (2) 11.3 / 11.7, N = 32, D = 10 (4)
-// 14.4 / 13.5, N = 100, D = 30 15.5 / 7.9.  One block needs no exchange, but its
-// SM's FP64 unit (or issue slots) serves every particle.
-constexpr int ONE_BLOCK_WARPS_F64 = 1, ONE_BLOCK_WARPS_F32 = 2;
+// Whether a swarm of at most four passes of a default block (`groups` warps of
+// 32 / G particles) is spread over pipelined blocks of one compute warp each
+// instead, no launch shape given.  One block needs no exchange, but its SM's
+// FP64 unit (or issue slots) serves every particle.  Measured: time in one block
+// over time spread, the smallest of sphere, Rastrigin, Rosenbrock and Ackley in
+// both interval orders, runs of 2000 generations.
+//   FP64  4 warps and fewer at D <= 14: 0.86 (Ackley, N = 96, D = 3) .. 1.8; D >= 16 from 2
+//         warps on: 1.11 (N = 12, D = 16) .. 1.8; more than 4 warps: 1.12 (N = 80, D = 5) .. 7.4.
+//   FP32  a converged swarm leaves several candidates in most generations; their
+//         FP64 values then cost the spread form a second exchange, one block a
+//         few microseconds.  Such generations come late in wide rows: D >= 64: 1.11
+//         (N = 6) .. 4.  The fourth pass pays for them: 29 to 32 warps: 0.99 (N = 128,
+//         D = 32) .. 2.7.  Below: 0.70 (N = 12, D = 45), 0.72 (N = 64, D = 20), 0.77 (N = 64,
+//         D = 16), 0.89 (N = 100, D = 30), and from N = 128 on (D <= 16) 1.04 .. 2.0 in the
+//         default order against 0.49 .. 1.4 in the paper's order, which converges sooner.
+bool spread_small(int variant, int64_t N, int64_t D, int64_t groups, bool paper_order)
+{
+    if (variant != V_F32R) return groups > 4 || (groups > 1 && D > 14);
+    return groups > 2 && (D >= 64 || groups > 28 || (N >= 128 && !paper_order));
+}
 
 // Picks blocks per instance and assigns units to blocks.
 psso_status plan(psso_ctx* h)
@@ -280,8 +291,10 @@ psso_status plan(psso_ctx* h)
         const HostInst& I = h->inst[only];
         const int gpw = 32 / I.G;
         const int64_t groups = (I.pr.N + gpw - 1) / gpw;
-        const bool spread = h->cfg.single_block_max == 0 &&
-                            groups > (h->variant == V_F32R ? ONE_BLOCK_WARPS_F32 : ONE_BLOCK_WARPS_F64);
+        // (a given block size keeps the swarm in one block, so that the tuner can
+        // choose between both forms)
+        const bool spread = h->cfg.single_block_max == 0 && h->cfg.threads_per_block == 0 &&
+                            spread_small(h->variant, I.pr.N, I.pr.D, groups, I.pr.order == PSSO_ORDER_PAPER);
         if (!I.one_block || spread) {
             // at most 128 blocks: each lane of the control warp then polls <= 4
             // records, all in flight at once
