@@ -78,6 +78,8 @@ struct HostInst {
     size_t off_tab = 0;           // Griewank: sqrt(j + 1), j < D (a constant, not part of the saved state)
     bool one_block = false;       // at most four passes of a default block: psso_set_gbest takes it
                                   // whether it runs in one block or, pipelined, in several
+    int alt_grid = 0, alt_block = 0;   // such a swarm with the default block size: the launch shape of the
+                                  // form that it does not run in (psso_load takes both forms' states)
     int64_t i_base = 0;           // shard of a larger swarm: index of its first particle
     bool tc = false;              // generations run by the tensor-core pipeline
     bool bp = false;              // generations run by the batched throughput pipeline
@@ -288,19 +290,27 @@ psso_status plan(psso_ctx* h)
         I.one_block = (I.pr.N + (int64_t)nw * gpw - 1) / ((int64_t)nw * gpw) <= sbm;
     }
     if (n_kernel == 1 && h->cfg.pipeline != 2) {
-        const HostInst& I = h->inst[only];
+        HostInst& I = h->inst[only];
         const int gpw = 32 / I.G;
         const int64_t groups = (I.pr.N + gpw - 1) / gpw;
+        // at most 128 blocks: each lane of the control warp then polls <= 4
+        // records, all in flight at once
+        const int64_t blocks_cap = std::min<int64_t>(prop.multiProcessorCount, 128);
+        const int cw_auto = (int)std::min<int64_t>((groups + blocks_cap - 1) / blocks_cap, max_threads / 32 - 1);
         // (a given block size keeps the swarm in one block, so that the tuner can
         // choose between both forms)
-        const bool spread = h->cfg.single_block_max == 0 && h->cfg.threads_per_block == 0 &&
+        const bool spread = I.one_block && cw_auto >= 1 && h->cfg.single_block_max == 0 &&
+                            h->cfg.threads_per_block == 0 &&
                             spread_small(h->variant, I.pr.N, I.pr.D, groups, I.pr.order == PSSO_ORDER_PAPER);
+        if (spread) {
+            I.alt_grid = 1;
+            I.alt_block = h->block;
+        } else if (I.one_block && cw_auto >= 1 && h->block == std::min(256, max_threads)) {
+            I.alt_grid = (int)((groups + cw_auto - 1) / cw_auto);
+            I.alt_block = 32 * (cw_auto + 1);
+        }
         if (!I.one_block || spread) {
-            // at most 128 blocks: each lane of the control warp then polls <= 4
-            // records, all in flight at once
-            const int64_t blocks_cap = std::min<int64_t>(prop.multiProcessorCount, 128);
-            int cw = (int)std::min<int64_t>((groups + blocks_cap - 1) / blocks_cap, max_threads / 32 - 1);
-            if (h->cfg.threads_per_block != 0) cw = h->block / 32 - 1;
+            const int cw = h->cfg.threads_per_block != 0 ? h->block / 32 - 1 : cw_auto;
             if (cw >= 1) {
                 pipe = true;
                 h->block = 32 * (cw + 1);
@@ -1626,14 +1636,14 @@ psso_status psso_save(psso_handle h, void* buf, size_t cap, size_t* n)
     return PSSO_OK;
 }
 
-// A state saved by a one-block run of a swarm that this handle spreads over
-// several blocks: everything but the exchange records is copied
-// by field, the records are made from the gBest.
-static psso_status load_one_block(psso_ctx* h, const SaveHeader& hd, const char* state)
+// A small swarm's state saved by a handle that runs it in the other form (one
+// block, or pipelined blocks): everything but the exchange records is copied by
+// field, the records are made from the gBest.
+static psso_status load_other_form(psso_ctx* h, const SaveHeader& hd, const char* state)
 {
     const HostInst& I = h->inst[0];
     HostInst J = I;
-    layout_state(h, J, 1, h->state_off);
+    layout_state(h, J, hd.grid, h->state_off);
     auto src = [&](size_t off) { return state + (off - h->state_off); };
     auto put = [&](size_t to, size_t from, size_t bytes) {
         return cudaMemcpy(h->arena + to, src(from), bytes, cudaMemcpyHostToDevice);
@@ -1643,6 +1653,7 @@ static psso_status load_one_block(psso_ctx* h, const SaveHeader& hd, const char*
     CUDA_TRY(put(I.off_gb, J.off_gb, sizeof(GBestDev)));
     CUDA_TRY(put(I.off_gbrow, J.off_gbrow, row));
     CUDA_TRY(put(I.off_log, J.off_log, J.off_o64 - J.off_log));
+    if (I.R == 1) return PSSO_OK;
     GBestDev gb;
     std::memcpy(&gb, src(J.off_gb), sizeof gb);
     return publish_gbest(h, I, hd.gen, gb, src(J.off_gbrow));
@@ -1657,19 +1668,19 @@ psso_status psso_load(psso_handle h, const void* buf, size_t n)
     const char* data = static_cast<const char*>(buf) + sizeof hd;
     const size_t state = h->arena_size - h->state_off;
     const bool same = hd.state_bytes == (int64_t)state && hd.grid == h->grid && hd.block == h->block;
-    bool one_block = false;
-    if (!same && h->inst.size() == 1 && h->inst[0].one_block && h->inst[0].R > 1 && hd.grid == 1 &&
-        hd.block == (h->cfg.threads_per_block ? h->cfg.threads_per_block : 256)) {
+    bool other_form = false;
+    if (!same && h->inst.size() == 1 && h->inst[0].alt_grid > 0 && hd.grid == h->inst[0].alt_grid &&
+        hd.block == h->inst[0].alt_block && hd.gen >= 0 && hd.gen <= 0xfffffff0LL) {
         HostInst J = h->inst[0];
-        one_block = hd.state_bytes == (int64_t)(align_up(layout_state(h, J, 1, h->state_off), 256) - h->state_off);
+        other_form = hd.state_bytes == (int64_t)(align_up(layout_state(h, J, hd.grid, h->state_off), 256) - h->state_off);
     }
-    if (std::memcmp(hd.magic, "PSSOST01", 8) != 0 || !(same || one_block) ||
+    if (std::memcmp(hd.magic, "PSSOST01", 8) != 0 || !(same || other_form) ||
         n != sizeof hd + (size_t)hd.state_bytes || hd.n_inst != (int32_t)h->inst.size() || hd.variant != h->variant)
         return fail(PSSO_ERR_ARG, "state was saved from a handle with other problems or launch shape");
     CUDA_TRY(cudaSetDevice(h->device));
     CUDA_TRY(cudaStreamSynchronize(h->stream));
-    if (one_block) {
-        const psso_status st = load_one_block(h, hd, data);
+    if (other_form) {
+        const psso_status st = load_other_form(h, hd, data);
         if (st != PSSO_OK) return st;
     } else {
         CUDA_TRY(cudaMemcpy(h->arena + h->state_off, data, state, cudaMemcpyHostToDevice));
