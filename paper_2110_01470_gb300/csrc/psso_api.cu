@@ -138,6 +138,7 @@ struct psso_ctx {
     size_t arena_size = 0, state_off = 0;
     size_t off_instdev = 0, off_units = 0, off_block_first = 0, off_status = 0, off_best = 0;
     int64_t gen = 0;
+    bool rows_diverged = false;   // the exchange rows may be those of a run that psso_reset does not repeat
     int64_t evals = 0, updates = 0;
     int64_t h2d = 0, d2h = 0;
     int64_t launches = 0;       // kernels this handle enqueued (graph nodes included)
@@ -485,6 +486,18 @@ size_t layout_state(const psso_ctx* h, HostInst& I, int R, size_t off)
     I.off_M64 = take(I.M.size() * 8);
     I.off_M32 = take(I.M.size() * 8);   // float(M), then float(M - float(M))
     return off;
+}
+
+// Empties a multi-block instance's exchange rows: no generation's tag is left in
+// them.  A reader takes a row by its tags alone, and its writer publishes it
+// after the record that names it, so rows must not hold a tag that their run has
+// yet to use: the zeros of new memory are generation 0's, and those of a run that
+// went another way (rows_diverged) are the next run's.  (The rows of the same
+// run, started again by psso_reset, are the ones it will write.)
+cudaError_t clear_rows(const psso_ctx* h, const HostInst& I, cudaStream_t s)
+{
+    return cudaMemsetAsync(h->arena + I.off_grow, 0xff,
+                           SLOTS * (size_t)I.R * I.Dp * (h->pos_size / 4) * 8, s);
 }
 
 // Several blocks: the exchange records and row of generation g rewritten so
@@ -1183,6 +1196,7 @@ psso_status create_impl(const psso_problem* problems, int32_t count, const psso_
         const size_t rb = SLOTS * (size_t)I.R * REC_WORDS * 8;
         e = cudaMemsetAsync(h->arena + I.off_rec, 0xff, rb, h->stream);
         if (e == cudaSuccess) e = cudaMemsetAsync(h->arena + I.off_rec2, 0xff, rb, h->stream);
+        if (e == cudaSuccess && I.R > 1) e = clear_rows(h, I, h->stream);
         if (e == cudaSuccess && logcap)
             e = cudaMemsetAsync(h->arena + I.off_log, 0xff, logcap * sizeof(LogDev), h->stream);
         const size_t nd = (size_t)I.pr.D;
@@ -1309,6 +1323,10 @@ psso_status psso_reset(psso_handle h)
     for (auto& I : h->inst)
         if (I.tc) CUDA_TRY(cudaMemsetAsync(&I.rh.dev.ctl->status, 0, sizeof(int), h->stream));
     if (h->actl) CUDA_TRY(cudaMemsetAsync(h->actl, 0, sizeof(AsyncCtl), h->stream));
+    if (h->rows_diverged)
+        for (const auto& I : h->inst)
+            if (I.R > 1) CUDA_TRY(clear_rows(h, I, h->stream));
+    h->rows_diverged = false;
     psso_status st = launch(h, 0, 0);
     if (st != PSSO_OK) return st;
     h->gen = 0;
@@ -1408,6 +1426,7 @@ psso_status psso_set_gbest(psso_handle h, int32_t instance, double value, int64_
     CUDA_TRY(cudaMemcpy(h->arena + I.off_gbrow, buf.data(), (size_t)I.Dp * h->pos_size, cudaMemcpyHostToDevice));
     CUDA_TRY(cudaMemcpy(h->arena + I.off_gb, &gb, sizeof gb, cudaMemcpyHostToDevice));
     h->h2d += (int64_t)((size_t)I.Dp * h->pos_size + sizeof gb);
+    h->rows_diverged = true;
     if (I.R > 1) return publish_gbest(h, I, h->gen, gb, buf.data());
     return PSSO_OK;
 }
@@ -1520,6 +1539,7 @@ psso_status psso_polish(psso_handle h, int32_t instance, int32_t steps, double l
     if (I.R > 1)
         for (const auto& u : h->units)
             if (u.inst == instance && before.idx >= u.i0 && before.idx < u.i1) owner = u.rank;
+    h->rows_diverged = true;
     CUDA_TRY(launch_polish(reinterpret_cast<const InstDev*>(h->arena + h->off_instdev), instance, h->lattice,
                            owner, h->gen, steps, (float)lr, h->stream));
     GBestDev after;
@@ -1654,6 +1674,12 @@ static psso_status load_other_form(psso_ctx* h, const SaveHeader& hd, const char
     CUDA_TRY(put(I.off_gbrow, J.off_gbrow, row));
     CUDA_TRY(put(I.off_log, J.off_log, J.off_o64 - J.off_log));
     if (I.R == 1) return PSSO_OK;
+    // records and rows of this handle's own earlier run
+    const size_t rb = SLOTS * (size_t)I.R * REC_WORDS * 8;
+    CUDA_TRY(cudaMemsetAsync(h->arena + I.off_rec, 0xff, rb, h->stream));
+    CUDA_TRY(cudaMemsetAsync(h->arena + I.off_rec2, 0xff, rb, h->stream));
+    CUDA_TRY(clear_rows(h, I, h->stream));
+    CUDA_TRY(cudaStreamSynchronize(h->stream));
     GBestDev gb;
     std::memcpy(&gb, src(J.off_gb), sizeof gb);
     return publish_gbest(h, I, hd.gen, gb, src(J.off_gbrow));
@@ -1679,6 +1705,7 @@ psso_status psso_load(psso_handle h, const void* buf, size_t n)
         return fail(PSSO_ERR_ARG, "state was saved from a handle with other problems or launch shape");
     CUDA_TRY(cudaSetDevice(h->device));
     CUDA_TRY(cudaStreamSynchronize(h->stream));
+    h->rows_diverged = true;
     if (other_form) {
         const psso_status st = load_other_form(h, hd, data);
         if (st != PSSO_OK) return st;
