@@ -501,12 +501,18 @@ cudaError_t clear_rows(const psso_ctx* h, const HostInst& I, cudaStream_t s)
 }
 
 // Several blocks: the exchange records and row of generation g rewritten so
-// that the next launch's first step A finds this gBest (rank 0 carries it; the
-// other ranks' records lose against every value).
+// that the next launch's first step A finds this gBest.  The rank that owns its
+// particle carries it, since it must evaluate the row when the bounds leave a
+// doubt (an upper bound beyond the floats always does); rank 0 for a label that
+// is no particle's, which comes with its value.  The other ranks' records lose
+// against every value.
 psso_status publish_gbest(psso_ctx* h, const HostInst& I, int64_t g, const GBestDev& gb, const char* row)
 {
     const uint64_t tag = (uint64_t)(g & 0xffff) << 48;
     const size_t slot = (size_t)(g % SLOTS), R = (size_t)I.R, wpe = h->pos_size / 4;
+    size_t own = 0;
+    for (const auto& u : h->units)
+        if (&h->inst[u.inst] == &I && gb.idx >= u.i0 && gb.idx < u.i1) own = (size_t)u.rank;
     auto u64 = [](double v) {
         uint64_t b;
         std::memcpy(&b, &v, 8);
@@ -520,13 +526,13 @@ psso_status publish_gbest(psso_ctx* h, const HostInst& I, int64_t g, const GBest
     std::vector<uint64_t> rec(R * REC_WORDS), words((size_t)I.Dp * wpe);
     for (size_t r = 0; r < R; ++r) {
         // a losing record: a NaN with FP64 fitness, infinite bounds with FP32
-        const bool has64 = r == 0 ? gb.has64 != 0 : h->variant != V_F32R;
-        const uint64_t v = !has64 ? (r == 0 ? u32(gb.lo) | (u32(gb.hi) << 32) : 0x7f8000007f800000ull)
-                                  : r == 0 ? u64(gb.f64) : 0x7ff8000000000000ull;
-        const uint64_t idx = r == 0 ? (uint64_t)(uint32_t)gb.idx : 0x7ffffffeull;
+        const bool has64 = r == own ? gb.has64 != 0 : h->variant != V_F32R;
+        const uint64_t v = !has64 ? (r == own ? u32(gb.lo) | (u32(gb.hi) << 32) : 0x7f8000007f800000ull)
+                                  : r == own ? u64(gb.f64) : 0x7ff8000000000000ull;
+        const uint64_t idx = r == own ? (uint64_t)(uint32_t)gb.idx : 0x7ffffffeull;
         uint64_t* w = rec.data() + r * REC_WORDS;
         w[RW_IDX] = tag | ((uint64_t)has64 << 32) | idx;
-        w[RW_VER] = tag | (r == 0 ? gb.ver : 0u);
+        w[RW_VER] = tag | (r == own ? gb.ver : 0u);
         w[RW_V0] = tag | (v & 0xffffffffull);
         w[RW_V1] = tag | (v >> 32);
         w[RW_ACC] = w[RW_RCK] = tag;
@@ -538,7 +544,7 @@ psso_status publish_gbest(psso_ctx* h, const HostInst& I, int64_t g, const GBest
     }
     CUDA_TRY(cudaMemcpy(h->arena + I.off_rec + slot * R * REC_WORDS * 8, rec.data(), rec.size() * 8,
                         cudaMemcpyHostToDevice));
-    CUDA_TRY(cudaMemcpy(h->arena + I.off_grow + slot * R * words.size() * 8, words.data(), words.size() * 8,
+    CUDA_TRY(cudaMemcpy(h->arena + I.off_grow + (slot * R + own) * words.size() * 8, words.data(), words.size() * 8,
                         cudaMemcpyHostToDevice));
     return PSSO_OK;
 }

@@ -1,6 +1,8 @@
 """States of small swarms saved in one of their two forms (one block, several
 pipelined blocks) and loaded by a handle that runs the other: the run goes on
 as the oracle's does."""
+import struct
+
 import numpy as np
 import pytest
 
@@ -48,3 +50,32 @@ def lib_spreads(lib, p, precision):
         return lib.psso_stats(h)["blocks"] > 1
     finally:
         lib.psso_destroy(h)
+
+
+def test_interval_of_the_gbest_without_an_upper_bound(lib):
+    """A saved gBest known by an interval that reaches beyond the floats is
+    evaluated by the block that owns its particle."""
+    N, D = 250, 16
+    p = workload.problem("rastrigin", N, D, seed=6, lattice="f32")
+    tried = 0
+    for t1 in range(1, 30):
+        h1 = lib.psso_create_ex([p], "f32", single_block_max=4, log_stride=1, log_capacity=64)
+        h2 = lib.psso_create_ex([p], "f32", log_stride=1, log_capacity=64)
+        try:
+            lib.psso_run(h1, t1)
+            blob = bytearray(lib.psso_save(h1))
+            index = int(lib.psso_get_log(h1, 0)["index"][-1])
+            at = blob.find(struct.pack("<qq", index, t1))          # GBestDev: idx, gen, ..., lo, hi, ver, has64
+            if index < N // 2 or at < 0 or blob[at + 60:at + 64] != bytes(4):
+                continue
+            tried += 1
+            blob[at + 52:at + 56] = struct.pack("<f", float("inf"))
+            lib.psso_load(h2, bytes(blob))
+            lib.psso_run(h2, 6)
+            X, P, _ = lib.psso_get_state(h2, 0, N, D)
+        finally:
+            lib.psso_destroy(h1)
+            lib.psso_destroy(h2)
+        r = oracle.run_problem(p, t1 + 6)
+        assert np.array_equal(X, r["X"]) and np.array_equal(P, r["P"])
+    assert tried
