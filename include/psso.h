@@ -350,7 +350,7 @@ psso_status psso_evaluate(psso_fn fn, int64_t N, int64_t D, const double* X, con
  * row-major), shift and weights (D doubles each, or NULL as in psso_problem),
  * and the outputs f (N doubles) and err (N doubles, or NULL).  It allocates
  * nothing: its only scratch, the padded shift / weight vectors, lives in one
- * static device array of 24 KiB (D at most 1024; larger D is rejected with
+ * static device array of 24 KiB and 16 bytes (D at most 1024; larger D is rejected with
  * PSSO_ERR_ARG; N at most 8 * (2^31 - 1)).  With PSSO_PREC_F32_RECHECK the
  * FP32 terms and the bound err are only valid for float inputs: every row
  * holding an X value that is not a float gets NaN in f and err, and so does

@@ -22,18 +22,22 @@ namespace {
 
 constexpr int NOALLOC_MAX_D = 1024;   // largest D this entry point accepts
 
-// Layout of the scratch array: padded shift and weights in FP64, then in FP32.
+constexpr int FILL_THREADS = 256;     // of a block that fills the scratch array
+
+// Layout of the scratch array: padded shift and weights in FP64, then in FP32,
+// and for each block that filled it whether its shift values are all floats.
 struct NoAllocScratch {
     double o64[NOALLOC_MAX_D];
     double w64[NOALLOC_MAX_D];
     float o32[NOALLOC_MAX_D];
     float w32[NOALLOC_MAX_D];
+    int32_t exact[NOALLOC_MAX_D / FILL_THREADS];
 };
-constexpr size_t SCRATCH_BYTES = sizeof(NoAllocScratch);   // 24 KiB
+constexpr size_t SCRATCH_BYTES = sizeof(NoAllocScratch);   // 24 KiB and 16 bytes
 
 }  // namespace
 
-// The scratch array (24 KiB, held by every GPU that loads the library until
+// The scratch array (24 KiB and 16 bytes, held by every GPU that loads the library until
 // the process exits).  In host code this name is only a stand-in for the
 // device symbol; its device address comes from cudaGetSymbolAddress.
 static __device__ __align__(256) unsigned char g_scratch[SCRATCH_BYTES];
@@ -76,11 +80,15 @@ psso_status scratch_on_current_device(NoAllocScratch** out, int* sms)
 // Fills the padded shift / weight vectors (zeros beyond D); hyper: the
 // weights of the hyper-ellipsoid, w_j = j + 1; griewank: the divisors of its
 // cosines, sqrt(j + 1), once per call instead of once per row.
-__global__ void fill_scratch(NoAllocScratch* s, const double* shift, const double* weights, int D, int Dp,
-                             bool hyper, bool griewank)
+// A thread per variable.
+__global__ void __launch_bounds__(FILL_THREADS) fill_scratch(NoAllocScratch* s, const double* shift,
+                                                             const double* weights, int D, int Dp, bool hyper,
+                                                             bool griewank)
 {
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < Dp; j += gridDim.x * blockDim.x) {
-        const double o = (j < D && shift) ? shift[j] : 0.0;
+    const int j = blockIdx.x * FILL_THREADS + threadIdx.x;
+    double o = 0.0;
+    if (j < Dp) {
+        o = (j < D && shift) ? shift[j] : 0.0;
         const double w = j >= D     ? 0.0
                          : hyper    ? (double)(j + 1)
                          : griewank ? __dsqrt_rn((double)(j + 1))
@@ -91,42 +99,65 @@ __global__ void fill_scratch(NoAllocScratch* s, const double* shift, const doubl
         s->w64[j] = w;
         s->w32[j] = (float)w;
     }
-}
-
-// d as a float when it is exactly one: a normal float's exponent and no bits
-// below its 24, read from the bit pattern (a conversion and a compare through
-// the FP64 unit, which an SM runs at 1.66 lanes per clock, only for the rest:
-// zeros, denormals, infinities, NaN and values that are not floats).
-__device__ __forceinline__ float exact_float(double d, bool& exact)
-{
-    const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
-    const uint32_t mag = hi & 0x7fffffffu;
-    if (mag - (897u << 20) < ((1151u - 897u) << 20) && (lo & 0x1fffffffu) == 0u)
-        return __uint_as_float((hi & 0x80000000u) | __funnelshift_l(lo, mag - (896u << 20), 3));
-    const float f = (float)d;
-    exact = exact && ((double)f == d);
-    return f;
+    // the FP32 terms use the shift rounded to float; the bound holds for the FP64
+    // value only when that rounding is exact
+    const int exact = __syncthreads_and((double)(float)o == o);
+    if (threadIdx.x == 0) s->exact[blockIdx.x] = exact;
 }
 
 // One warp per row of X (N x D doubles, unpadded): the same fitness routines
 // and the same 32-lane chunk layout as psso_evaluate.
+//
+// FP32.  A double that is exactly a normal float is one by its exponent and the
+// absence of bits below its 24, and is converted by a shift: the conversions and
+// the compare hold the FP64 unit (1.66 lanes per clock and SM) for three
+// instructions a value.  A lane that meets anything else (zeros, denormals,
+// infinities, NaN, values that are not floats) converts its values by
+// instruction.  All loads come first, since an SM holds only eight of these warps.
+// Rastrigin, N = 34366, D = 118: 86 us a call with conversions, 51 so; tested and
+// converted value by value, each branch between two loads, up to 15 % slower than
+// with conversions.
 template <bool F32, int MAXC>
-__device__ void eval_row(const Hot& in, const double* xr, double* f, double* err)
+__device__ void eval_row(const Hot& in, const int32_t* shift_exact, const double* xr, double* f, double* err)
 {
     const int lane = threadIdx.x & 31;
-    bool exact = true;
     if constexpr (F32) {
+        bool exact = lane >= (in.Dp + FILL_THREADS - 1) / FILL_THREADS || shift_exact[lane] != 0;
         float x[MAXC][4];
+        bool rare = false;
+        {
+            double d[MAXC][4];
 #pragma unroll
-        for (int q = 0; q < MAXC; ++q)
+            for (int q = 0; q < MAXC; ++q)
 #pragma unroll
-            for (int m = 0; m < 4; ++m) {
-                const int j = 4 * (lane + 32 * q) + m;
-                x[q][m] = j < in.D ? exact_float(xr[j], exact) : 0.f;
-                // the FP32 terms use the shift rounded to float; the bound holds for
-                // the FP64 value only when that rounding is exact
-                if (j < in.D) (void)exact_float(in.o64[j], exact);
-            }
+                for (int m = 0; m < 4; ++m) {
+                    const int j = 4 * (lane + 32 * q) + m;
+                    d[q][m] = j < in.D ? xr[j] : 1.0;
+                }
+#pragma unroll
+            for (int q = 0; q < MAXC; ++q)
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    const uint32_t hi = (uint32_t)__double2hiint(d[q][m]), lo = (uint32_t)__double2loint(d[q][m]);
+                    const uint32_t mag = hi & 0x7fffffffu;
+                    rare = rare || mag - (897u << 20) >= ((1151u - 897u) << 20) || (lo & 0x1fffffffu) != 0u;
+                    x[q][m] = 4 * (lane + 32 * q) + m < in.D
+                                  ? __uint_as_float((hi & 0x80000000u) | __funnelshift_l(lo, mag - (896u << 20), 3))
+                                  : 0.f;
+                }
+        }
+        if (rare) {
+#pragma unroll
+            for (int q = 0; q < MAXC; ++q)
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    const int j = 4 * (lane + 32 * q) + m;
+                    if (j >= in.D) continue;
+                    const double v = xr[j];
+                    x[q][m] = (float)v;
+                    exact = exact && (double)x[q][m] == v;
+                }
+        }
         const Fit32 r = fit32<MAXC>(in, x, lane, 0xffffffffu, 32);
         exact = __all_sync(0xffffffffu, exact);
         if (lane == 0) {
@@ -151,7 +182,8 @@ __device__ void eval_row(const Hot& in, const double* xr, double* f, double* err
 }
 
 template <bool F32>
-__global__ void eval_noalloc(const Hot in, const double* X, int64_t N, double* f, double* err)
+__global__ void eval_noalloc(const Hot in, const int32_t* shift_exact, const double* X, int64_t N, double* f,
+                             double* err)
 {
     const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (row >= N) return;
@@ -159,10 +191,10 @@ __global__ void eval_noalloc(const Hot in, const double* X, int64_t N, double* f
     const double* xr = X + row * in.D;
     double* e = err ? err + row : nullptr;
     switch (in.maxc) {
-    case 1: eval_row<F32, 1>(in, xr, f + row, e); break;
-    case 2: eval_row<F32, 2>(in, xr, f + row, e); break;
-    case 4: eval_row<F32, 4>(in, xr, f + row, e); break;
-    default: eval_row<F32, 8>(in, xr, f + row, e); break;
+    case 1: eval_row<F32, 1>(in, shift_exact, xr, f + row, e); break;
+    case 2: eval_row<F32, 2>(in, shift_exact, xr, f + row, e); break;
+    case 4: eval_row<F32, 4>(in, shift_exact, xr, f + row, e); break;
+    default: eval_row<F32, 8>(in, shift_exact, xr, f + row, e); break;
     }
 }
 
@@ -228,13 +260,13 @@ extern "C" psso_status psso_evaluate_noalloc(psso_fn fn, int64_t N, int64_t D, c
     cudaStream_t cs = static_cast<cudaStream_t>(stream);
     // clear an earlier, unrelated launch error so that only this call's launches are reported
     (void)cudaGetLastError();
-    fill_scratch<<<(Dp + 255) / 256, 256, 0, cs>>>(s, shift, weights, (int)D, Dp, hyper, griewank);
+    fill_scratch<<<(Dp + FILL_THREADS - 1) / FILL_THREADS, FILL_THREADS, 0, cs>>>(s, shift, weights, (int)D, Dp, hyper, griewank);
     const int wpb = 8;
     const unsigned grid = (unsigned)((N + wpb - 1) / wpb);
     cudaError_t e = cudaSuccess;
-    if (precision == PSSO_PREC_F32_RECHECK) eval_noalloc<true><<<grid, 32 * wpb, 0, cs>>>(in, X, N, f, err);
+    if (precision == PSSO_PREC_F32_RECHECK) eval_noalloc<true><<<grid, 32 * wpb, 0, cs>>>(in, s->exact, X, N, f, err);
     else if (ev64::covers(fn)) e = ev64::launch(in, X, D, N, sms, f, err, cs);
-    else eval_noalloc<false><<<grid, 32 * wpb, 0, cs>>>(in, X, N, f, err);
+    else eval_noalloc<false><<<grid, 32 * wpb, 0, cs>>>(in, s->exact, X, N, f, err);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) {
         set_last_error("psso_evaluate_noalloc: kernel launch failed");
