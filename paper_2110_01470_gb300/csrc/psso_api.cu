@@ -757,6 +757,7 @@ psso_status setup_tc(psso_ctx* h, size_t k)
     R.z32_grid = 8 * prop.multiProcessorCount;
     R.fix_grid = prop.multiProcessorCount;
     R.gemm_grid = tc::pair_grid(r.Np, r.Jp, prop.multiProcessorCount);
+    R.gemm_one = tc::PairTiles(r.Np, r.Jp, R.gemm_grid / 2).count <= R.gemm_grid / 2;
     if (!tc::make_tmap_bf16(&R.tmA, r.A, r.Kp, tc::SLICES * r.Np) ||
         !tc::make_tmap_bf16(&R.tmB, R.B, r.Kp, tc::SLICES * r.Jp, tc::SBN))
         return fail(PSSO_ERR_CUDA, "cuTensorMapEncodeTiled failed for the tensor-core operands");

@@ -270,6 +270,7 @@ __device__ __forceinline__ void term32(int fn, float zt, float ez, const float* 
     }
 }
 
+template <bool ONE>
 struct FitEpi {
     const RotDev* r;
     int fn, D;
@@ -278,16 +279,35 @@ struct FitEpi {
     int64_t i;
     int nt;
     float ds, dl1;
-    float t[64], em[64];          // joined accumulators, sums of the partial sums' magnitudes
+    // ONE: no pair has a second item, so the accumulators need not make way and are
+    // read eight columns at a time where they are used
+    float t[ONE ? 8 : 64], em[ONE ? 8 : 64];   // joined accumulators, sums of the partial sums' magnitudes
+    uint32_t at;                  // ONE: the accumulators' address
     __device__ __forceinline__ void tile(int tm, int g, int row)
     {
         i = (int64_t)tm * tc::PBM + row;
         nt = g;
         ds = i < r->N ? r->dscale[i] : 1.f;
         dl1 = i < r->N ? r->dl1[i] : 0.f;
+        // the scales (and weights) of the group's columns: two lines each
+        const int lane = threadIdx.x & 31, j = nt * 64 + 32 * (lane & 1);
+        const float* const at = lane < 2 ? r->mscale : lane < 4 ? r->ml1 : r->inst_w32;
+        if (lane < 6 && at && j < D) asm volatile("prefetch.global.L1 [%0];" ::"l"(at + j));
     }
-    // joins the accumulators from the smallest weight up; each step one
-    // rounding (the scaled accumulator is exact)
+    // joins the accumulators of column q (v: by weight) from the smallest weight up;
+    // each step one rounding (the scaled accumulator is exact)
+    __device__ __forceinline__ void join_low(int q, float v2, float v3)
+    {
+        t[q] = __fmaf_rn(v2, 0x1p-14f, __fmul_rn(v3, 0x1p-21f));   // the product is exact
+        em[q] = fabsf(t[q]);
+    }
+    __device__ __forceinline__ void join_high(int q, float v0, float v1)
+    {
+        const float t1 = __fmaf_rn(v1, 0x1p-7f, t[q]);
+        const float t2 = __fadd_rn(v0, t1);
+        em[q] = __fadd_ru(__fadd_ru(em[q], fabsf(t1)), fabsf(t2));
+        t[q] = t2;
+    }
     template <int C>
     __device__ __forceinline__ void load32(uint32_t taddr)
     {
@@ -295,29 +315,24 @@ struct FitEpi {
         tc::tmem_ld32(taddr + (uint32_t)(3 * 128), v);
         tc::tmem_ld32(taddr + (uint32_t)(2 * 128), w);
 #pragma unroll
-        for (int q = 0; q < 32; ++q) {
-            t[32 * C + q] = __fmaf_rn(w[q], 0x1p-14f, __fmul_rn(v[q], 0x1p-21f));   // the product is exact
-            em[32 * C + q] = fabsf(t[32 * C + q]);
-        }
+        for (int q = 0; q < 32; ++q) join_low(32 * C + q, w[q], v[q]);
         tc::tmem_ld32(taddr + (uint32_t)128, v);
         tc::tmem_ld32(taddr, w);
 #pragma unroll
-        for (int q = 0; q < 32; ++q) {
-            const float t1 = __fmaf_rn(v[q], 0x1p-7f, t[32 * C + q]);
-            const float t2 = __fadd_rn(w[q], t1);
-            em[32 * C + q] = __fadd_ru(__fadd_ru(em[32 * C + q], fabsf(t1)), fabsf(t2));
-            t[32 * C + q] = t2;
-        }
+        for (int q = 0; q < 32; ++q) join_high(32 * C + q, w[q], v[q]);
     }
     __device__ __forceinline__ void load(uint32_t taddr, int n)
     {
-        load32<0>(taddr);
-        if (n == 2) load32<1>(taddr + 32);
+        if constexpr (ONE) {
+            at = taddr;
+        } else {
+            load32<0>(taddr);
+            if (n == 2) load32<1>(taddr + 32);
+        }
     }
-    // The terms of the 32-column blocks c0 .. c0 + n - 1 of the group.  Eight
-    // columns a step, the rest of the registers moved up: unrolled over 64
-    // columns, the code of a tile takes longer to fetch than to run where a CTA
-    // has one tile.
+    // The terms of the 32-column blocks c0 .. c0 + n - 1 of the group, eight columns a
+    // step (without ONE the rest of the registers move up): unrolled over 64 columns,
+    // the code of a tile takes longer to fetch than to run where a CTA has one tile.
     __device__ __forceinline__ void compute(int c0, int n, float4* xch)
     {
         float acc = 0.f, acc2 = 0.f, accE = 0.f, rQ = 0.f;
@@ -325,6 +340,15 @@ struct FitEpi {
 #pragma unroll 1
         for (int h = 0; h < 4 * n; ++h) {
             const int j0 = nt * 64 + 32 * c0 + 8 * h;
+            if constexpr (ONE) {
+                float v[4][8];
+                tc::tmem_ld8x4(at + (uint32_t)(8 * h), 128u, v);
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    join_low(q, v[2][q], v[3][q]);
+                    join_high(q, v[0][q], v[1][q]);
+                }
+            }
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
                 const int j = j0 + q;
@@ -339,10 +363,12 @@ struct FitEpi {
                                           0x1p-38f * em[q] * sc) + 0x1p-126f;
                 term32(fn, zt, ez, r->inst_w32, j, s, s2, e, eq);
             }
+ if constexpr (!ONE) {
 #pragma unroll
-            for (int q = 0; q < 56; ++q) {
-                t[q] = t[q + 8];
-                em[q] = em[q + 8];
+                for (int q = 0; q < 56; ++q) {
+                    t[q] = t[q + 8];
+                    em[q] = em[q + 8];
+                }
             }
             if ((h & 3) == 3) {                 // a block of 32 terms ends
                 acc = __fadd_rn(acc, s);
@@ -378,12 +404,17 @@ struct SliceCfg {
 };
 
 // Persistent, one CTA pair per two SMs (tc_pair.cuh).  N = 8192, D = 1000: 160 ->
-// 138 us per launch.
+// 138 us per launch.  A launch of at most one item a pair is latency: the loads of
+// the row's and the columns' scales start before the wait for the accumulators, and
+// ONE moves no registers (N = 169, D = 33: 17.6 -> 14.6 us between events, 5 of them
+// the events'; N = 4096, D = 256 has 64 items for 76 pairs).  The kernel of one CTA per
+// 128 x 64 tile took 14.1 us there, but 19.2 against 16.8 at N = 256, D = 128.
+template <bool ONE>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(tc::P_THREADS, 1)
     rot_gemm_fit(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                  const __grid_constant__ RotDev r)
 {
-    FitEpi epi;
+    FitEpi<ONE> epi;
     epi.r = &r;
     epi.fn = base_fn(r.fn);
     epi.D = r.D;
@@ -1096,7 +1127,10 @@ cudaError_t enqueue_generation_timed(const RotHost& h, cudaStream_t s, cudaEvent
     const int wpb = 8;
     rot_update<<<std::min(4 * h.fix_grid, (N + UPDATE_WARPS - 1) / UPDATE_WARPS), 32 * UPDATE_WARPS, 0, s>>>(r);
     mark();
-    rot_gemm_fit<<<h.gemm_grid, tc::P_THREADS, tc::pair_smem<SliceCfg::PLANES, SliceCfg::STG>(), s>>>(h.tmA, h.tmB, r);
+    if (h.gemm_one)
+        rot_gemm_fit<true><<<h.gemm_grid, tc::P_THREADS, tc::pair_smem<SliceCfg::PLANES, SliceCfg::STG>(), s>>>(h.tmA, h.tmB, r);
+    else
+        rot_gemm_fit<false><<<h.gemm_grid, tc::P_THREADS, tc::pair_smem<SliceCfg::PLANES, SliceCfg::STG>(), s>>>(h.tmA, h.tmB, r);
     mark();
     rot_decide<<<(N + wpb - 1) / wpb, 32 * wpb, 0, s>>>(r);
     mark();
@@ -1227,8 +1261,10 @@ cudaError_t set_generation(const RotHost& h, long long g, cudaStream_t s)
 
 cudaError_t configure()
 {
-    return cudaFuncSetAttribute(rot_gemm_fit, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                tc::pair_smem<SliceCfg::PLANES, SliceCfg::STG>());
+    constexpr int smem = tc::pair_smem<SliceCfg::PLANES, SliceCfg::STG>();
+    const cudaError_t e = cudaFuncSetAttribute(rot_gemm_fit<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(rot_gemm_fit<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
 }
 
 }  // namespace rot

@@ -184,6 +184,33 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32])
     for (int t = 0; t < 32; ++t) v[t] = __uint_as_float(r[t]);
 }
 
+// Eight consecutive columns of each of four accumulators (`step` columns apart).
+__device__ __forceinline__ void tmem_ld8x4(uint32_t taddr, uint32_t step, float (&v)[4][8])
+{
+    uint32_t r[4][8];
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+            : "=r"(r[a][0]), "=r"(r[a][1]), "=r"(r[a][2]), "=r"(r[a][3]), "=r"(r[a][4]), "=r"(r[a][5]), "=r"(r[a][6]),
+              "=r"(r[a][7])
+            : "r"(taddr + (uint32_t)a * step));
+    // The wait names the registers so that no use of them moves above it.
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0][0]), "+r"(r[0][1]), "+r"(r[0][2]), "+r"(r[0][3]), "+r"(r[0][4]), "+r"(r[0][5]),
+                   "+r"(r[0][6]), "+r"(r[0][7]), "+r"(r[1][0]), "+r"(r[1][1]), "+r"(r[1][2]), "+r"(r[1][3]),
+                   "+r"(r[1][4]), "+r"(r[1][5]), "+r"(r[1][6]), "+r"(r[1][7]), "+r"(r[2][0]), "+r"(r[2][1]),
+                   "+r"(r[2][2]), "+r"(r[2][3]), "+r"(r[2][4]), "+r"(r[2][5]), "+r"(r[2][6]), "+r"(r[2][7]),
+                   "+r"(r[3][0]), "+r"(r[3][1]), "+r"(r[3][2]), "+r"(r[3][3]), "+r"(r[3][4]), "+r"(r[3][5]),
+                   "+r"(r[3][6]), "+r"(r[3][7])
+                 :
+                 : "memory");
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[a][q] = __uint_as_float(r[a][q]);
+}
+
 // Exact three-part BF16 split of a float (see the header comment).
 __device__ __forceinline__ void split3(float v, __nv_bfloat16& h, __nv_bfloat16& m, __nv_bfloat16& l)
 {

@@ -304,6 +304,7 @@ __device__ __forceinline__ bool gemm_pair(const CUtensorMap* tmA, const CUtensor
             int tm, g0, ng;
             tiles.item(k, tm, g0, ng);
             if (ng == 0) continue;
+            epi.tile(tm, ng == 2 ? g0 + half : g0, (int)rank * 128 + 32 * qtr + lane);   // its loads travel now
             // the two warps of a lane quarter go on or leave together: each times its
             // own wait, and pair_exchange waits for the other warp without a limit
             const bool ok = mbar_wait(tfull, (uint32_t)(tl & 1));
@@ -313,7 +314,6 @@ __device__ __forceinline__ bool gemm_pair(const CUtensorMap* tmA, const CUtensor
                 break;
             }
             tc_fence_after();
-            epi.tile(tm, ng == 2 ? g0 + half : g0, (int)rank * 128 + 32 * qtr + lane);
             epi.load(tmem + lane_base + (uint32_t)((ng == 2 ? 64 : 32) * half), ng);
             // the accumulators may be overwritten once all warps of the pair have read them
             tc_fence_before();
