@@ -914,7 +914,7 @@ __global__ void __launch_bounds__(128) rot_fix(const RotDev r, int which)
 // Lowest-index arg-min of the pBest bounds by one block: only the keys are
 // read and reduced (the smallest and second-smallest lower bound, the first's
 // index, the smallest upper bound), four particles per thread and load; the
-// winner's other fields are read afterwards (12.3 -> 10.1 us at N = 8192).
+// winner's other fields are read afterwards, together (12.3 -> 10.1 us at N = 8192).
 struct Key {
     float l1, l2, mh;
     int i;
@@ -974,10 +974,11 @@ __global__ void __launch_bounds__(1024) rot_argmin(const RotDev r, int phase)
     const InstDev& d = *r.inst;
     RotCtl* ctl = r.ctl;
     const int64_t g = ctl->gen;
-    const int N = (int)d.N, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int N = (int)d.N, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     if (phase == 0) {
-        Key k = {FLT_MAX, FLT_MAX, FLT_MAX, INT_MAX};
-        for (int i = 4 * (int)threadIdx.x; i < N; i += 4096) {
+        const Key none = {FLT_MAX, FLT_MAX, FLT_MAX, INT_MAX};
+        Key k = none;
+        for (int i = 4 * (int)threadIdx.x; i < N; i += 4 * (int)blockDim.x) {
             if (i + 4 <= N) {
                 float lo[4], hi[4];
                 ld4(d.plo + i, lo);
@@ -991,15 +992,17 @@ __global__ void __launch_bounds__(1024) rot_argmin(const RotDev r, int phase)
         k = key_warp(k);
         if (lane == 0) shk[warp] = k;
         __syncthreads();
-        k = key_warp(shk[lane]);           // 32 warps: every warp has the block's result
+        k = key_warp(lane < nw ? shk[lane] : none);     // every warp has the block's result
         if (k.i >= N) k.i = 0;             // no finite bound at all
         if (k.l2 > k.mh) {                 // one interval lies below every other: the arg-min
             if (threadIdx.x == 0) {
                 // the gBest value the generation reports must lie within 1e-6 of
                 // FP64: an interval too wide for that gets the winner's FP64 value
                 // (list 2; the exact pass of phase 1 then keeps the same winner)
-                const int has = (int)(d.pflag[k.i] & 1u);
+                const int has = (int)(d.pflag[k.i] & 1u);      // (the four loads travel together)
                 const float hi = d.phi[k.i];
+                const double v = d.pf64[k.i];
+                const uint32_t ver = d.pver[k.i];
                 const bool wide = !has && too_wide(r.fn, k.l1, hi);
                 ctl->amb = wide ? 1 : 0;
                 if (wide) {
@@ -1007,11 +1010,11 @@ __global__ void __launch_bounds__(1024) rot_argmin(const RotDev r, int phase)
                     ctl->n2 = 1;
                 }
                 ctl->win_i = k.i;
-                ctl->win_v = has ? d.pf64[k.i] : DBL_MAX;
+                ctl->win_v = has ? v : DBL_MAX;
                 ctl->win_lo = k.l1;
                 ctl->win_hi = hi;
                 ctl->win_has = has;
-                ctl->win_ver = d.pver[k.i];
+                ctl->win_ver = ver;
             }
             return;
         }
@@ -1037,7 +1040,7 @@ __global__ void __launch_bounds__(1024) rot_argmin(const RotDev r, int phase)
         k = exact_warp(k);
         if (lane == 0) she[warp] = k;
         __syncthreads();
-        k = exact_warp(she[lane]);
+        k = exact_warp(lane < nw ? she[lane] : Exact{LLONG_MAX, INT_MAX});
         if (k.i >= N) k.i = 0;
         if (threadIdx.x == 0) {
             const double v = d.pf64[k.i];
@@ -1142,13 +1145,13 @@ cudaError_t enqueue_generation_timed(const RotHost& h, cudaStream_t s, cudaEvent
     mark();
     rot_fix<<<h.fix_grid, 128, 0, s>>>(r, 1);
     mark();
-    rot_argmin<<<1, 1024, 0, s>>>(r, 0);
+    rot_argmin<<<1, h.argmin_threads, 0, s>>>(r, 0);
     mark();
     rot_z64<<<h.z64_grid, 128, 0, s>>>(r, 2);
     mark();
     rot_fix<<<h.fix_grid, 128, 0, s>>>(r, 2);
     mark();
-    rot_argmin<<<1, 1024, 0, s>>>(r, 1);
+    rot_argmin<<<1, h.argmin_threads, 0, s>>>(r, 1);
     mark();
     return cudaGetLastError();
 }

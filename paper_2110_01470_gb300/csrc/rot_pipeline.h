@@ -62,7 +62,7 @@ struct RotHost {
     const float* M32;
     const double* M64;
     long long N;
-    int z64_grid, z32_grid, fix_grid;
+    int z64_grid, z32_grid, fix_grid, argmin_threads;
     int gemm_grid;                 // CTAs of the persistent GEMM (tc::pair_grid)
     bool gemm_one = false;         // every CTA pair has at most one work item
     void* mem;                     // the one allocation holding the buffers above

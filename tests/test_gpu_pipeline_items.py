@@ -10,7 +10,9 @@ import workload
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("N,D", [(130, 32), (257, 33), (2000, 63), (10000, 65), (9000, 129), (20000, 65)])
+# the first four: the arg-min block's smallest and largest sizes
+@pytest.mark.parametrize("N,D", [(1, 32), (5, 33), (129, 300), (1025, 32),
+                                 (130, 32), (257, 33), (2000, 63), (10000, 65), (9000, 129), (20000, 65)])
 @pytest.mark.parametrize("fn", ["rot_ellipsoid", "rot_rastrigin", "rot_ackley"])
 def test_same_decisions(lib, fn, N, D):
     p = workload.problem(fn, N, D, seed=D, lattice="f32")
