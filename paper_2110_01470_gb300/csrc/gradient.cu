@@ -452,13 +452,15 @@ __global__ void __launch_bounds__(256) prep_planes(const PrepArgs a)
 
 // The terms of f summed over the 64 columns: part[i][g] = (s1, s2) (ellipsoid
 // sum w z^2, Rastrigin sum z^2 + 20 sin^2, Ackley sum z^2 and sum sin^2).
+// Blocks of 32 terms, then the two blocks: with the tree of finish_rows the longest
+// chain is 32 + 1 + 4 additions (D = 1024).
 struct SumEpi : tc::JoinEpi {
     float2* part;
     const float* w;
     int fn, groups;
     __device__ __forceinline__ void compute(int c0, int n, float4* xch)
     {
-        float s1 = 0.f, s2 = 0.f;
+        float s1 = 0.f, s2 = 0.f, a1 = 0.f, a2 = 0.f;
 #pragma unroll 1
         for (int h = 0; h < 4 * n; ++h) {            // eight columns a step (short code)
 #pragma unroll
@@ -467,19 +469,24 @@ struct SumEpi : tc::JoinEpi {
                 if (j >= D) break;
                 const float zj = z[0][q];
                 if (fn == FN_ELLIPSOID) {
-                    s1 = __fmaf_rn(__fmul_rn(__ldg(w + j), zj), zj, s1);
+                    a1 = __fmaf_rn(__fmul_rn(__ldg(w + j), zj), zj, a1);
                 } else {
                     const float sn = sinpi_reduced_f32(__fsub_rn(zj, rint_f32(zj)));
                     if (fn == FN_RASTRIGIN) {
-                        s1 = __fadd_rn(s1, __fmaf_rn(zj, zj, __fmul_rn(__fmul_rn(20.f, sn), sn)));
+                        a1 = __fadd_rn(a1, __fmaf_rn(zj, zj, __fmul_rn(__fmul_rn(20.f, sn), sn)));
                     } else {
-                        s1 = __fmaf_rn(zj, zj, s1);
-                        s2 = __fmaf_rn(sn, sn, s2);
+                        a1 = __fmaf_rn(zj, zj, a1);
+                        a2 = __fmaf_rn(sn, sn, a2);
                     }
                 }
             }
 #pragma unroll
             for (int q = 0; q < 56; ++q) z[q >> 5][q & 31] = z[(q + 8) >> 5][(q + 8) & 31];
+            if ((h & 3) == 3) {                      // a block of 32 terms ends
+                s1 = __fadd_rn(s1, a1);
+                s2 = __fadd_rn(s2, a2);
+                a1 = a2 = 0.f;
+            }
         }
         if (n == 1) {
             const float4 o = tc::pair_exchange(make_float4(s1, s2, 0.f, 0.f), c0, xch);
@@ -507,12 +514,22 @@ __global__ void finish_rows(const float2* part, int groups, int fn, int N, int D
     pdl_entry();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
-    float s1 = 0.f, s2 = 0.f;
-    for (int t = 0; t < groups; ++t) {
-        const float2 p = part[(size_t)i * groups + t];
-        s1 = __fadd_rn(s1, p.x);
-        s2 = __fadd_rn(s2, p.y);
+    float p1[16], p2[16];                    // at most 1024 / 64 groups, added as a tree
+#pragma unroll
+    for (int t = 0; t < 16; ++t) {
+        const float2 p = t < groups ? part[(size_t)i * groups + t] : make_float2(0.f, 0.f);
+        p1[t] = p.x;
+        p2[t] = p.y;
     }
+#pragma unroll
+    for (int w = 8; w > 0; w >>= 1)
+#pragma unroll
+        for (int t = 0; t < 8; ++t)
+            if (t < w) {
+                p1[t] = __fadd_rn(p1[t], p1[t + w]);
+                p2[t] = __fadd_rn(p2[t], p2[t + w]);
+            }
+    const float s1 = p1[0], s2 = p2[0];
     float v = s1;
     if (fn == FN_ACKLEY)
         v = -20.f * expm1f(-0.2f * sqrtf(s1 / (float)D)) - 2.7182818f * expm1f(-2.f * s2 / (float)D);
