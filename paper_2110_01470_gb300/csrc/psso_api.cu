@@ -1333,7 +1333,7 @@ psso_status psso_reset(psso_handle h)
     for (auto& I : h->inst)
         if (I.tc) CUDA_TRY(cudaMemsetAsync(&I.rh.dev.ctl->status, 0, sizeof(int), h->stream));
     if (h->actl) CUDA_TRY(cudaMemsetAsync(h->actl, 0, sizeof(AsyncCtl), h->stream));
-    if (h->rows_diverged)
+    if (h->rows_diverged || h->gen >= 65536)       // (a tag is a generation modulo 2^16)
         for (const auto& I : h->inst)
             if (I.R > 1) CUDA_TRY(clear_rows(h, I, h->stream));
     h->rows_diverged = false;

@@ -68,3 +68,18 @@ def test_load_after_another_run(lib, fn, precision, N, D):
             lib.psso_destroy(h2)
         r = oracle.run_problem(p, 14)
         assert np.array_equal(X, r["X"]) and np.array_equal(P, r["P"]), seed
+
+
+def test_reset_after_the_tags_came_round(lib):
+    """Generation 3 * 2^16 has generation 0's tag and slot."""
+    p = workload.problem("sphere", 100, 30, seed=2, lattice="f64")
+    r = oracle.run_problem(p, 0)
+    h = lib.psso_create_ex([p], "f64")
+    try:
+        lib.psso_run(h, 3 * 65536)
+        for _ in range(3):
+            lib.psso_reset(h)
+            _, i, row = lib.psso_best(h, 0, 30)
+            assert i == r["log_b"][0] and np.array_equal(row, r["P"][i])
+    finally:
+        lib.psso_destroy(h)
