@@ -451,9 +451,10 @@ __global__ void __launch_bounds__(256, RowsBound<Pos, F32R>::min_blocks) bat_row
                 }
                 const Fit32 fr = rs.finish(G, D, nq);
                 const bool same = same_row(r, pi, valid);
-                const float lo0 = __fsub_rd(fr.f, fr.E);
+                // (beyond the floats' range f - E is a NaN: nothing is known of the value)
+                const float lo0 = fmaxf(__fsub_rd(fr.f, fr.E), -INFINITY);
                 if constexpr (F32R) {
-                    const float hi = __fadd_ru(fr.f, fr.E);
+                    const float hi = fminf(__fadd_ru(fr.f, fr.E), INFINITY);
                     // an identical row: identical fitness, its state is kept
                     const bool keep = valid && same;
                     const bool take = valid && !same && (g == 0 || hi < bl);

@@ -473,7 +473,8 @@ __global__ void rot_decide(const RotDev r)
             aq = __fadd_rn(aq, __shfl_sync(0xffffffffu, p.w, t));
         }
         const Fit32 f = rot_final(base_fn(r.fn), r.D, a, a2, ae, aq, 38.f + (float)r.nJt);
-        const float lo = __fsub_rd(f.f, f.E), hi = __fadd_ru(f.f, f.E);
+        // (beyond the floats' range f - E is a NaN: nothing is known of the value)
+        const float lo = fmaxf(__fsub_rd(f.f, f.E), -INFINITY), hi = fminf(__fadd_ru(f.f, f.E), INFINITY);
         int accept = 0, write = 0, undecided = 0;
         if (g == 0) {
             accept = write = 1;

@@ -256,10 +256,15 @@ struct Cand {
     int rank;          // publishing rank of the first (records only)
 };
 
+// No candidate: loses against every particle.  FP64: its value is a NaN, above
+// everything in cand_merge's order and behind any particle's index, also for
+// fitness that overflows.  FP32: the bounds are intervals without a NaN (FP64
+// values of float positions are finite).
+template <bool F32R = true>
 __device__ __forceinline__ Cand cand_none()
 {
     Cand c;
-    c.v = DBL_MAX; c.i = LLONG_MAX; c.mh = FLT_MAX; c.l1 = FLT_MAX; c.h1 = FLT_MAX;
+    c.v = F32R ? DBL_MAX : __longlong_as_double(0x7ff8000000000000LL); c.i = LLONG_MAX; c.mh = FLT_MAX; c.l1 = FLT_MAX; c.h1 = FLT_MAX;
     c.l2 = FLT_MAX; c.ver = 0; c.has1 = 0; c.rank = -1;
     return c;
 }
@@ -319,7 +324,7 @@ template <bool F32R>
 __device__ __forceinline__ Cand cand_of(long long i, double f64, float lo, float hi, int has64,
                                         uint32_t ver)
 {
-    Cand c = cand_none();
+    Cand c = cand_none<F32R>();
     c.i = i;
     c.ver = ver;
     if (!F32R) {
@@ -523,8 +528,9 @@ __device__ __forceinline__ void particle_compute(const Hot& in, const View<Pos>&
         s.hi = 0.f;
     } else {
         const Fit32 r = fit32<MAXC>(in, s.x, lane_g, gmask, in.G);
-        s.lo = __fsub_rd(r.f, r.E);
-        s.hi = __fadd_ru(r.f, r.E);
+        // (beyond the floats' range f - E is a NaN: nothing is known of the value)
+        s.lo = fmaxf(__fsub_rd(r.f, r.E), -INFINITY);
+        s.hi = fminf(__fadd_ru(r.f, r.E), INFINITY);
         s.has64 = 0;
         s.f64v = 0.0;
         s.wstate = true;
@@ -710,7 +716,7 @@ __device__ Cand step_b(const InstDev& desc, const UnitDev& un, const View<Pos>& 
     const Hot in = hot_of(desc);
     const Groups gr = groups_of(in.G);
     const int64_t n = un.i1 - un.i0;
-    Cand best = cand_none();
+    Cand best = cand_none<F32R>();
     for (int64_t k = gr.gid; k < n; k += gr.ngroups) {
         const int64_t i = un.i0 + k;
         const int64_t e = i - v.base;
@@ -821,7 +827,7 @@ __device__ __forceinline__ Winner step_c(const InstDev& in, const UnitDev& un, c
                                          BlockShared& sh, int64_t g)
 {
     const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    const Cand c = lane < nw ? sh.warp_cand[lane] : cand_none();   // unused slots hold none
+    const Cand c = lane < nw ? sh.warp_cand[lane] : cand_none<F32R>();   // unused slots hold none
     trace_point(g, 6);
     int top = 1;
     while (2 * top < nw) top <<= 1;                 // lanes >= nw hold nothing
@@ -869,7 +875,7 @@ template <bool F32R>
 __device__ __forceinline__ bool step_c_spec(const BlockShared& sh, Winner& w)
 {
     const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    const Cand c = lane < nw ? sh.spec_cand[lane] : cand_none();
+    const Cand c = lane < nw ? sh.spec_cand[lane] : cand_none<F32R>();
     int top = 1;
     while (2 * top < nw) top <<= 1;
     unsigned long long acc = lane < nw ? sh.spec_acc[lane] : 0ull;
@@ -1084,7 +1090,7 @@ __device__ __noinline__ void step_a(const KParams& p, const InstDev& in, const U
     const uint64_t* recs = in.rec + (size_t)slot_of(gp) * R * REC_WORDS;
     constexpr int WPE = WordsPer<Pos>::value;
 
-    Cand c = cand_none();
+    Cand c = cand_none<F32R>();
     unsigned long long acc = 0, rck = 0;
     // only the block that writes the gBest record and log sums the counters
     // (and, lagging, not yet)
@@ -1291,12 +1297,12 @@ __device__ Cand spec_b(const KParams& p, const InstDev& desc, const UnitDev& un,
         if ((threadIdx.x >> 5) == 0)
             step_a<Pos, F32R>(p, desc, un, v, slot, gs, g - 1, g - 1 >= p.g_begin, sh);
         __syncthreads();
-        if (sh.flag) return cand_none();
+        if (sh.flag) return cand_none<F32R>();
         trace_point(g, 1);
         need = have && sh.row_changed;     // the gBest moved: recompute with the new row
         if (!need) break;
     }
-    Cand best = cand_none();
+    Cand best = cand_none<F32R>();
     if (have) {
         particle_commit<Pos, F32R, MAXC>(in, v, e, g, gr.lane_g, gr.gmask, st, n_acc, n_rck);
         if (gr.lane_g == 0) best = particle_cand<Pos, F32R, MAXC>(i, st);
@@ -1342,8 +1348,8 @@ __device__ void pipelined_unit(const KParams& p, const InstDev& desc, const Unit
     const int nth = blockDim.x;
     if (warp == 0) {
         if (lane == 0) {      // the control warp's own slots hold no candidate
-            sh.warp_cand[0] = cand_none(); sh.warp_acc[0] = 0; sh.warp_rck[0] = 0;
-            sh.spec_cand[0] = cand_none(); sh.spec_acc[0] = 0; sh.spec_bad[0] = 0;
+            sh.warp_cand[0] = cand_none<F32R>(); sh.warp_acc[0] = 0; sh.warp_rck[0] = 0;
+            sh.spec_cand[0] = cand_none<F32R>(); sh.spec_acc[0] = 0; sh.spec_bad[0] = 0;
         }
         __syncwarp();
         const int nw = nth >> 5;
@@ -1394,7 +1400,7 @@ __device__ void pipelined_unit(const KParams& p, const InstDev& desc, const Unit
         if (have) particle_compute<Pos, F32R, MAXC>(in, v, gs, i, e, g, gr.lane_g, gr.gmask, st);
         {   // speculative candidate: exact unless the row changes or a decision needs FP64
             unsigned long long s_acc = 0, s_rck = 0;
-            Cand sb = cand_none();
+            Cand sb = cand_none<F32R>();
             int bad = 0;
             if (have && gr.lane_g == 0) {
                 if (F32R && st.undecided) bad = 1;
@@ -1419,7 +1425,7 @@ __device__ void pipelined_unit(const KParams& p, const InstDev& desc, const Unit
         if (have && sh.row_changed)       // the gBest moved: recompute with the new row
             particle_compute<Pos, F32R, MAXC>(in, v, gs, i, e, g, gr.lane_g, gr.gmask, st);
         unsigned long long n_acc = 0, n_rck = 0;
-        Cand best = cand_none();
+        Cand best = cand_none<F32R>();
         if (have) {
             particle_commit<Pos, F32R, MAXC>(in, v, e, g, gr.lane_g, gr.gmask, st, n_acc, n_rck);
             if (gr.lane_g == 0) best = particle_cand<Pos, F32R, MAXC>(i, st);
