@@ -123,6 +123,9 @@ __device__ __forceinline__ double expm1_f64(double x)
     constexpr double LN2_LO = 0x1.abc9e3b39803fp-56; // nearest double to ln 2 - LN2_HI
     constexpr double INV_LN2 = 0x1.71547652b82fep+0; // nearest double to 1/ln 2
     if (fabs(x) <= 0x1.62e42fefa39efp-2) return expm1_series_f64(x);  // LN2_HI / 2
+    // finite x <= -40: e^x is below half an ulp of 1, the result -1 (and 2^k below
+    // leaves the normal range at -708); from the sign, exponent and leading bits
+    if ((uint32_t)__double2hiint(x) - 0xc0440000u < 0xfff00000u - 0xc0440000u) return -1.0;
     const double k = rint(__dmul_rn(x, INV_LN2));
     double r = __fma_rn(-k, LN2_HI, x);
     r = __fma_rn(-k, LN2_LO, r);

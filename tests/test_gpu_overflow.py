@@ -50,3 +50,31 @@ def test_rotated_fp32_beyond_the_floats(lib, fn):
     ps = [workload.problem(fn, 150, 40, seed=3, lattice="f32", bounds=(-b, b), shift_range=(0.0, 0.0))]
     check(lib, ps, "f32", tensor_rotation=1)
     check(lib, ps, "f32", tensor_rotation=-1)
+
+
+@pytest.mark.parametrize("precision", ["f64", "f32"])
+@pytest.mark.parametrize("fn", ["ackley", "rot_ackley"])
+def test_ackley_far_from_its_optimum(lib, fn, precision):
+    """Ackley where its exponential has left the normal doubles (rows beyond
+    about 3500 in magnitude), and on both sides of the exponents at which it
+    becomes 0 against 1."""
+    rng = np.random.default_rng(4)
+    D = 20
+    X = np.concatenate([s * rng.uniform(-1.0, 1.0, (30, D))
+                        for s in (100.0, 250.0, 330.0, 400.0, 1e3, 4e3, 1e4, 1e6, 1e10, 1e18)])
+    X = X.astype(np.float32).astype(np.float64)
+    M = workload.rotation(D, 3) if fn == "rot_ackley" else None
+    o = np.zeros(D)
+    f, err = lib.psso_evaluate(fn, X, o, None, M, precision=precision)
+    want = np.array([oracle.fitness(fn, x, o, None, M) for x in X])
+    if precision == "f64":
+        assert np.array_equal(f, want)
+    else:
+        assert np.all(np.abs(f - want) <= err)
+
+
+def test_fp32_ackley_beyond_the_floats(lib):
+    b = float(np.float32(1e30))
+    for N, D, cfg in [(3, 3, {}), (250, 16, {}), (400, 100, {}), (40, 20, dict(batch_stream=1))]:
+        check(lib, [workload.problem("ackley", N, D, seed=2, lattice="f32", bounds=(-b, b), shift_range=(0.0, 0.0))],
+              "f32", **cfg)
