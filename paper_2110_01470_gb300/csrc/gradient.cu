@@ -618,7 +618,7 @@ inline void launch_gz(int maxc, const float* Z, const float* w, const float* gf,
 // Workspace layout of the tensor-core path (byte offsets, 256-aligned).
 struct WsLayout {
     int Np, Jp, Kp;
-    size_t a, b, bt, mn, z, zero, status, total;
+    size_t a, b, bt, z, status, total;
 };
 inline size_t al256(size_t v) { return (v + 255) & ~(size_t)255; }
 inline WsLayout ws_layout(int64_t N, int64_t D)
@@ -632,9 +632,7 @@ inline WsLayout ws_layout(int64_t N, int64_t D)
     w.a = take((size_t)3 * w.Np * w.Kp * 2);
     w.b = take((size_t)3 * w.Jp * w.Kp * 2);
     w.bt = take((size_t)3 * w.Jp * w.Kp * 2);
-    w.mn = take((size_t)w.Jp * 4);
     w.z = take((size_t)N * D * 4);     // Z; a forward pass: the row sums (8 bytes per 64 columns)
-    w.zero = take((size_t)(D + 4) * 4);
     w.status = take(4);
     w.total = off;
     return w;

@@ -231,8 +231,8 @@ psso_status check_problem(const psso_problem& pr, int precision, int idx)
 //   FP32  a converged swarm leaves several candidates in most generations; their
 //         FP64 values then cost the spread form a second exchange, one block a
 //         few microseconds.  Such generations come late in wide rows: D >= 64: 1.11
-//         (N = 6) .. 4.  The fourth pass pays for them: 29 to 32 warps: 0.99 (N = 128,
-//         D = 32) .. 2.7.  Below: 0.70 (N = 12, D = 45), 0.72 (N = 64, D = 20), 0.77 (N = 64,
+//         (N = 6) .. 4.  The fourth pass pays for them: 29 to 32 warps: 0.94 (Rastrigin, N = 128,
+//         D = 32; the others 1.07 and more) .. 2.7.  Below: 0.70 (N = 12, D = 45), 0.72 (N = 64, D = 20), 0.77 (N = 64,
 //         D = 16), 0.89 (N = 100, D = 30), and from N = 128 on (D <= 16) 1.04 .. 2.0 in the
 //         default order against 0.49 .. 1.4 in the paper's order, which converges sooner.
 bool spread_small(int variant, int64_t N, int64_t D, int64_t groups, bool paper_order)

@@ -7,9 +7,9 @@
 // Generation g (the number g is read from device memory, so the sequence can
 // be replayed by a CUDA graph):
 //   1. rot_update    Eq. 2.1 for every variable (the same draws as the
-//                    persistent kernel), X written in place, d = fl32(x - o)
-//                    split into the three BF16 planes, ||d|| bound per row,
-//                    "x equals pBest" flag per row.
+//                    persistent kernel), X written in place, d = x - o (exactly, a
+//                    float pair) as four BF16 planes of integer slices, the slice
+//                    scale and sum |d_k| per row, "x equals pBest" flag per row.
 //   2. rot_gemm_fit  the tcgen05 GEMM; its epilogue turns each z into the
 //                    function's FP32 terms and per-term error bounds and
 //                    writes per-(particle, 64-column group) partial sums.

@@ -32,11 +32,11 @@ struct RotDev {
     int fn, D;
     long long N;
     int Np, Jp, Kp, nJt;           // padded extents, tc::SBN-column tiles
-    __nv_bfloat16* A;              // [4][Np][Kp] integer slices of d = fl32(x - o) (tc_gemm.cuh)
+    __nv_bfloat16* A;              // [4][Np][Kp] integer slices of d = x - o, exactly (tc_gemm.cuh)
     float* dscale;                 // [Np] slice scale s_d of particle i (a power of two)
     float* dl1;                    // [Np] sum_k |d_ik|, rounded up
     float* mscale;                 // [Jp] slice scale s_M of output j
-    float* ml1;                    // [Jp] sum_k |M32_jk|, rounded up
+    float* ml1;                    // [Jp] sum_k |M_jk|, rounded up
     uint32_t* same;                // [N] x_i equals pBest_i bit for bit
     float4* part;                  // [N][nJt] tile sums (s1, s2, e1, e2)
     int32_t* list1;                // [N] pBest updates undecided by the GEMM bounds
@@ -55,7 +55,7 @@ struct RotDev {
 struct RotHost {
     RotDev dev;
     CUtensorMap tmA, tmB;
-    __nv_bfloat16* B;              // [4][Jp][Kp] integer slices of M32
+    __nv_bfloat16* B;              // [4][Jp][Kp] integer slices of the FP64 M
     float* Mh;                     // float pair of M (refinement)
     float* Ml;
     double* Mt;                    // M^T

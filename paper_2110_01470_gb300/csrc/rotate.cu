@@ -1,6 +1,5 @@
-// rotate.cu -- operand preparation for the tensor-core rotation (split BF16
-// planes, row norms, tensor maps) and psso_rotate: z = M (x - o) for N rows
-// on the tensor cores.
+// rotate.cu -- the tensor maps of the operand planes, and psso_rotate: z = M (x - o)
+// for N rows on the tensor cores (split BF16 planes).
 #include <cmath>
 #include <cstdio>
 #include <cudaTypedefs.h>
@@ -37,13 +36,11 @@ bool make_tmap_bf16(CUtensorMap* map, const void* base, int Kp, int rows, int bo
                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// B planes and row-norm bounds of the FP32 rotation: one block per row j of
-// the padded [Jp][Kp] planes (rows >= D and columns >= D are zero).
-__global__ void split_matrix(const float* __restrict__ M32, int D, int Jp, int Kp, __nv_bfloat16* B,
-                             float* mnorm)
+// B planes of the FP32 rotation: one block per row j of the padded [Jp][Kp]
+// planes (rows >= D and columns >= D are zero).
+__global__ void split_matrix(const float* __restrict__ M32, int D, int Jp, int Kp, __nv_bfloat16* B)
 {
     const int j = blockIdx.x;
-    double s = 0.0;
     for (int k = threadIdx.x; k < Kp; k += blockDim.x) {
         const float v = (j < D && k < D) ? M32[(size_t)j * D + k] : 0.f;
         __nv_bfloat16 h, m, l;
@@ -52,17 +49,6 @@ __global__ void split_matrix(const float* __restrict__ M32, int D, int Jp, int K
         B[o] = h;
         B[plane + o] = m;
         B[2 * plane + o] = l;
-        s = fma((double)v, (double)v, s);
-    }
-    __shared__ double red[32];
-    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-        // FP64 sum of at most 2^20 squares: relative error far below 1e-9.
-        mnorm[j] = f64_to_f32_ru(sqrt(t) * (1.0 + 1e-9));
     }
 }
 
@@ -110,16 +96,14 @@ extern "C" psso_status psso_rotate(int64_t N, int64_t D, const float* X, const f
     const int Np = (int)((N + BM - 1) / BM * BM), Jp = (int)((D + BN - 1) / BN * BN),
               Kp = (int)((D + BK - 1) / BK * BK);
     __nv_bfloat16 *A = nullptr, *B = nullptr;
-    float* mn = nullptr;
     int* status = nullptr;
     auto cleanup = [&] {
         cudaFree(A);
         cudaFree(B);
-        cudaFree(mn);
         cudaFree(status);
     };
     if (cudaMalloc(&A, (size_t)3 * Np * Kp * 2) != cudaSuccess || cudaMalloc(&B, (size_t)3 * Jp * Kp * 2) != cudaSuccess ||
-        cudaMalloc(&mn, (size_t)Jp * 4) != cudaSuccess || cudaMalloc(&status, 4) != cudaSuccess) {
+        cudaMalloc(&status, 4) != cudaSuccess) {
         cleanup();
         set_last_error("psso_rotate: device allocation failed");
         return PSSO_ERR_OOM;
@@ -131,7 +115,7 @@ extern "C" psso_status psso_rotate(int64_t N, int64_t D, const float* X, const f
         return PSSO_ERR_CUDA;
     }
     cudaMemsetAsync(status, 0, 4, s);
-    split_matrix<<<Jp, 256, 0, s>>>(rotation, (int)D, Jp, Kp, B, mn);
+    split_matrix<<<Jp, 256, 0, s>>>(rotation, (int)D, Jp, Kp, B);
     split_rows<<<(Np + 7) / 8, 256, 0, s>>>(X, shift, (int)N, (int)D, Np, Kp, A);
     constexpr int smem = pair_smem<SplitCfg::PLANES, SplitCfg::STG>();
     int dev = 0, sms = 0;

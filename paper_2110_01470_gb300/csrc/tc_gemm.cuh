@@ -1,12 +1,13 @@
-// tc_gemm.cuh -- z = M (x - o) for a tile of 128 particles x 128 outputs on
-// the sm_103a tensor cores (tcgen05.mma, operands staged by TMA, FP32
-// accumulators in tensor memory).
+// tc_gemm.cuh -- what the tensor-core GEMMs over operand planes (tc_pair.cuh)
+// share: mbarrier and tensor-memory access, descriptors, and the two ways of
+// writing FP32 and FP64 operands as BF16 planes -- the exact split into three parts
+// (this comment) and the exact integer slices (below).
 //
-// Precision scheme (split BF16): d = fl32(x - o) and the FP32 copy of M are
-// each written exactly as three BF16 parts, v = v_h + v_m + v_l (RN splits:
-// |v_m| <= 2^-8 |v| (1.01), |v_l| <= 2^-16 |v| (1.01); the third remainder is
-// exactly representable, so the split loses nothing).  Of the nine products
-// of the parts, the six above 2^-24 are formed:
+// Split BF16 (z = M (x - o) of psso_rotate and the differentiable fitness): d =
+// fl32(x - o) and the FP32 copy of M are each written exactly as three BF16 parts,
+// v = v_h + v_m + v_l (RN splits: |v_m| <= 2^-8 |v| (1.01), |v_l| <= 2^-16 |v|
+// (1.01); the third remainder is exactly representable, so the split loses
+// nothing).  Of the nine products of the parts, the six above 2^-24 are formed:
 //     acc0[kb % 3] += d_h M_h               (main part; three accumulators, K
 //                                            blocks dealt round robin, so each
 //                                            chain is a third as long)
@@ -15,13 +16,11 @@
 // products are exact in FP32.
 //
 // Operand layout in global memory (bf16, row-major, K contiguous):
-//     A: [3][Np][Kp]   part p of d for particle i at (p, i, k)
-//     B: [3][Jp][Kp]   part p of M_jk at (p, j, k)
-// Np, Jp multiples of 128, Kp a multiple of 64; padding is zero.  Each
-// pipeline stage holds one 64-wide K block of all six planes (6 x 16 KiB,
-// TMA boxes of 64 x 128 with the 128-byte swizzle).  One thread issues the
-// copies, one thread the MMAs; all four warps run the epilogue, warp w owning
-// tensor-memory lanes 32w..32w+31 (one particle each).
+//     A: [planes][Np][Kp]   plane p of d for particle i at (p, i, k)
+//     B: [planes][Jp][Kp]   plane p of M_jk at (p, j, k)
+// Np a multiple of 128, Jp of 64 (slices) or 128, Kp of 64.  Columns k >= D are zero.
+// Rows beyond N and D may hold anything: an output depends on its own row of A and
+// of B only, and theirs are not stored.
 #pragma once
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -31,12 +30,7 @@
 namespace psso {
 namespace tc {
 
-constexpr int BM = 128, BN = 128, BK = 64, STAGES = 2;
-constexpr int TILE_BYTES = BM * BK * 2;                    // 16 KiB (BM == BN)
-constexpr int STAGE_BYTES = 6 * TILE_BYTES;                // 96 KiB
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024;    // + alignment slack
-constexpr int NCHAIN = 3;                                  // main-part accumulators (K split)
-constexpr int TMEM_COLS = 512;                             // acc0[0..2] | acc1
+constexpr int BM = 128, BN = 128, BK = 64;                 // what Np, Jp and Kp are padded to
 constexpr long long WAIT_CYCLES = 4000000000LL;            // ~2 s at 2 GHz
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p)
@@ -81,33 +75,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
     }
 }
 
-// ---- TMA ----------------------------------------------------------------------
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y,
-                                            uint32_t bar)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
-        : "memory");
-}
-
 // ---- tcgen05 ------------------------------------------------------------------
-__device__ __forceinline__ void tmem_alloc(uint32_t slot, uint32_t ncols)
-{
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(slot),
-                 "r"(ncols)
-                 : "memory");
-}
-__device__ __forceinline__ void tmem_relinquish()
-{
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols)
-{
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols)
-                 : "memory");
-}
 __device__ __forceinline__ void tc_fence_before()
 {
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -116,26 +84,6 @@ __device__ __forceinline__ void tc_fence_after()
 {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
-// D[tmem] (+)= A[smem] * B[smem]^T, BF16 inputs, FP32 accumulation.
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
-                                         uint32_t idesc, uint32_t accumulate)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-// Arrives once on the mbarrier when every MMA issued so far by this thread
-// has completed.
-__device__ __forceinline__ void mma_commit(uint32_t bar)
-{
-    asm volatile(
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-        : "memory");
-}
-
 // Instruction descriptor, kind::f16: FP32 accumulator (bits 4-5 = 1), A and
 // B BF16 (bits 7-9, 10-12 = 1), both K-major (bits 15, 16 = 0), N >> 3 in
 // bits 17-22, M >> 4 in bits 24-28.
@@ -229,25 +177,12 @@ __device__ __forceinline__ void split3(float v, __nv_bfloat16& h, __nv_bfloat16&
 // the largest vanish (an accumulator of 1 absorbs any number of products of
 // magnitude 0.99 * 2^-25 unchanged).  One MMA then errs by less than
 // 16 * 2^-25 * max|addend| + 2^-23 |sum| <= 0.625 * 2^-20 (|accumulator| +
-// sum |products|); MMA_EPS takes 2^-20, a margin of 1.6 over that.
+// sum |products|); MMA_EPS takes 2^-20, a margin of 1.6 over that (the figure that
+// psso.h states for the differentiable fitness and psso_rotate).
 constexpr float MMA_EPS = 0x1p-20f;
 
-// z error per unit of S = sum_k |M32_jk| |d_k| (S <= ||d|| ||M32_j||) for a
-// K extent of Kp: the acc0 chains (at most 4 ceil(Kp / 192) MMAs each, over
-// products summing to <= 1.03 S in all), the acc1 chain (5 Kp / 16 MMAs
-// over products <= 2^-7 1.03 S), the three dropped products (<= 1.03 2^-23
-// S), d and M rounded to float (2 x 1.01 2^-24 S), the three additions that
-// join the accumulators (3.1 2^-24 S).
-__host__ __device__ inline float z_err_per_s(int Kp)
-{
-    const int nkb = Kp / 64;
-    const float n0 = 4.f * (float)((nkb + NCHAIN - 1) / NCHAIN), n1 = 5.f * (float)(Kp / 16);
-    return 1.05f * (MMA_EPS * 1.04f * (n0 + n1 * 0x1p-7f) + 1.03f * 0x1p-23f + 2.02f * 0x1p-24f +
-                    3.1f * 0x1p-24f);
-}
-
 struct GemmArgs {
-    int Np, Jp, Kp;   // padded extents (multiples of 128, 128, 64)
+    int Np, Jp, Kp;   // padded extents (multiples of 128, of 64 or 128, of 64)
     int* status;      // set to 1 when a wait ran out (device memory)
 };
 
