@@ -528,9 +528,8 @@ __device__ __forceinline__ void particle_compute(const Hot& in, const View<Pos>&
         s.hi = 0.f;
     } else {
         const Fit32 r = fit32<MAXC>(in, s.x, lane_g, gmask, in.G);
-        // (beyond the floats' range f - E is a NaN: nothing is known of the value)
-        s.lo = fmaxf(__fsub_rd(r.f, r.E), -INFINITY);
-        s.hi = fminf(__fadd_ru(r.f, r.E), INFINITY);
+        s.lo = __fsub_rd(r.f, r.E);
+        s.hi = __fadd_ru(r.f, r.E);
         s.has64 = 0;
         s.f64v = 0.0;
         s.wstate = true;
@@ -540,8 +539,10 @@ __device__ __forceinline__ void particle_compute(const Hot& in, const View<Pos>&
         // relative of the FP64 oracle's.
         const bool tighten = is_rotated(in.fn) && too_wide(in.fn, s.lo, s.hi);
         if (g == 0) {
-            s.accept = !tighten;
-            s.undecided = tighten;
+            // beyond the floats' range f - E is a NaN: the value is made exact at commit
+            // (in later generations a NaN decides nothing and the particle goes to FP64)
+            s.undecided = tighten || !(s.lo <= FLT_MAX);
+            s.accept = !s.undecided;
         } else {
             const float plo = v.plo[e], phi = v.phi[e];
             const uint32_t pfl = v.pflag[e];
