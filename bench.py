@@ -292,8 +292,10 @@ def job_rate(units_per_step, steps, world, max_total_ms):
 # digest of the kernel's sources at capture time and is reported only while
 # the sources still match (a changed kernel reports traffic null).
 TRAFFIC = {
-    ("rot_gemm_fit", "rotated_d1000"): ("0922b0332ae7952f", 75.903232e6 + 2.123904e6),
-    ("sso_generations", "rastrigin_d100"): ("c5a611e6e84c4e41", 1.407488e6 + 0.055552e6),
+    ("rot_gemm_fit", "rotated_d1000"): ("18eace040bf495d8", 75.686e6 + 3.447e6),
+    ("sso_generations", "rastrigin_d100"): ("f77557e853dd7dd6", 1.939e6 + 0.052e6),
+    # a generation's four launches for rows over 128 variables
+    ("bat_rows", "batched_512"): ("1dc547ac10255d63", 659.993e6 + 409.877e6),
 }
 _COMMON = ["sso_common.cuh", "devmath.cuh", "psso_internal.h", "checked.cuh"]
 KERNEL_SOURCES = {

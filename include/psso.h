@@ -324,7 +324,9 @@ int64_t psso_generation(psso_handle h);
 psso_status psso_save(psso_handle h, void* buf, size_t cap, size_t* n);
 
 /* Restores a state written by psso_save for a handle created with the same
- * problems and configuration. */
+ * problems and configuration.  (A small single swarm with the default block
+ * size: also a state of the other of its two forms, one block or pipelined
+ * blocks.) */
 psso_status psso_load(psso_handle h, const void* buf, size_t n);
 
 /* Batched fitness (Kernel Function (E), Sec. 2.3.2): f_i = f(X_i) for N rows of

@@ -11,7 +11,9 @@
 // generations, and CUDA-event timing of the requested generations on a
 // private stream.  The search is a coordinate descent: particles per block
 // first (persistent kernel), then blocks per SM (batched step kernels) with
-// that choice fixed.  Results are cached per process.
+// that choice fixed.  A small swarm's two forms are both among the candidates:
+// with a block size given it runs in one block if it fits, without one as the
+// planner's rule says.  Results are cached per process.
 #include <cuda_runtime.h>
 
 #include <cstring>
